@@ -60,12 +60,12 @@ typedef struct {
 } poro_material;
 
 typedef enum {
-    PORO_FP64 = 0,          /* every step in IEEE binary64 */
-    PORO_FP32_REFINE = 1,   /* binary32 back-substitution + refinement against an
-                               FP64-accurate residual of the predictor system */
-    PORO_BF16X3_REFINE = 2  /* as PORO_FP32_REFINE with the tensor-core split products
-                               in bf16 (hi + lo, ~16 significant bits per product);
-                               one refinement sweep by default, as for FP32_REFINE */
+    PORO_FP64 = 0,          /* IEEE binary64; the Khat products as exact integer sums of
+                               62-bit fixed-point rows, rounded once */
+    PORO_FP32_REFINE = 1,   /* double-binary32 (~48 bits) with integer Khat products: within
+                               1e-10 of binary64 at the default refinement (about 1e-14) */
+    PORO_BF16X3_REFINE = 2  /* the same; the two differ in the unrefined form only (tf32 or
+                               bf16 split products, poro_set_refinement) */
 } poro_precision;
 
 typedef enum {
@@ -105,9 +105,9 @@ typedef enum {
  * reference matrices (Khat^alpha = M^{-1} K^alpha, Section "Block-wise
  * back-substitution"; Z = S^{-1}(W - K^tau)).  *out receives the handle, or
  * NULL on error.  Errors: PORO_EINVAL (out NULL), PORO_EUNSUPPORTED,
- * PORO_ECUDA, PORO_ENOMEM, and PORO_ENUMERIC for a mixed-precision context
- * whose Khat rows are not integer rows over a common denominator with a sum
- * of |numerators| below 2^22 (the exact integer residual needs that). */
+ * PORO_ECUDA, PORO_ENOMEM, and PORO_ENUMERIC if the Khat rows were not integer
+ * rows over a common denominator with a sum of |numerators| below 2^23 (the
+ * exact integer sums need that). */
 poro_status poro_create(int device, int degree_N, poro_precision precision, poro_ctx** out);
 
 /* poro_create for a given system.  PORO_SYSTEM_MAXWELL and
@@ -134,22 +134,20 @@ poro_status poro_destroy(poro_ctx* ctx);
  * context (e.g. a failed poro_create), thread-local. */
 const char* poro_last_error(const poro_ctx* ctx);
 
-/* Number of refinement sweeps of a mixed-precision context (0, 1 or 2;
- * default 1).  The binary32 solution is first rounded onto a fixed-point grid
- * per quantity (integers of at most 22 bits times a power of two set by the
- * quantity's largest entry).  Each sweep then forms the residual of the
- * predictor system for that solution, binary64-accurate:
- *   - the Khat and time-matrix products as exact integer sums;
- *   - the star, E* and coupling products in double-binary32 arithmetic
- *     (error-free products and sums, ~2^-48 relative).
- * It solves for the correction with the low-precision back-substitution.
- * The result is the rounded solution plus the corrections, in binary64.
+/* Accuracy of a mixed-precision context, by the number of refinement sweeps
+ * that would reach it (0, 1 or 2; default 1):
+ *   0  one binary32 back-substitution with its Khat products on the tensor
+ *      cores as three split products (tf32, or bf16 for PORO_BF16X3_REFINE);
+ *   1  Algorithm 3 in double-binary32 with the Khat products as integer sums,
+ *      about 1e-14 relative;
+ *   2  the binary64 predictor.
+ * With 1 and 2 a non-finite value makes its element's whole predictor NaN.
  * Errors: PORO_EUNSUPPORTED for a PORO_FP64 context, PORO_EINVAL. */
 poro_status poro_set_refinement(poro_ctx* ctx, int32_t sweeps);
 
 /* Limit of the bounded waits of a mixed-precision context's predictor (the
- * tensor-core and bulk-copy completions of its low-precision sweeps), in SM
- * clock cycles; 0 restores the default (2e9 cycles, about 1 s).  The paper has
+ * bulk copy of an element's constants; unrefined, the tensor-core and bulk-copy
+ * completions of the sweep), in SM clock cycles; 0 restores the default (2e9 cycles, about 1 s).  The paper has
  * no counterpart: every wait in the library's kernels gives up after its
  * limit instead of spinning forever.  When a wait gives up, the CTA stops,
  * waits with the default limit for its own copies and MMAs still in flight,
@@ -456,8 +454,8 @@ poro_status poro_lu_release(poro_ctx* ctx);
 poro_status poro_lu_predict_static(poro_ctx* ctx, int64_t first, int64_t count, const double* Q0_dev,
                                    double* Qt_dev, double* I_dev, void* stream);
 
-/* Autotuner of the predictor kernels: times the CTA-size variants (0: 256
- * threads at N >= 5, 128 at N = 4, 64 at N <= 3; 1: the alternative) on the
+/* Autotuner of the predictor kernels: times the CTA-size variants (0: 512
+ * threads at N = 6, 256 at N = 5, 128 at N = 4, 64 at N <= 3; 1: the alternative) on the
  * first `sample` elements of the loaded population (<= 0: all), three timed
  * runs after two warm-ups each, and keeps the fastest for this context.
  * *variant_out (nullable) receives the choice, ms_out[2] (nullable) the
@@ -470,16 +468,12 @@ poro_status poro_autotune(poro_ctx* ctx, int64_t sample, int32_t* variant_out, d
 poro_status poro_set_variant(poro_ctx* ctx, int32_t variant);
 
 /* Tile choices of the predictor kernels: choice = 6 * cta + layout, with cta
- * the CTA-size variant (as poro_set_variant) and layout capping the operand
- * buffers of the mixed kernel's tensor-core sweeps per degree block
- * (A-tile buffers, Khat image slots): 0 (3, 3) = as many as fit (default),
- * 1 (2, 3), 2 (1, 3), 3 (2, 2), 4 (1, 2), 5 (1, 1).  Fewer buffers serialise
- * the star products, image copies and MMAs of the three directions; more
- * buffers take shared memory the block may not have, so the kernel still
- * uses only what fits.  Every choice gives bitwise the same predictor.
- * Available: FP64 contexts layouts 0 only (choices 0 and 6), the bf16 form
- * cta 0 only (choices 0..5), the tf32 form all 12; layouts 1..5 with one
- * refinement sweep (the default) only. */
+ * the CTA-size variant (as poro_set_variant).  The layouts 0..5 named operand
+ * buffers of kernels that had a choice of them; the present kernels run alike
+ * with each, and the numbers stay valid.  Every choice gives bitwise the same
+ * predictor.  Available: FP64 contexts layouts 0 only (choices 0 and 6), the
+ * bf16 form cta 0 only (choices 0..5), the tf32 form all 12; layouts 1..5 with
+ * one refinement sweep (the default) only. */
 #define PORO_TILE_CHOICES 12
 
 /* Autotuner over the available tile choices: times each on the first

@@ -183,10 +183,6 @@ void free_reference(poro_ctx* c) {
     dfree(c->lref.kcol);
     dfree(c->lref.kval);
 
-    dfree(c->mref.res_inv);
-    dfree(c->mref.res_order8);
-    dfree(c->mref.res_order4);
-    dfree(c->mref.res_order2);
     dfree(c->mref.khat_tc);
     dfree(c->mref.status);
     dfree(c->mref.zinv_f32);
@@ -198,6 +194,8 @@ void free_reference(poro_ctx* c) {
     dfree(c->dref.khat_row);
     for (int w = 0; w < 3; ++w) dfree(c->dref.lists[w]);
     dfree(c->dref.zinv);
+    dfree(c->dref.inv_d);
+    dfree(c->dref.inv_d2);
 }
 
 }  // namespace
@@ -244,34 +242,6 @@ static std::vector<int32_t> deal_rows(const std::vector<int64_t>& cost, int warp
     for (int k = 0; k < warps; ++k) out[k + 1] = out[k] + (int32_t)lists[k].size();
     for (int k = 0; k < warps; ++k) out.insert(out.end(), lists[k].begin(), lists[k].end());
     return out;
-}
-
-// x = num / den with den <= 10^6 (continued-fraction convergents), if x is
-// such a rational to 1e-14 relative
-static bool rational_of(double x, int64_t& num, int64_t& den) {
-    const double ax = std::fabs(x);
-    int64_t h0 = 0, h1 = 1, k0 = 1, k1 = 0;
-    double r = ax;
-    for (int it = 0; it < 64; ++it) {
-        const double a = std::floor(r);
-        if (a > 9.0e15) break;
-        const int64_t ai = (int64_t)a;
-        const int64_t h2 = ai * h1 + h0, k2 = ai * k1 + k0;
-        if (k2 > 1000000) break;
-        h0 = h1;
-        h1 = h2;
-        k0 = k1;
-        k1 = k2;
-        if (std::fabs((double)h1 / (double)k1 - ax) <= 1e-14 * ax) {
-            num = x < 0 ? -h1 : h1;
-            den = k1;
-            return true;
-        }
-        const double f = r - a;
-        if (f <= 0.0) break;
-        r = 1.0 / f;
-    }
-    return false;
 }
 
 poro_status poro_create(int device, int degree_N, poro_precision precision, poro_ctx** out) {
@@ -358,6 +328,30 @@ poro_status poro_create_system(int device, int degree_N, poro_precision precisio
         return e == cudaErrorMemoryAllocation ? fail(nullptr, PORO_ENOMEM, "poro_create: out of device memory")
                                               : cuda_fail(nullptr, e, "poro_create: upload");
     }
+    if (system == PORO_SYSTEM_BIOT) {
+        // integer Khat rows of Biot's predictor
+        std::vector<int32_t> ent, list;
+        std::vector<double> inv;
+        if (!poro::direct_tables(c->ref, ent, list, inv, err)) {
+            free_reference(c);
+            cudaStreamDestroy(c->stream);
+            delete c;
+            return fail(nullptr, PORO_ENUMERIC, "poro_create: " + err);
+        }
+        std::vector<float> inv2;
+        for (double v : inv) {
+            inv2.push_back((float)v);
+            inv2.push_back((float)(v - (double)(float)v));
+        }
+        if ((e = (cudaError_t)poro::upload_direct_tables(degree_N, ent, list)) != cudaSuccess ||
+            (e = upload((void**)&c->dref.inv_d, inv.data(), inv.size() * sizeof(double))) != cudaSuccess ||
+            (e = upload((void**)&c->dref.inv_d2, inv2.data(), inv2.size() * sizeof(float))) != cudaSuccess) {
+            free_reference(c);
+            cudaStreamDestroy(c->stream);
+            delete c;
+            return cuda_fail(nullptr, e, "poro_create: upload (integer rows)");
+        }
+    }
     {
         // full-row CSR of Khat^j in binary64 and Z for the dense-LU comparator
         const int B = c->B;
@@ -388,72 +382,8 @@ poro_status poro_create_system(int device, int degree_N, poro_precision precisio
         }
     }
     if (precision != PORO_FP64) {
-        // Residual CSR of Khat^j (all rows): every row l of every Khat^j is an
-        // integer row over a common denominator d (the reference matrices are
-        // rational with small denominators), so an entry is packed as
-        // (numerator << 7) | column and the row carries 1/d as a
-        // double-binary32 pair.  The kernel multiplies the numerators with
-        // 21-bit fixed-point values and sums in 64-bit integers, exact while a
-        // row's sum of |numerators| stays below 2^22 (3.6e6 at N = 6).
         const int B = c->B;
-        std::vector<float> zf(c->ref.zinv.begin(), c->ref.zinv.end());
-        std::vector<int32_t> rrow, rint;
-        std::vector<float> rinv;
-        std::string rerr;
-        for (int j = 0; j < 3 && rerr.empty(); ++j) {
-            rrow.push_back((int32_t)rint.size());
-            for (int l = 0; l < B && rerr.empty(); ++l) {
-                const double* row = c->ref.khat.data() + ((size_t)j * B + l) * B;
-                int64_t d = 1;
-                for (int m = 0; m < B; ++m) {
-                    int64_t num = 0, den = 1;
-                    if (row[m] == 0.0) continue;
-                    if (!rational_of(row[m], num, den)) {
-                        rerr = "Khat entry is not a small-denominator rational";
-                        break;
-                    }
-                    d = d / std::gcd(d, den) * den;
-                    if (d > (1 << 30)) {
-                        rerr = "Khat row denominator too large";
-                        break;
-                    }
-                }
-                int64_t abs_sum = 0;  // the residual's 64-bit integer sums need sum |c| < 2^22
-                for (int m = 0; m < B && rerr.empty(); ++m) {
-                    if (row[m] == 0.0) continue;
-                    const double cv = row[m] * (double)d;
-                    const int64_t ci = std::llround(cv);
-                    abs_sum += std::llabs(ci);
-                    if (std::fabs(cv - (double)ci) > 1e-6 || std::llabs(ci) >= (1 << 23) || abs_sum >= (1 << 22)) {
-                        rerr = "Khat numerator out of range";
-                        break;
-                    }
-                    rint.push_back((int32_t)(((uint32_t)(int32_t)ci << 7) | (uint32_t)m));
-                }
-                const double inv = 1.0 / (double)d;
-                const float ih = (float)inv;
-                rinv.push_back(ih);
-                rinv.push_back((float)(inv - (double)ih));
-                rrow.push_back((int32_t)rint.size());
-            }
-        }
-        // residual row order per warp count: a row costs its Khat entries (all
-        // directions) plus a fixed share for the star and time terms
-        auto deal = [&](int warps) {
-            std::vector<int64_t> cost(B);
-            for (int l = 0; l < B; ++l) {
-                cost[l] = 40;
-                for (int j = 0; j < 3; ++j) cost[l] += rrow[j * (B + 1) + l + 1] - rrow[j * (B + 1) + l];
-            }
-            return deal_rows(cost, warps, false);
-        };
-        const std::vector<int32_t> ord8 = deal(8), ord4 = deal(4), ord2 = deal(2);
-        if (!rerr.empty()) {
-            free_reference(c);
-            cudaStreamDestroy(c->stream);
-            delete c;
-            return fail(nullptr, PORO_ENUMERIC, "poro_create: " + rerr);
-        }
+        const std::vector<float> zf(c->ref.zinv.begin(), c->ref.zinv.end());
         // tensor-core images of the blocks, hi image then lo image in the
         // K-major core-matrix layout: tf32 words, or bf16 for the bf16 form
         const bool bf16 = precision == PORO_BF16X3_REFINE;
@@ -493,14 +423,7 @@ poro_status poro_create_system(int device, int degree_N, poro_precision precisio
             }
         }
         c->mref.base = &c->dref;
-        if ((e = (cudaError_t)poro::upload_residual_table(degree_N, rrow.data(), rint.data(), (int)rint.size())) !=
-                cudaSuccess ||
-
-            (e = upload((void**)&c->mref.res_inv, rinv.data(), rinv.size() * sizeof(float))) != cudaSuccess ||
-            (e = upload((void**)&c->mref.res_order8, ord8.data(), ord8.size() * sizeof(int32_t))) != cudaSuccess ||
-            (e = upload((void**)&c->mref.res_order4, ord4.data(), ord4.size() * sizeof(int32_t))) != cudaSuccess ||
-            (e = upload((void**)&c->mref.res_order2, ord2.data(), ord2.size() * sizeof(int32_t))) != cudaSuccess ||
-            (e = upload((void**)&c->mref.zinv_f32, zf.data(), zf.size() * sizeof(float))) != cudaSuccess ||
+        if ((e = upload((void**)&c->mref.zinv_f32, zf.data(), zf.size() * sizeof(float))) != cudaSuccess ||
             (e = upload((void**)&c->mref.khat_tc, tci.data(), tci.size())) != cudaSuccess ||
             (e = cudaMalloc((void**)&c->mref.status, sizeof(int32_t))) != cudaSuccess ||
             (e = cudaMemset(c->mref.status, 0, sizeof(int32_t))) != cudaSuccess) {
@@ -806,9 +729,9 @@ static poro_status dispatch_predict(poro_ctx* c, int64_t first, int64_t count, c
         rc = poro::launch_stp_subcell(c->dref, c->sub, count, q0, ec, c->d_evar + first * poro::subcell_var_stride(),
                                       qt, iout, c->d_iters + first, c->sub_tol, c->sub_max_iter, st);
     } else if (c->system == PORO_SYSTEM_MAXWELL) {
-        rc = poro::launch_stp_fp64_maxwell(c->dref, nullptr, count, q0, ec, qt, iout, st);
+        rc = poro::launch_stp_fp64_maxwell(c->dref, count, q0, ec, qt, iout, st);
     } else if (c->system == PORO_SYSTEM_VISCOELASTIC) {
-        rc = poro::launch_stp_fp64_visco(c->dref, nullptr, count, q0, ec, qt, iout, st);
+        rc = poro::launch_stp_fp64_visco(c->dref, count, q0, ec, qt, iout, st);
     } else if (c->prec == PORO_FP64) {
         rc = poro::launch_stp_fp64(c->dref, nullptr, count, q0, ec, qt, iout, st, c->variant);
     } else {
@@ -2100,9 +2023,9 @@ poro_status poro_autotune(poro_ctx* c, int64_t sample, int32_t* variant_out, dou
     return PORO_OK;
 }
 
-// tile choices: CTA-size variant x operand layout caps (A buffers, Khat slots)
-static const int kTileCaps[6][2] = {{3, 3}, {2, 3}, {1, 3}, {2, 2}, {1, 2}, {1, 1}};
-
+// tile choices: CTA-size variant x 6 operand layouts.  No kernel has more than
+// one operand layout now, so the layouts of one CTA size run alike; the
+// choices stay for programs that keep one.
 static bool tile_choice_valid(const poro_ctx* c, int choice) {
     if (choice < 0 || choice >= PORO_TILE_CHOICES) return false;
     const int cta = choice / 6, lay = choice % 6;
@@ -2114,8 +2037,6 @@ static bool tile_choice_valid(const poro_ctx* c, int choice) {
 
 static void apply_tile_choice(poro_ctx* c, int choice) {
     c->variant = choice / 6;
-    c->mref.cap_a = kTileCaps[choice % 6][0];
-    c->mref.cap_b = kTileCaps[choice % 6][1];
 }
 
 poro_status poro_set_tiles(poro_ctx* c, int32_t choice) {
@@ -2133,12 +2054,7 @@ poro_status poro_autotune_tiles(poro_ctx* c, int64_t sample, int32_t* choice_out
     if (!c->d_econst || c->n_elem <= 0) return fail(c, PORO_ESTATE, "poro_autotune_tiles: no element population loaded");
     cudaSetDevice(c->device);
     const int64_t n = std::max<int64_t>(1, std::min(sample > 0 ? sample : c->n_elem, c->n_elem));
-    const int saved_v = c->variant, saved_a = c->mref.cap_a, saved_b = c->mref.cap_b;
-    auto restore = [&] {
-        c->variant = saved_v;
-        c->mref.cap_a = saved_a;
-        c->mref.cap_b = saved_b;
-    };
+    const int saved_v = c->variant;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
         if (e0) cudaEventDestroy(e0);
@@ -2170,7 +2086,7 @@ poro_status poro_autotune_tiles(poro_ctx* c, int64_t sample, int32_t* choice_out
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    restore();
+    c->variant = saved_v;
     if (st != PORO_OK) return st;
     apply_tile_choice(c, bestc);
     if (choice_out) *choice_out = bestc;

@@ -120,12 +120,14 @@ PORO_HD constexpr int elem_const_stride(int N) {
 //   star[3][54]       A^{j*} = dt A^j on the union pattern
 //   zinv_uf[T][T]     (Z - e I)^{-1}, e = E*_{uf,uf} (row-major, [u][s])
 //   e, g, dt, pad     E*_{uf,uf}, E*_{u,uf}, time step
-PORO_HD constexpr int elem_const_stride(int N) {
-    // keep 16-byte alignment of every element's block
-    return (3 * STAR_NNZ + (N + 1) * (N + 1) + 4 + 1) & ~1;
-}
+//   iso[16]           (from an even offset) the star products of the isotropic
+//                     Jacobians in factored form: n^j = -mu dt grad xi_j
+//                     [3][3], then lambda_c / mu, M alpha / mu, M / mu,
+//                     m / (D mu), rho_F / (D mu), rho / (D mu), pad
 PORO_HD constexpr int ec_zinv(int) { return 3 * STAR_NNZ; }
 PORO_HD constexpr int ec_scalars(int N) { return 3 * STAR_NNZ + (N + 1) * (N + 1); }
+PORO_HD constexpr int ec_iso(int N) { return (ec_scalars(N) + 4 + 1) & ~1; }
+PORO_HD constexpr int elem_const_stride(int N) { return ec_iso(N) + 16; }  // keeps every element's block 16-byte aligned
 
 // Khat^j restricted to the columns of one degree block g, in CSR over the
 // rows l < o_g (the only rows Lemma 1 leaves non-zero); entries
@@ -219,18 +221,16 @@ struct DeviceReference {
     // starts, then the lists
     int32_t* lists[3] = {nullptr, nullptr, nullptr};
     int32_t list_base[3][MAX_N + 1][3] = {};
+    // 1 / d_l of the integer Khat rows (khat_tables) [B], and the same as
+    // (hi, lo) binary32 words [B][2]
+    double* inv_d = nullptr;
+    float* inv_d2 = nullptr;
 };
 
-// Extra device data of the mixed-precision (refinement) path.
+// Extra device data of the mixed-precision path (the unrefined sweeps).
 struct MixedReference {
     const DeviceReference* base = nullptr;
     bool bf16 = false;              // sweeps' split products in bf16 (else tf32)
-    float* res_inv = nullptr;       // [3][B][2] 1 / d_jl as (hi, lo) binary32 words
-    // residual rows dealt to 8, 4 and 2 warps (longest work first, each row to
-    // the least loaded warp): [warps + 1] list starts, then the lists
-    int32_t* res_order8 = nullptr;
-    int32_t* res_order4 = nullptr;
-    int32_t* res_order2 = nullptr;
     float* zinv_f32 = nullptr;      // [T][T]
     // tensor-core images of Khat^j restricted to block g (rows l < o_g, columns
     // of the block), K-major core-matrix layout of tc_np(g) x tc_kp(g) words
@@ -240,16 +240,7 @@ struct MixedReference {
     int32_t tc_off[MAX_N + 1][3] = {};
     int32_t* status = nullptr;      // device word: 1 after a bounded wait gave up
     long long wait_limit = 0;       // SM clocks a wait of the sweeps may take (0: about 1 s)
-    // operand layout of the tensor-core sweeps (the autotuner's tile choice):
-    // at most cap_a A-tile buffers and cap_b Khat image slots per degree block
-    // (3, 3: as many as fit in the operand region)
-    int cap_a = 3, cap_b = 3;
 };
-
-// Fill the constant-memory residual table of degree N on the current device
-// (row pointers relative to the entries); idempotent, same data for every
-// context of that degree.
-int upload_residual_table(int N, const int32_t* rows, const int32_t* entries, int n_entries);
 
 // Per-run buffers of a predictor launch that covers the elements of several
 // simulations of the same degree and precision (the server's batched mode):
@@ -262,8 +253,8 @@ struct RunPtrs {
     double* iout;          // [ne][13][B] or nullptr
 };
 
-// Launch the mixed-precision predictor (binary32 sweeps, `refine` residual
-// corrections in double-binary32) for `count` elements.  With `runs`
+// Launch the mixed-precision predictor for `count` elements: binary32 sweeps
+// (refine 0), double-binary32 (1) or binary64 (2).  With `runs`
 // (device array) and `item_run`, the items come from several runs and q0,
 // econst, qt, iout are ignored.
 int launch_stp_mixed(const MixedReference& ref, int refine, const int32_t* elems, int64_t count,
@@ -392,8 +383,29 @@ int group_enqueue(RunGroup* g, int64_t n_cycles, std::string& err);
 poro_status group_finish(RunGroup* g, std::string& err);
 void group_destroy(RunGroup* g);
 
+// x = num / den with den <= 10^6 if x is such a rational to 1e-14 relative
+bool rational_of(double x, int64_t& num, int64_t& den);
+// Integer Khat rows in passes of at most `columns` columns (direction, mode) of
+// X: entries (column * stride, numerator) pass by pass, 1 / d_l per row, and
+// (appended to list) per pass the rows dealt to `warps` warps, [warps + 1]
+// starts, then words l << 21 | entries << 13 | first entry.
+bool khat_tables(const ReferenceData& R, int columns, int stride, int warps, std::vector<int32_t>& ent,
+                 std::vector<int32_t>& list, std::vector<double>& inv_d, std::string& err);
+// The same for Biot's predictor kernel (stp_direct.cu), lists of all its warp
+// counts; then their upload (once per device and degree).
+bool direct_tables(const ReferenceData& R, std::vector<int32_t>& ent, std::vector<int32_t>& list,
+                   std::vector<double>& inv_d, std::string& err);
+int upload_direct_tables(int N, const std::vector<int32_t>& ent, const std::vector<int32_t>& list);
+// Biot's predictor in binary64 or (dw) double-binary32, arguments as for
+// launch_stp_fp64.  whole_nan: a non-finite value makes the element's whole
+// result NaN; status, wait_limit: the bounded wait of the double-binary32 form.
+int launch_stp_direct(const DeviceReference& ref, bool dw, bool whole_nan, int32_t* status, long long wait_limit,
+                      const int32_t* elems, int64_t count, const double* q0, const double* econst, double* qt,
+                      double* iout, void* stream, int variant, const RunPtrs* runs,
+                      const int32_t* item_run);
+
 // Launch the FP64 Algorithm-3 predictor for `count` elements.
-// q0[count][13][B], econst[count][stride], qt (nullable), iout (nullable).
+// q0[count][13][B], econst[count][stride], qt, iout nullable.
 // `elems` (nullable): element index list; outputs are indexed by element.
 // `variant` selects the CTA size (0: default, 1: the alternative the
 // autotuner may pick).  `runs` / `item_run`: items of several runs, as for
@@ -403,8 +415,8 @@ int launch_stp_fp64(const DeviceReference& ref, const int32_t* elems, int64_t co
                     const RunPtrs* runs = nullptr, const int32_t* item_run = nullptr);
 // The same kernel for the damped Maxwell system (q0 [count][6][B], econst
 // [count][maxwell::elem_const_stride(N)], qt [count][6][B][T]).
-int launch_stp_fp64_maxwell(const DeviceReference& ref, const int32_t* elems, int64_t count, const double* q0,
-                            const double* econst, double* qt, double* iout, void* stream);
+int launch_stp_fp64_maxwell(const DeviceReference& ref, int64_t count, const double* q0, const double* econst,
+                            double* qt, double* iout, void* stream);
 // Sub-cell material predictor (subcell.cu): evar [count][subcell_var_stride()],
 // iters [count] (iterations of each element, negative if not converged).
 int launch_stp_subcell(const DeviceReference& ref, const SubcellReference& sub, int64_t count, const double* q0,
@@ -412,7 +424,7 @@ int launch_stp_subcell(const DeviceReference& ref, const SubcellReference& sub, 
                        double tol, int max_iter, void* stream);
 // ... and for the viscoelastic system (q0 [count][27][B], econst
 // [count][visco::elem_const_stride(N)], qt [count][27][B][T]).
-int launch_stp_fp64_visco(const DeviceReference& ref, const int32_t* elems, int64_t count, const double* q0,
-                          const double* econst, double* qt, double* iout, void* stream);
+int launch_stp_fp64_visco(const DeviceReference& ref, int64_t count, const double* q0, const double* econst,
+                            double* qt, double* iout, void* stream);
 
 }  // namespace poro

@@ -358,6 +358,34 @@ bool tet_geometry(const double* v, double jinv[3][3], double& volume, double& in
     return true;
 }
 
+// x = num / den with den <= 10^6 (continued-fraction convergents), if x is
+// such a rational to 1e-14 relative
+bool rational_of(double x, int64_t& num, int64_t& den) {
+    const double ax = std::fabs(x);
+    int64_t h0 = 0, h1 = 1, k0 = 1, k1 = 0;
+    double r = ax;
+    for (int it = 0; it < 64; ++it) {
+        const double a = std::floor(r);
+        if (a > 9.0e15) break;
+        const int64_t ai = (int64_t)a;
+        const int64_t h2 = ai * h1 + h0, k2 = ai * k1 + k0;
+        if (k2 > 1000000) break;
+        h0 = h1;
+        h1 = h2;
+        k0 = k1;
+        k1 = k2;
+        if (std::fabs((double)h1 / (double)k1 - ax) <= 1e-14 * ax) {
+            num = x < 0 ? -h1 : h1;
+            den = k1;
+            return true;
+        }
+        const double f = r - a;
+        if (f <= 0.0) break;
+        r = 1.0 / f;
+    }
+    return false;
+}
+
 bool element_constants(const ReferenceData& ref, const double* v12, const poro_material& mat,
                        double dt, double* out, std::string& err) {
     if (!(dt > 0.0) || !std::isfinite(dt)) { err = "element: time step must be positive"; return false; }
@@ -384,6 +412,20 @@ bool element_constants(const ReferenceData& ref, const double* v12, const poro_m
     sc[0] = e;
     sc[1] = g;
     sc[2] = dt;
+    // factored star products: n^j from the shear entries -mu, the ratios from
+    // the x-direction Jacobian
+    double* iso = out + ec_iso(ref.N);
+    const double(*A)[NQ] = abc[0];
+    const double mu = -A[SXY][QV];
+    const double md = mu * dt, md_low = std::fma(mu, dt, -md);  // one rounding each, like the stars' entries
+    for (int j = 0; j < 3; ++j)
+        for (int d = 0; d < 3; ++d) iso[3 * j + d] = -std::fma(md, jinv[j][d], md_low * jinv[j][d]);
+    iso[9] = -A[SYY][QU] / mu;
+    iso[10] = A[QP][QU] / mu;
+    iso[11] = A[QP][QUF] / mu;
+    iso[12] = -A[QU][SXX] / mu;
+    iso[13] = A[QUF][SXX] / mu;
+    iso[14] = A[QUF][QP] / mu;
     return true;
 }
 

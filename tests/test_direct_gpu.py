@@ -1,0 +1,79 @@
+"""GPU tests of the fixed-point predictor of Biot's system beyond the oracle parity tests: scale invariance to the last
+bit, the widest ranges, non-finite rows."""
+import numpy as np
+import pytest
+
+from _oracle_cases import oracle_predictor, population, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2108_10565_gb300 import _lib
+
+    return _lib
+
+
+def _predict(L, d, precision, q0, sweeps=1):
+    ctx = L.poro_create(0, d["N"], precision)
+    try:
+        if precision:
+            L.poro_set_refinement(ctx, sweeps)
+        L.poro_set_isolated(ctx, d["vertices"], d["materials"], d["dt"])
+        L.poro_set_dofs(ctx, q0)
+        L.poro_predict(ctx)
+        return L.poro_get_predictor(ctx, 0, q0.shape[0])
+    finally:
+        L.poro_destroy(ctx)
+
+
+@pytest.mark.parametrize("precision,sweeps,powers", [(0, 1, (-900, -300, 300, 900)), (1, 1, (-60, 60)), (1, 2, (-300, 300))])
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6])
+def test_power_of_two_scaling_is_exact(L, N, precision, sweeps, powers):
+    """The fixed-point scales are powers of two that follow the data, so Q0 times 2^k gives the predictor times 2^k bit by
+    bit (away from the ends of the arithmetic's range: the star products carry up to about 1e+-20)."""
+    d = population(7, N, seed=800 + N)
+    ref = _predict(L, d, precision, d["Q0"], sweeps)
+    for k in powers:
+        got = _predict(L, d, precision, np.ldexp(d["Q0"], k), sweeps)
+        np.testing.assert_array_equal(np.ldexp(got, -k), ref, err_msg=f"2^{k}")
+
+
+@pytest.mark.parametrize("N", [1, 3, 6])
+@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 1e-10), (2, 1e-10)])
+def test_rows_of_unlike_size(L, N, precision, tol):
+    """Quantities many orders of magnitude apart (stresses in Pa beside velocities in m/s), zero rows among them: every
+    quantity of the predictor is accurate by itself where the data reach it at its own size."""
+    d = population(5, N, seed=900 + N)
+    q0 = d["Q0"].copy()
+    q0[:, [0, 1, 2, 3, 4, 5, 9]] *= 1e7
+    q0[:, 10:] = 0.0
+    q0[1] = 0.0
+    qt = _predict(L, d, precision, q0)
+    assert not qt[1].any()
+    d = dict(d, Q0=q0)
+    for i in (0, 2, 3, 4):
+        ref = oracle_predictor(d, i)
+        for p in range(13):
+            assert rel_l2(qt[i, p], ref[p]) <= tol, (i, p)
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("mode", [0, -1])
+def test_non_finite_binary64_rows(L, bad, mode):
+    """A non-finite entry of one element's data makes what depends on it non-finite and touches no other element."""
+    N = 4
+    d = population(6, N, seed=77)
+    q0 = d["Q0"].copy()
+    q0[2, 7, mode] = bad
+    clean, dirty = _predict(L, d, 0, d["Q0"]), _predict(L, d, 0, q0)
+    keep = np.arange(6) != 2
+    np.testing.assert_array_equal(clean[keep], dirty[keep])
+    assert not np.isfinite(dirty[2, 7]).all()
+    if mode == -1:  # the last mode feeds the lower ones
+        assert not np.isfinite(dirty[2, :, 0]).all()
