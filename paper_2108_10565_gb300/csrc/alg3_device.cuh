@@ -1,25 +1,54 @@
 // Device building blocks of the degree-block back-substitution (Section
-// "Block-wise back-substitution", Algorithm 3), templated on the arithmetic
-// type so the binary64 kernel and the binary32 sweeps of the refinement
-// kernel run the same code.
+// "Block-wise back-substitution", Algorithm 3): the binary64 sweep of the
+// systems other than Biot's and of the sub-cell iteration, and the layout that
+// the binary32 sweep of stp_mixed.cu shares.
 //
 // Shared-memory layout of one element's b / Q tensor: quantity p at offset
 // p * QS, mode l at l * T, time mode u at u, where the quantity stride QS is
-// B * T padded so that QS = T (mod 32): the 13 T lanes (p, u) of one mode then
-// fall on consecutive 4-byte banks (conflict-free).  The star products X use
-// the same rule with the block size d_g in place of B.
+// B * T padded so that the T lanes (p, u) of neighbouring quantities fall on
+// consecutive banks: QS = T (mod 32) in 4-byte, (mod 16) in 8-byte words.
 #pragma once
 
 #include <cuda_runtime.h>
 
+#include "fixed_device.cuh"
 #include "poro_internal.h"
 
 namespace poro {
 
 __host__ __device__ constexpr int bank_stride(int n, int T) { return n + ((T - n % 32) + 32) % 32; }
 
-template <int T, class Real>
-__device__ __forceinline__ void solve_row(Real* row, const Real* Zi);
+// row <- Z^{-1} row, tridiagonal: row u is 1 / (2 (2u - 1)) on u - 1 (u = 0: 1/2
+// on itself) and -1 / (2 (2u + 3)) on u + 1 (the last: 1 / (2 (2u + 1)) on
+// itself); the high words of the result go to qmax[u] (a maximum)
+template <int T>
+__device__ __forceinline__ void solve_plain(double* row, uint32_t* qmax) {
+    double x[T];
+#pragma unroll
+    for (int s = 0; s < T; ++s) x[s] = row[s];
+#pragma unroll
+    for (int u = 0; u < T; ++u) {
+        const double lo = u == 0 ? 0.5 : 0.5 / (2 * u - 1), hi = u == T - 1 ? 0.5 / (2 * u + 1) : -0.5 / (2 * u + 3);
+        const double y = fma(hi, x[u == T - 1 ? u : u + 1], lo * x[u == 0 ? 0 : u - 1]);
+        row[u] = y;
+        atomicMax(qmax + u, (uint32_t)__double2hiint(y) & 0x7FFFFFFFu);
+    }
+}
+// row <- Zi row, dense
+template <int T>
+__device__ __forceinline__ void solve_row(double* row, const double* Zi, uint32_t* qmax) {
+    double x[T];
+#pragma unroll
+    for (int s = 0; s < T; ++s) x[s] = row[s];
+#pragma unroll
+    for (int u = 0; u < T; ++u) {
+        double y = 0.0;
+#pragma unroll
+        for (int s = 0; s < T; ++s) y = fma(Zi[u * T + s], x[s], y);
+        row[u] = y;
+        atomicMax(qmax + u, (uint32_t)__double2hiint(y) & 0x7FFFFFFFu);
+    }
+}
 
 // The linear system of the predictor: its quantities, the union pattern of
 // its reference Jacobians and the structure of its source matrix E (upper
@@ -69,37 +98,37 @@ struct ViscoSystem {
     // modes [o, o + d) of one degree block; zsh: NMECH matrices (Z - e_l I)^{-1};
     // cp: per mechanism the couplings (normal diagonal, normal off-diagonal,
     // shear) of E*.  The caller's barrier follows.
-    template <int T, int NT, int QS, class Real>
-    __device__ static void solve_block(Real* bq, int o, int d, const Real* zin, const Real* zsh, const Real* cp) {
+    template <int T, int NT, int QS>
+    __device__ static void solve_block(double* bq, int o, int d, const double* zsh, const double* cp, uint32_t* qmax) {
         const int tid = threadIdx.x;
         constexpr int NM = visco::NMECH;
         for (int it = tid; it < (3 + 6 * NM) * d; it += NT) {
-            const int kind = it / d, m = o + it % d;
-            if (kind < 3) solve_row<T>(bq + (6 + kind) * QS + m * T, zin);
-            else solve_row<T>(bq + (9 + (kind - 3)) * QS + m * T, zsh + ((kind - 3) / 6) * T * T);
+            const int kind = it / d, m = o + it % d, q = 6 + kind;
+            if (kind < 3) solve_plain<T>(bq + q * QS + m * T, qmax + q * T);
+            else solve_row<T>(bq + q * QS + m * T, zsh + ((kind - 3) / 6) * T * T, qmax + q * T);
         }
         __syncthreads();
         for (int it = tid; it < 6 * d; it += NT) {
             const int c = it / d, m = o + it % d;
-            Real* row = bq + c * QS + m * T;
+            double* row = bq + c * QS + m * T;
 #pragma unroll
             for (int l = 0; l < NM; ++l) {
-                const Real* th = bq + (9 + 6 * l) * QS + m * T;
+                const double* th = bq + (9 + 6 * l) * QS + m * T;
                 if (c < 3) {
                     // normal stress c: (Ylam + 2 Ymu) on th_cc, Ylam on the other two
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
-                        const Real g = k == c ? cp[3 * l] : cp[3 * l + 1];
+                        const double g = k == c ? cp[3 * l] : cp[3 * l + 1];
 #pragma unroll
                         for (int u = 0; u < T; ++u) row[u] = fma(g, th[k * QS + u], row[u]);
                     }
                 } else {
-                    const Real g = cp[3 * l + 2];
+                    const double g = cp[3 * l + 2];
 #pragma unroll
                     for (int u = 0; u < T; ++u) row[u] = fma(g, th[c * QS + u], row[u]);
                 }
             }
-            solve_row<T>(row, zin);
+            solve_plain<T>(row, qmax + c * T);
         }
     }
 };
@@ -117,166 +146,186 @@ struct Alg3Shape {
     static constexpr int PUL = (PT + 31) / 32;             // pairs per lane
 };
 
-// Khat^j block CSR (rows l < o_g, columns m_local of block g) for one precision
-template <class Real>
-struct KhatBlocks {
-    const Real* val;
-    const int32_t* col;
-    const int32_t* row;
-    int32_t row_base[MAX_N + 1][3];
-    // optional (one direction per pass): block (g, j)'s rows dealt to the
-    // warps, [warps + 1] starts then the lists, at lists + list_base[g][j]
-    const int32_t* lists = nullptr;
-    int32_t list_base[MAX_N + 1][3];
+// The binary64 sweep's layout: quantity stride for 8-byte words, and the
+// integer X with room for XC columns (direction, mode) of PT rows (p, u)
+template <int N, class Sys, int XC_>
+struct SweepShape {
+    static constexpr int NQ = Sys::NQ, B = n_modes(N), T = N + 1, XC = XC_;
+    static constexpr int QS = B * T + ((T - B * T % 16) + 16) % 16, SQ = NQ * QS;
+    static constexpr int PT = NQ * T, PUL = (PT + 31) / 32;
+    static constexpr int X_WORDS = XC * PT + 32;      // 8-byte words (slack read by idle lanes)
+    // scratch in 32-bit words: max |Q| of two blocks, row scales, row starts of the star pattern
+    static constexpr int I_SCALE = 2 * PT, I_ROW = 3 * PT, I_WORDS = (3 * PT + NQ + 1 + 1) & ~1;
 };
 
-template <int T, class Real>
-__device__ __forceinline__ void solve_row(Real* row, const Real* Zi) {
-    Real x[T];
+// Integer Khat rows (khat_tables with stride PT and this kernel's XC and warps)
+struct KhatRows {
+    const int2* ent;
+    const int32_t* list;
+    const double* inv_d;
+};
+
+// Scratch of the sweep in shared memory
+template <class S>
+struct SweepScratch {
+    int2* X;
+    int* w;              // I_WORDS
+    const double* smax;  // [NNZ] max_j |star_j|
+    __device__ uint32_t* qmax(int buf) const { return reinterpret_cast<uint32_t*>(w) + buf * S::PT; }
+    __device__ int* scale() const { return w + S::I_SCALE; }
+    __device__ int* row() const { return w + S::I_ROW; }
+};
+// clears the maxima and fills the row starts and smax; the caller's barrier follows
+template <int NT, class S, class Sys>
+__device__ void sweep_setup(const SweepScratch<S>& W, double* smax, const double* star) {
+    for (int i = threadIdx.x; i < 2 * S::PT; i += NT) W.w[i] = 0;
+    for (int i = threadIdx.x; i <= Sys::NQ; i += NT) {
+        int n = 0;
+        while (n < Sys::NNZ && Sys::row(n) < i) ++n;
+        W.row()[i] = n;
+    }
+    for (int i = threadIdx.x; i < Sys::NNZ; i += NT)
+        smax[i] = fmax(fabs(star[i]), fmax(fabs(star[Sys::NNZ + i]), fabs(star[2 * Sys::NNZ + i])));
+}
+
+// dst[p, l, u] += SIGN sum_j sum_m Khat^j[l, o_g + m] X^j[p, m, u] for l < o_g with
+// X^j[p, m, u] = sum_q A^{j*}_pq src[q, o_g + m, u], X in fixed point: one scale per
+// row (p, u) from the block's max |src| in qmax.  Lanes run over the rows; the
+// l are dealt to the warps.  Clears qmax_next; `list` moves to the next
+// block's lists.  Begins after and ends with a barrier.
+template <int N, int NT, class Sys, class S, int SIGN>
+__device__ void khat_block(double* dst, const double* src, int g, const double* star, const KhatRows& K,
+                           const int32_t*& list, const SweepScratch<S>& W, const uint32_t* qmax, uint32_t* qmax_next) {
+    constexpr int NQ = Sys::NQ, NNZ = Sys::NNZ, T = S::T, QS = S::QS, PT = S::PT, PUL = S::PUL, NW = NT / 32;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int o = block_offset(g), d = block_size(g), dm = pass_modes(g, S::XC);
+    for (int r = tid; r < PT; r += NT) {
+        const int p = r / T, u = r - p * T;
+        double b = 0.0;
+        for (int n = W.row()[p]; n < W.row()[p + 1]; ++n) b += W.smax[n] * bound_of(qmax[Sys::col(n) * T + u], 0.0);
+        W.scale()[r] = row_scale(b);
+        qmax_next[r] = 0u;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int m0 = 0; m0 < d; m0 += dm) {
+        const int nm = min(dm, d - m0);
+        // X, quantised: column j * dm + ml
+        for (int it = tid; it < 3 * nm * T; it += NT) {
+            const int j = it / (nm * T), r = it - j * (nm * T), ml = r / T, u = r - ml * T;
+            const double* q = src + (o + m0 + ml) * T + u;
+            const double* sj = star + j * NNZ;
+            double qv[NQ], acc[NQ];
 #pragma unroll
-    for (int s = 0; s < T; ++s) x[s] = row[s];
+            for (int p = 0; p < NQ; ++p) {
+                qv[p] = q[p * QS];
+                acc[p] = 0.0;
+            }
 #pragma unroll
-    for (int u = 0; u < T; ++u) {
-        Real acc = Real(0);
+            for (int n = 0; n < NNZ; ++n) acc[Sys::row(n)] = fma(sj[n], qv[Sys::col(n)], acc[Sys::row(n)]);
+            int2* x = W.X + (j * dm + ml) * PT + u;
+            const int* sc = W.scale() + u;
 #pragma unroll
-        for (int s = 0; s < T; ++s) acc = fma(Zi[u * T + s], x[s], acc);
-        row[u] = acc;
+            for (int p = 0; p < NQ; ++p) x[p * T] = quantise(acc[p], sc[p * T]);
+        }
+        __syncthreads();
+        const int i1 = __ldg(list + warp + 1);
+        const int32_t* rows = list + NW + 1;
+#pragma unroll 1
+        for (int i = __ldg(list + warp); i < i1; ++i) {
+            const int w = __ldg(rows + i), l = w >> 21, n0 = w & 8191, n1 = n0 + ((w >> 13) & 255);
+            const int2* xl = W.X + lane;
+            long long hi[PUL];
+            long long lo[PUL];
+#pragma unroll
+            for (int k = 0; k < PUL; ++k) {
+                hi[k] = 0;
+                lo[k] = 0;
+            }
+#pragma unroll 4
+            for (int n = n0; n < n1; ++n) {
+                const int2 en = __ldg(K.ent + n);
+                const int2* xc = xl + en.x;
+#pragma unroll
+                for (int k = 0; k < PUL; ++k)
+                    fixed_mac(en.y, xc[32 * k], hi[k], lo[k]);
+            }
+            const double inv = SIGN * __ldg(K.inv_d + l);
+#pragma unroll
+            for (int k = 0; k < PUL; ++k) {
+                const int r = lane + 32 * k;
+                if (r < PT) {
+                    double* b = dst + (r / T) * QS + l * T + r % T;
+                    *b = fma(fixed_sum(hi[k], lo[k], W.scale()[r]), inv, *b);
+                }
+            }
+        }
+        list = rows + __ldg(list + NW);
+        __syncthreads();
     }
 }
 
 // b[p,l,u] = (S^{-1} w)_u q0[p,l] with (S^{-1} w)_u = (2u+1)(-1)^u
-template <int N, int NT, class Real, class In, int NQ_ = NQ>
-__device__ __forceinline__ void init_rhs(Real* bq, const In* q0) {
-    using S = Alg3Shape<N, NQ_>;
-    for (int i = threadIdx.x; i < NQ_ * S::B; i += NT) {
-        const Real v = (Real)q0[i];
+template <int NT, class S>
+__device__ __forceinline__ void init_rhs(double* bq, const double* q0) {
+    for (int i = threadIdx.x; i < S::NQ * S::B; i += NT) {
+        const double v = q0[i];
         const int p = i / S::B, l = i % S::B;
-        Real* row = bq + p * S::QS + l * S::T;
+        double* row = bq + p * S::QS + l * S::T;
 #pragma unroll
-        for (int u = 0; u < S::T; ++u) row[u] = Real((2 * u + 1) * ((u & 1) ? -1 : 1)) * v;
+        for (int u = 0; u < S::T; ++u) row[u] = (double)((2 * u + 1) * ((u & 1) ? -1 : 1)) * v;
     }
 }
 
-// In-place sweep: on entry bq holds b, on exit the solution Q.  X is a
-// scratch area of JX * Sys::NQ * XSMAX values in shared memory; star[3][NNZ]
-// the element's reference Jacobians on the union pattern; zuf = (Z - e I)^{-1},
-// zin = Z^{-1}; gcoup = the coupling entry g of E* (Biot: E*_{u,uf}); for
-// two-phase systems zuf holds their NSHM shifted matrices and cpl their
-// couplings.  JX
-// directions are handled per pass (1 or 3).  Ends with a barrier.
-template <int N, int NT, class Real, int JX, class Sys = BiotSystem>
-__device__ void alg3_sweep(Real* bq, Real* X, const Real* star, const Real* zuf, const Real* zin,
-                           const Real gcoup, const KhatBlocks<Real>& K, const Real* cpl = nullptr) {
-    constexpr int NQ = Sys::NQ, STAR_NNZ = Sys::NNZ;
-    using S = Alg3Shape<N, NQ>;
-    constexpr int T = S::T, QS = S::QS, PT = S::PT, PUL = S::PUL, NW = NT / 32;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    int lp[PUL], lu[PUL];
-#pragma unroll
-    for (int k = 0; k < PUL; ++k) {
-        const int pu = lane + 32 * k;
-        lp[k] = pu < PT ? pu / T : 0;
-        lu[k] = pu < PT ? pu % T : 0;
-    }
+// In-place sweep: on entry bq holds b, on exit the solution Q.  star[3][NNZ]:
+// the element's reference Jacobians on the union pattern; zsh: its NSHM shifted
+// matrices (Z - e I)^{-1}; gcoup = the coupling entry g of E* (Biot: E*_{u,uf});
+// cpl: the couplings of two-phase systems.  Begins after and ends with a
+// barrier; both maxima are clear at its ends.
+template <int N, int NT, class Sys, class S>
+__device__ void alg3_sweep(double* bq, const double* star, const double* zsh, const double gcoup, const KhatRows& K,
+                           const SweepScratch<S>& W, const double* cpl = nullptr) {
+    constexpr int T = S::T, QS = S::QS;
+    const int tid = threadIdx.x;
+    const int32_t* list = K.list;
+    int buf = 0;
 #pragma unroll 1
     for (int g = N; g >= 0; --g) {
         const int o = block_offset(g), d = block_size(g);
+        uint32_t* qm = W.qmax(buf);
         // time solves of block g, per mode: the plain rows, the shifted rows,
         // and the coupled pairs (Biot: 6 stresses and p; u_f then u, v_f
         // then v, w_f then w)
         constexpr int NKIND = Sys::NPLAIN + Sys::NSHIFT + Sys::NPAIR;
         if constexpr (Sys::TWO_PHASE) {
-            Sys::template solve_block<T, NT, QS, Real>(bq, o, d, zin, zuf, cpl);
+            Sys::template solve_block<T, NT, QS>(bq, o, d, zsh, cpl, qm);
         } else {
-          for (int it = tid; it < NKIND * d; it += NT) {
-            const int kind = it / d, m = o + it % d;
-            if (kind < Sys::NPLAIN) {
-                solve_row<T>(bq + Sys::plain(kind) * QS + m * T, zin);
-            } else if (kind < Sys::NPLAIN + Sys::NSHIFT) {
-                solve_row<T>(bq + Sys::shifted(kind - Sys::NPLAIN) * QS + m * T, zuf);
-            } else {
-                const int i = kind - Sys::NPLAIN - Sys::NSHIFT;
-                Real* rf = bq + Sys::pair_src(i) * QS + m * T;
-                Real* rv = bq + Sys::pair_dst(i) * QS + m * T;
-                solve_row<T>(rf, zuf);
+            for (int it = tid; it < NKIND * d; it += NT) {
+                const int kind = it / d, m = o + it % d;
+                if (kind < Sys::NPLAIN) {
+                    const int q = Sys::plain(kind);
+                    solve_plain<T>(bq + q * QS + m * T, qm + q * T);
+                } else if (kind < Sys::NPLAIN + Sys::NSHIFT) {
+                    const int q = Sys::shifted(kind - Sys::NPLAIN);
+                    solve_row<T>(bq + q * QS + m * T, zsh, qm + q * T);
+                } else {
+                    const int i = kind - Sys::NPLAIN - Sys::NSHIFT, qf = Sys::pair_src(i), qv = Sys::pair_dst(i);
+                    double* rf = bq + qf * QS + m * T;
+                    double* rv = bq + qv * QS + m * T;
+                    solve_row<T>(rf, zsh, qm + qf * T);
 #pragma unroll
-                for (int u = 0; u < T; ++u) rv[u] = fma(gcoup, rf[u], rv[u]);
-                solve_row<T>(rv, zin);
+                    for (int u = 0; u < T; ++u) rv[u] = fma(gcoup, rf[u], rv[u]);
+                    solve_plain<T>(rv, qm + qv * T);
+                }
             }
-          }
         }
         __syncthreads();
         if (g == 0) break;
-        const int XS = bank_stride(d * T, T);
-#pragma unroll 1
-        for (int jb = 0; jb < 3; jb += JX) {
-            // X^j[p, ml, u] = sum_q A^{j*}_pq Q[q, o+ml, u]
-            for (int it = tid; it < d * T; it += NT) {
-                const int ml = it / T, u = it % T;
-                Real qv[NQ];
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) qv[q] = bq[q * QS + (o + ml) * T + u];
-#pragma unroll
-                for (int jj = 0; jj < JX; ++jj) {
-                    const Real* sj = star + (jb + jj) * STAR_NNZ;
-                    Real acc[NQ];
-#pragma unroll
-                    for (int p = 0; p < NQ; ++p) acc[p] = Real(0);
-#pragma unroll
-                    for (int n = 0; n < STAR_NNZ; ++n)
-                        acc[Sys::row(n)] = fma(sj[n], qv[Sys::col(n)], acc[Sys::row(n)]);
-                    Real* xj = X + jj * NQ * S::XSMAX + ml * T + u;
-#pragma unroll
-                    for (int p = 0; p < NQ; ++p) xj[p * XS] = acc[p];
-                }
-            }
-            __syncthreads();
-            // b[p, l, u] -= sum_j sum_m Khat^j[l, o+m] X^j[p, m, u], l < o;
-            // one warp per row l, each lane owns PUL (p, u) pairs
-            int xo[PUL];
-#pragma unroll
-            for (int k = 0; k < PUL; ++k) xo[k] = lp[k] * XS + lu[k];
-            auto row = [&](int l) {
-                Real acc[PUL];
-#pragma unroll
-                for (int k = 0; k < PUL; ++k) acc[k] = Real(0);
-#pragma unroll
-                for (int jj = 0; jj < JX; ++jj) {
-                    const int32_t* rp = K.row + K.row_base[g][jb + jj] + l;
-                    const int n0 = __ldg(rp), n1 = __ldg(rp + 1);
-                    const Real* xj = X + jj * NQ * S::XSMAX;
-                    int n = n0;
-                    for (; n + 1 < n1; n += 2) {
-                        const Real v0 = __ldg(K.val + n), v1 = __ldg(K.val + n + 1);
-                        const int m0 = __ldg(K.col + n) * T, m1 = __ldg(K.col + n + 1) * T;
-#pragma unroll
-                        for (int k = 0; k < PUL; ++k) {
-                            acc[k] = fma(v0, xj[xo[k] + m0], acc[k]);
-                            acc[k] = fma(v1, xj[xo[k] + m1], acc[k]);
-                        }
-                    }
-                    if (n < n1) {
-                        const Real v0 = __ldg(K.val + n);
-                        const int m0 = __ldg(K.col + n) * T;
-#pragma unroll
-                        for (int k = 0; k < PUL; ++k) acc[k] = fma(v0, xj[xo[k] + m0], acc[k]);
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < PUL; ++k)
-                    if (lane + 32 * k < PT) bq[lp[k] * QS + l * T + lu[k]] -= acc[k];
-            };
-            if (JX == 1 && K.lists) {
-                // this warp's rows of the block, dealt so that the warps' work is balanced
-                const int32_t* L = K.lists + K.list_base[g][jb];
-                const int i0 = __ldg(L + warp), i1 = __ldg(L + warp + 1);
-                for (int i = i0; i < i1; ++i) row(__ldg(L + NW + 1 + i));
-            } else {
-                for (int l = warp; l < o; l += NW) row(l);
-            }
-            __syncthreads();
-        }
+        khat_block<N, NT, Sys, S, -1>(bq, bq, g, star, K, list, W, qm, W.qmax(buf ^ 1));
+        buf ^= 1;
     }
+    for (int i = tid; i < 2 * S::PT; i += NT) W.w[i] = 0;
+    __syncthreads();
 }
 
 }  // namespace poro

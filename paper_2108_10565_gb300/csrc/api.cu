@@ -189,11 +189,8 @@ void free_reference(poro_ctx* c) {
     dfree(c->sub.m3_row);
     dfree(c->sub.m3_col);
     dfree(c->sub.m3_val);
-    dfree(c->dref.khat_val);
-    dfree(c->dref.khat_col);
-    dfree(c->dref.khat_row);
-    for (int w = 0; w < 3; ++w) dfree(c->dref.lists[w]);
-    dfree(c->dref.zinv);
+    dfree(c->dref.sweep_ent);
+    dfree(c->dref.sweep_list);
     dfree(c->dref.inv_d);
     dfree(c->dref.inv_d2);
 }
@@ -220,29 +217,6 @@ void ctx_set_error(poro_ctx* c, const std::string& msg) {
 extern "C" {
 
 const char* poro_last_error(const poro_ctx* ctx) { return ctx ? ctx->err.c_str() : g_err.c_str(); }
-
-// Rows dealt to `warps` lists, longest first, each to the least loaded list
-// (ties to the lower index); rows of zero cost are left out when `drop_free`.
-// Layout: [warps + 1] list starts, then the lists one after another.
-static std::vector<int32_t> deal_rows(const std::vector<int64_t>& cost, int warps, bool drop_free) {
-    std::vector<int> order;
-    for (int l = 0; l < (int)cost.size(); ++l)
-        if (!drop_free || cost[l] > 0) order.push_back(l);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
-    std::vector<std::vector<int32_t>> lists(warps);
-    std::vector<int64_t> load(warps, 0);
-    for (int l : order) {
-        int best = 0;
-        for (int k = 1; k < warps; ++k)
-            if (load[k] < load[best]) best = k;
-        load[best] += cost[l];
-        lists[best].push_back(l);
-    }
-    std::vector<int32_t> out(warps + 1, 0);
-    for (int k = 0; k < warps; ++k) out[k + 1] = out[k] + (int32_t)lists[k].size();
-    for (int k = 0; k < warps; ++k) out.insert(out.end(), lists[k].begin(), lists[k].end());
-    return out;
-}
 
 poro_status poro_create(int device, int degree_N, poro_precision precision, poro_ctx** out) {
     return poro_create_system(device, degree_N, precision, PORO_SYSTEM_BIOT, out);
@@ -288,51 +262,19 @@ poro_status poro_create_system(int device, int degree_N, poro_precision precisio
         delete c;
         return cuda_fail(nullptr, e, "poro_create: cudaStreamCreate");
     }
-    // concatenate the (g, j) CSR blocks of Khat
-    std::vector<double> val;
-    std::vector<int32_t> col, row;
     c->dref.N = degree_N;
-    for (int g = 1; g <= degree_N; ++g)
-        for (int j = 0; j < 3; ++j) {
-            const poro::KhatBlockCSR& C = c->ref.blocks[g * 3 + j];
-            c->dref.row_base[g][j] = (int32_t)row.size();
-            const int32_t base = (int32_t)val.size();
-            for (int32_t r : C.row_ptr) row.push_back(base + r);
-            val.insert(val.end(), C.val.begin(), C.val.end());
-            col.insert(col.end(), C.col.begin(), C.col.end());
-        }
-    // per block (g, j): its rows l < o_g dealt to 2, 4 and 8 warps by Khat
-    // entries (rows without entries in the block are left out)
-    std::vector<int32_t> blists[3];
-    for (int w = 0; w < 3; ++w)
-        for (int g = 1; g <= degree_N; ++g)
-            for (int j = 0; j < 3; ++j) {
-                const poro::KhatBlockCSR& C = c->ref.blocks[g * 3 + j];
-                std::vector<int64_t> cost(C.row_ptr.size() - 1);
-                for (size_t l = 0; l + 1 < C.row_ptr.size(); ++l) cost[l] = C.row_ptr[l + 1] - C.row_ptr[l];
-                c->dref.list_base[w][g][j] = (int32_t)blists[w].size();
-                const std::vector<int32_t> d = deal_rows(cost, 2 << w, true);
-                blists[w].insert(blists[w].end(), d.begin(), d.end());
-            }
-    if ((e = upload((void**)&c->dref.lists[0], blists[0].data(), blists[0].size() * sizeof(int32_t))) != cudaSuccess ||
-        (e = upload((void**)&c->dref.lists[1], blists[1].data(), blists[1].size() * sizeof(int32_t))) != cudaSuccess ||
-        (e = upload((void**)&c->dref.lists[2], blists[2].data(), blists[2].size() * sizeof(int32_t))) != cudaSuccess ||
-        (e = upload((void**)&c->dref.khat_val, val.data(), val.size() * sizeof(double))) != cudaSuccess ||
-        (e = upload((void**)&c->dref.khat_col, col.data(), col.size() * sizeof(int32_t))) != cudaSuccess ||
-        (e = upload((void**)&c->dref.khat_row, row.data(), row.size() * sizeof(int32_t))) != cudaSuccess ||
-        (e = upload((void**)&c->dref.zinv, c->ref.zinv.data(), c->ref.zinv.size() * sizeof(double))) !=
-            cudaSuccess) {
-        free_reference(c);
-        cudaStreamDestroy(c->stream);
-        delete c;
-        return e == cudaErrorMemoryAllocation ? fail(nullptr, PORO_ENOMEM, "poro_create: out of device memory")
-                                              : cuda_fail(nullptr, e, "poro_create: upload");
-    }
-    if (system == PORO_SYSTEM_BIOT) {
-        // integer Khat rows of Biot's predictor
-        std::vector<int32_t> ent, list;
+    {
+        // integer Khat rows: of the system's binary64 sweep (Biot: the sub-cell
+        // iteration's) and, for Biot, of its predictor kernel
+        const bool mx = system == PORO_SYSTEM_MAXWELL, ve = system == PORO_SYSTEM_VISCOELASTIC;
+        std::vector<int32_t> ent, list, sent, slist;
         std::vector<double> inv;
-        if (!poro::direct_tables(c->ref, ent, list, inv, err)) {
+        const int columns = mx ? poro::maxwell::columns(degree_N) : ve ? poro::visco::columns(degree_N)
+                                                                       : poro::subcell_columns(degree_N);
+        const int warps = (mx ? poro::maxwell::threads(degree_N) : ve ? poro::visco::threads(degree_N)
+                                                                      : poro::subcell_threads(degree_N)) / 32;
+        if (!poro::khat_tables(c->ref, columns, c->nq * c->T, warps, sent, slist, inv, err) ||
+            (system == PORO_SYSTEM_BIOT && !poro::direct_tables(c->ref, ent, list, inv, err))) {
             free_reference(c);
             cudaStreamDestroy(c->stream);
             delete c;
@@ -343,13 +285,17 @@ poro_status poro_create_system(int device, int degree_N, poro_precision precisio
             inv2.push_back((float)v);
             inv2.push_back((float)(v - (double)(float)v));
         }
-        if ((e = (cudaError_t)poro::upload_direct_tables(degree_N, ent, list)) != cudaSuccess ||
+        if ((system == PORO_SYSTEM_BIOT &&
+             (e = (cudaError_t)poro::upload_direct_tables(degree_N, ent, list)) != cudaSuccess) ||
             (e = upload((void**)&c->dref.inv_d, inv.data(), inv.size() * sizeof(double))) != cudaSuccess ||
-            (e = upload((void**)&c->dref.inv_d2, inv2.data(), inv2.size() * sizeof(float))) != cudaSuccess) {
+            (e = upload((void**)&c->dref.inv_d2, inv2.data(), inv2.size() * sizeof(float))) != cudaSuccess ||
+            (e = upload((void**)&c->dref.sweep_ent, sent.data(), sent.size() * sizeof(int32_t))) != cudaSuccess ||
+            (e = upload((void**)&c->dref.sweep_list, slist.data(), slist.size() * sizeof(int32_t))) != cudaSuccess) {
             free_reference(c);
             cudaStreamDestroy(c->stream);
             delete c;
-            return cuda_fail(nullptr, e, "poro_create: upload (integer rows)");
+            return e == cudaErrorMemoryAllocation ? fail(nullptr, PORO_ENOMEM, "poro_create: out of device memory")
+                                                  : cuda_fail(nullptr, e, "poro_create: upload (integer rows)");
         }
     }
     {

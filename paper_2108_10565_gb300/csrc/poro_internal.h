@@ -78,6 +78,9 @@ PORO_HD constexpr int star_col(int n) {
 }
 // per-element constants: star[3][12], (Z - e I)^{-1} [T][T], e, 0, dt, pad
 PORO_HD constexpr int elem_const_stride(int N) { return (3 * STAR_NNZ + (N + 1) * (N + 1) + 4 + 1) & ~1; }
+// CTA size of the predictor and the columns of X it holds
+constexpr int threads(int N) { return N >= 4 ? 128 : 64; }
+constexpr int columns(int N) { return 3 * block_size(N); }
 }  // namespace maxwell
 
 // Viscoelastic attenuation (Section "Other applications": upper-triangular
@@ -114,6 +117,10 @@ PORO_HD constexpr int sc_dt() { return 4 * NMECH; }
 PORO_HD constexpr int elem_const_stride(int N) {
     return (3 * STAR_NNZ + NMECH * (N + 1) * (N + 1) + NSC + 1) & ~1;
 }
+// CTA size of the predictor and the columns of X it holds (N = 5: block 5 in
+// three passes, so that two CTAs fit an SM; N = 6: blocks 6 and 5 in two)
+constexpr int threads(int N) { return N >= 4 ? 256 : N == 3 ? 128 : 64; }
+constexpr int columns(int N) { return N == 6 ? 42 : N == 5 ? 21 : 3 * block_size(N); }
 }  // namespace visco
 
 // Per-element constants, in doubles, in this order:
@@ -173,6 +180,8 @@ bool visco_element_constants(const ReferenceData& ref, const double* v12, const 
 // Per element, besides the mean-material constants (elem_const_stride
 // layout, from the mode-0 Jacobians): star_r[3][54] for the variation modes
 // r = 1..3 of the linearly interpolated Jacobians, then (e_r, g_r) of E*_r.
+constexpr int subcell_threads(int N) { return N >= 4 ? 256 : 128; }
+constexpr int subcell_columns(int N) { return N == 6 ? 30 : 3 * block_size(N); }
 PORO_HD constexpr int subcell_var_stride() { return (3 * 3 * STAR_NNZ + 6 + 1) & ~1; }
 // Mh3_r = M^{-1} int phi_k phi_r phi_l, r = 1..3, as CSR over all rows k:
 // row pointers [3][B + 1] absolute into col / val (device)
@@ -211,20 +220,13 @@ int face_permutation_index(const int p[3]);
 // ----- device side (kernels) -----
 struct DeviceReference {
     int N = 0;
-    double* khat_val = nullptr;   // concatenated CSR values of all (g, j) blocks
-    int32_t* khat_col = nullptr;  // concatenated CSR columns (m_local)
-    int32_t* khat_row = nullptr;  // concatenated row pointers, absolute into val/col
-    int32_t row_base[MAX_N + 1][3] = {};  // start of block (g, j)'s row pointers in khat_row
-    double* zinv = nullptr;       // [T][T]
-    // rows l < o_g of block (g, j) with Khat entries, dealt to 2, 4, 8 warps
-    // (index 0, 1, 2): at lists[w] + list_base[w][g][j], [warps + 1] list
-    // starts, then the lists
-    int32_t* lists[3] = {nullptr, nullptr, nullptr};
-    int32_t list_base[3][MAX_N + 1][3] = {};
-    // 1 / d_l of the integer Khat rows (khat_tables) [B], and the same as
-    // (hi, lo) binary32 words [B][2]
+    // the integer Khat rows (khat_tables): 1 / d_l [B] and the same as (hi, lo)
+    // binary32 words [B][2]; entries and lists of the binary64 sweep of the
+    // context's system (Biot: of the sub-cell iteration)
     double* inv_d = nullptr;
     float* inv_d2 = nullptr;
+    int32_t* sweep_ent = nullptr;
+    int32_t* sweep_list = nullptr;
 };
 
 // Extra device data of the mixed-precision path (the unrefined sweeps).
