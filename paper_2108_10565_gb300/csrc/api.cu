@@ -59,10 +59,8 @@ struct poro_ctx {
     std::vector<poro_material> h_mat;
     double dt = 0.0, t = 0.0;
     poro::CorrectorData cd;
-    int32_t *d_nb = nullptr, *d_tab = nullptr, *d_vrow = nullptr, *d_vcol = nullptr;
-    double *d_fc = nullptr, *d_fF = nullptr, *d_Pf = nullptr, *d_Pnb = nullptr, *d_vval = nullptr,
-           *d_minv = nullptr;
-    float *d_fF2 = nullptr, *d_Pf2 = nullptr, *d_Pnb2 = nullptr, *d_vval2 = nullptr;  // (hi, lo) pairs
+    int32_t *d_nb = nullptr, *d_tab = nullptr;
+    void *d_fvw = nullptr, *d_ftab = nullptr;
     struct Source {
         int64_t elem;
         double* d_coef;
@@ -122,18 +120,8 @@ void free_lu(poro_ctx* c);
 void free_mesh_device(poro_ctx* c) {
     dfree(c->d_nb);
     dfree(c->d_tab);
-    dfree(c->d_vrow);
-    dfree(c->d_vcol);
-    dfree(c->d_fc);
-    dfree(c->d_fF);
-    dfree(c->d_Pf);
-    dfree(c->d_Pnb);
-    dfree(c->d_vval);
-    dfree(c->d_minv);
-    dfree(c->d_fF2);
-    dfree(c->d_Pf2);
-    dfree(c->d_Pnb2);
-    dfree(c->d_vval2);
+    dfree(c->d_fvw);
+    dfree(c->d_ftab);
     for (auto& s : c->sources) dfree(s.d_coef);
     c->sources.clear();
     for (auto& p : c->d_cl_elems) dfree(p);
@@ -679,9 +667,9 @@ static poro_status dispatch_predict(poro_ctx* c, int64_t first, int64_t count, c
     } else if (c->system == PORO_SYSTEM_VISCOELASTIC) {
         rc = poro::launch_stp_fp64_visco(c->dref, count, q0, ec, qt, iout, st);
     } else if (c->prec == PORO_FP64) {
-        rc = poro::launch_stp_fp64(c->dref, nullptr, count, q0, ec, qt, iout, st, c->variant);
+        rc = poro::launch_stp_fp64(c->dref, nullptr, count, q0, ec, qt, iout, nullptr, st, c->variant);
     } else {
-        rc = poro::launch_stp_mixed(c->mref, c->refine, nullptr, count, q0, ec, qt, iout, st, c->variant);
+        rc = poro::launch_stp_mixed(c->mref, c->refine, nullptr, count, q0, ec, qt, iout, nullptr, st, c->variant);
     }
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "predict: kernel launch");
     return PORO_OK;
@@ -1052,7 +1040,10 @@ poro_status poro_set_clusters(poro_ctx* c, double cfl_c, int32_t max_clusters, d
     cudaMemsetAsync(c->d_q0, 0, (size_t)ne * NQ * B * sizeof(double), c->stream);
     // faces: neighbour face, vertex permutation, normal, area, flux solvers
     std::vector<int32_t> nb(4 * ne), tab(4 * ne);
-    std::vector<double> fc(4 * ne), fF((size_t)ne * 4 * 2 * NQ * NQ);
+    // the faces' factors V, c_f W as 8-byte words: binary64, or (hi, lo) binary32
+    // for the mixed-precision forms
+    const bool dw = c->prec != PORO_FP64;
+    std::vector<double> fvw((size_t)ne * 4 * poro::FACE_FACTORS);
     // per element (independent): run over host threads, each with its own
     // cache of flux solvers keyed by (materials, normal, kind)
     auto face_setup = [&](int64_t e, std::map<std::string, std::vector<double>>& cache, std::string& ferr) -> bool {
@@ -1081,7 +1072,7 @@ poro_status poro_set_clusters(poro_ctx* c, double cfl_c, int32_t max_clusters, d
             }
             if (dotv > 0)
                 for (int d = 0; d < 3; ++d) nr[d] = -nr[d];
-            fc[4 * e + f] = len / detJ[e];  // 2 |S_f| / |J| with |S_f| = len / 2
+            const double cf = len / detJ[e];  // 2 |S_f| / |J| with |S_f| = len / 2
             const int64_t r = c->h_nb[4 * e + f];
             nb[4 * e + f] = (int32_t)r;
             tab[4 * e + f] = -1;
@@ -1125,18 +1116,27 @@ poro_status poro_set_clusters(poro_ctx* c, double cfl_c, int32_t max_clusters, d
             key.append(reinterpret_cast<const char*>(nr), sizeof(nr));
             key.append(reinterpret_cast<const char*>(&kind), sizeof(kind));
             auto itc = cache.find(key);
-            double* dst = fF.data() + ((size_t)(4 * e + f) * 2) * NQ * NQ;
+            constexpr int HALF = poro::FACE_FACTORS / 2;
             if (itc == cache.end()) {
-                std::vector<double> F(2 * NQ * NQ);
+                std::vector<double> F(2 * HALF);
                 std::string err;
-                if (!poro::flux_solver(c->h_mat[e], r >= 0 ? &c->h_mat[r] : nullptr, nr, kind, F.data(),
-                                       F.data() + NQ * NQ, err)) {
+                if (!poro::flux_factors(c->h_mat[e], r >= 0 ? &c->h_mat[r] : nullptr, nr, kind, F.data(),
+                                        F.data() + HALF, err)) {
                     ferr = "flux at element " + std::to_string(e) + ": " + err;
                     return false;
                 }
                 itc = cache.emplace(key, std::move(F)).first;
             }
-            std::memcpy(dst, itc->second.data(), sizeof(double) * 2 * NQ * NQ);
+            double* dst = fvw.data() + (size_t)(4 * e + f) * poro::FACE_FACTORS;
+            for (int i = 0; i < 2 * HALF; ++i) {
+                const double x = i < HALF ? itc->second[i] : cf * itc->second[i];
+                if (dw) {
+                    const float h = (float)x, hl[2] = {h, (float)(x - (double)h)};
+                    std::memcpy(dst + i, hl, sizeof hl);
+                } else {
+                    dst[i] = x;
+                }
+            }
         }
         return true;
     };
@@ -1168,60 +1168,13 @@ poro_status poro_set_clusters(poro_ctx* c, double cfl_c, int32_t max_clusters, d
             return fail(c, msg.rfind("flux", 0) == 0 ? PORO_ENUMERIC : PORO_EINVAL, "poro_set_clusters: " + msg);
         }
     }
-    // volume CSR: Kv^j_kl = M_ll Khat^j_lk / M_kk
-    std::vector<int32_t> vrow, vcol;
-    std::vector<double> vval, minv(B);
-    for (int j = 0; j < 3; ++j) {
-        for (int k = 0; k < B; ++k) {
-            vrow.push_back((int32_t)vcol.size());
-            for (int l = 0; l < B; ++l) {
-                const double kh = c->ref.khat[((size_t)j * B + l) * B + k];
-                if (kh != 0.0) {
-                    vcol.push_back(l);
-                    vval.push_back(c->ref.mass_diag[l] * kh / c->ref.mass_diag[k]);
-                }
-            }
-        }
-        vrow.push_back((int32_t)vcol.size());
-    }
-    // absolute row offsets per direction: rows of direction j start at j*(B+1)
-    for (int k = 0; k < B; ++k) minv[k] = 1.0 / c->ref.mass_diag[k];
-    // face traces: Floc^f = Pf^T Pf, Fnb^{f,h,s} = Pf^T Pnb
-    std::vector<double> Pf, Pnb;
-    poro::face_traces(N, Pf, Pnb);
-    // the mixed-precision form corrects in double-binary32: (hi, lo) copies
-    const bool dw = c->prec != PORO_FP64;
-    auto split = [](const std::vector<double>& x) {
-        std::vector<float> o(2 * x.size());
-        for (size_t i = 0; i < x.size(); ++i) {
-            const float h = (float)x[i];
-            o[2 * i] = h;
-            o[2 * i + 1] = (float)(x[i] - (double)h);
-        }
-        return o;
-    };
+    std::vector<int32_t> ftab;
+    poro::face_tables(N, c->ref.mass_diag, dw, ftab);
     cudaError_t er = cudaSuccess;
-    if (dw) {
-        const std::vector<float> f2 = split(fF), l2 = split(Pf), n2 = split(Pnb), v2 = split(vval);
-        if ((er = upload((void**)&c->d_fF2, f2.data(), f2.size() * sizeof(float))) != cudaSuccess ||
-            (er = upload((void**)&c->d_Pf2, l2.data(), l2.size() * sizeof(float))) != cudaSuccess ||
-            (er = upload((void**)&c->d_Pnb2, n2.data(), n2.size() * sizeof(float))) != cudaSuccess ||
-            (er = upload((void**)&c->d_vval2, v2.data(), v2.size() * sizeof(float))) != cudaSuccess) {
-            free_population(c);
-            return er == cudaErrorMemoryAllocation ? fail(c, PORO_ENOMEM, "poro_set_clusters: out of device memory")
-                                                   : cuda_fail(c, er, "poro_set_clusters");
-        }
-    }
     if ((er = upload((void**)&c->d_nb, nb.data(), nb.size() * sizeof(int32_t))) != cudaSuccess ||
         (er = upload((void**)&c->d_tab, tab.data(), tab.size() * sizeof(int32_t))) != cudaSuccess ||
-        (er = upload((void**)&c->d_fc, fc.data(), fc.size() * sizeof(double))) != cudaSuccess ||
-        (!dw && (er = upload((void**)&c->d_fF, fF.data(), fF.size() * sizeof(double))) != cudaSuccess) ||
-        (er = upload((void**)&c->d_vrow, vrow.data(), vrow.size() * sizeof(int32_t))) != cudaSuccess ||
-        (er = upload((void**)&c->d_vcol, vcol.data(), vcol.size() * sizeof(int32_t))) != cudaSuccess ||
-        (er = upload((void**)&c->d_vval, vval.data(), vval.size() * sizeof(double))) != cudaSuccess ||
-        (er = upload((void**)&c->d_minv, minv.data(), minv.size() * sizeof(double))) != cudaSuccess ||
-        (er = upload((void**)&c->d_Pf, Pf.data(), Pf.size() * sizeof(double))) != cudaSuccess ||
-        (er = upload((void**)&c->d_Pnb, Pnb.data(), Pnb.size() * sizeof(double))) != cudaSuccess) {
+        (er = upload(&c->d_fvw, fvw.data(), fvw.size() * sizeof(double))) != cudaSuccess ||
+        (er = upload(&c->d_ftab, ftab.data(), ftab.size() * sizeof(int32_t))) != cudaSuccess) {
         free_population(c);
         return er == cudaErrorMemoryAllocation ? fail(c, PORO_ENOMEM, "poro_set_clusters: out of device memory")
                                                : cuda_fail(c, er, "poro_set_clusters");
@@ -1233,19 +1186,12 @@ poro_status poro_set_clusters(poro_ctx* c, double cfl_c, int32_t max_clusters, d
     d.q = c->d_q0;
     d.nb = c->d_nb;
     d.tab = c->d_tab;
-    d.fc = c->d_fc;
-    d.fF = c->d_fF;
-    d.Pf = c->d_Pf;
-    d.Pnb = c->d_Pnb;
-    d.vrow = c->d_vrow;
-    d.vcol = c->d_vcol;
-    d.vval = c->d_vval;
-    d.minv = c->d_minv;
     d.dw = dw;
-    d.fF2 = c->d_fF2;
-    d.Pf2 = c->d_Pf2;
-    d.Pnb2 = c->d_Pnb2;
-    d.vval2 = c->d_vval2;
+    d.fvw = c->d_fvw;
+    d.ftab = reinterpret_cast<const int4*>(c->d_ftab);
+    d.krow = c->lref.krow;
+    d.kcol = c->lref.kcol;
+    d.kval = c->lref.kval;
     // clusters: element lists, buffer slots of (element, larger neighbour level)
     c->C = C;
     c->cl_elems.assign(C, std::vector<int32_t>());
@@ -1369,6 +1315,10 @@ static int mark(std::vector<ClusterEvent>* prof, int cl, bool begin, cudaStream_
     return (int)cudaEventRecord(prof->back().b, st);
 }
 
+// whether a time step's predictor writes Q~(1) over Q, so that the corrector
+// adds the faces alone (the unrefined binary32 sweep does not)
+static bool step_in_place(const poro_ctx* c) { return c->prec == PORO_FP64 || c->refine > 0; }
+
 enum : unsigned { TICK_PREDICT = 1, TICK_BUFFERS = 2, TICK_CORRECT = 4, TICK_SOURCES = 8, TICK_ALL = 15 };
 
 static int enqueue_tick(poro_ctx* c, int64_t k, unsigned what, const double* d_rp, double* d_seis, int64_t cap,
@@ -1377,6 +1327,7 @@ static int enqueue_tick(poro_ctx* c, int64_t k, unsigned what, const double* d_r
     const int C = c->C;
     const int nrec = (int)c->rec_elem.size();
     const bool want_qt = C > 1;
+    const bool in_place = step_in_place(c);
     int rc = 0;
     for (int cl = 0; cl < C && rc == 0; ++cl) {
         if (k % ((int64_t)1 << cl) || c->cl_elems[cl].empty()) continue;
@@ -1385,10 +1336,11 @@ static int enqueue_tick(poro_ctx* c, int64_t k, unsigned what, const double* d_r
         const int64_t cnt = (int64_t)c->cl_elems[cl].size();
         if (predict && c->prec == PORO_FP64)
             rc = poro::launch_stp_fp64(c->dref, el, cnt, c->d_q0, c->d_econst, want_qt ? c->d_qt : nullptr,
-                                       c->d_iout, st, c->variant);
+                                       c->d_iout, c->d_q0, st, c->variant);
         else if (predict)
             rc = poro::launch_stp_mixed(c->mref, c->refine, el, cnt, c->d_q0, c->d_econst,
-                                        want_qt ? c->d_qt : nullptr, c->d_iout, st, c->variant);
+                                        want_qt ? c->d_qt : nullptr, c->d_iout, in_place ? c->d_q0 : nullptr, st,
+                                        c->variant);
         // (a cluster whose elements buffer for no larger neighbour has nothing to add)
         if (rc == 0 && C > 1 && (what & TICK_BUFFERS) && c->cl_has_slot[cl])
             rc = poro::launch_lts_buffers(c->N, C, el, cnt, c->d_slot, c->d_iout, c->d_buf, k, st);
@@ -1402,8 +1354,8 @@ static int enqueue_tick(poro_ctx* c, int64_t k, unsigned what, const double* d_r
             poro::CorrectorData d = c->cd;
             d.tick = k;
             if (what & TICK_CORRECT)
-                rc = poro::launch_corrector(d, C > 1 ? c->d_cl_elems[cl] : nullptr, (int64_t)c->cl_elems[cl].size(),
-                                            st);
+                rc = poro::launch_corrector(d, !in_place, C > 1 ? c->d_cl_elems[cl] : nullptr,
+                                            (int64_t)c->cl_elems[cl].size(), st);
             if (!(what & TICK_SOURCES)) {
                 if (rc == 0) rc = mark(prof, cl, false, st);
                 continue;
@@ -1585,17 +1537,17 @@ static int enqueue_group_cycle(RunGroup* g) {
             const int32_t* el = g->d_items + g->k_off[k];
             const int32_t* ir = g->d_item_run + g->k_off[k];
             if (lead->prec == PORO_FP64)
-                rc = launch_stp_fp64(lead->dref, el, cnt, nullptr, nullptr, nullptr, nullptr, g->stream, lead->variant,
-                                     g->d_runs, ir);
+                rc = launch_stp_fp64(lead->dref, el, cnt, nullptr, nullptr, nullptr, nullptr, nullptr, g->stream,
+                                     lead->variant, g->d_runs, ir);
             else
-                rc = launch_stp_mixed(lead->mref, lead->refine, el, cnt, nullptr, nullptr, nullptr, nullptr, g->stream,
-                                      lead->variant, g->d_runs, ir);
+                rc = launch_stp_mixed(lead->mref, lead->refine, el, cnt, nullptr, nullptr, nullptr, nullptr, nullptr,
+                                      g->stream, lead->variant, g->d_runs, ir);
         }
         for (poro_ctx* c : g->runs)
             if (rc == 0) rc = enqueue_tick(c, k, TICK_BUFFERS, c->d_rp, c->d_seis, c->seis_cap, c->d_cnt, g->stream);
         const int64_t cc = g->ck_cnt[k];
         if (rc == 0 && cc > 0)
-            rc = launch_corrector(lead->cd, g->d_citems + g->ck_off[k], cc, g->stream,
+            rc = launch_corrector(lead->cd, !step_in_place(lead), g->d_citems + g->ck_off[k], cc, g->stream,
                                   g->d_cdata + k * (int64_t)g->runs.size(), g->d_citem_run + g->ck_off[k]);
         // all runs' sources of the tick, then all their receivers (one launch each)
         if (rc == 0) rc = launch_tick_sources(lead->N, g->d_src + g->src_off[k], g->src_cnt[k], g->stream);
@@ -1654,7 +1606,8 @@ RunGroup* group_create(poro_ctx* const* runs, int n, std::string& err) {
     std::vector<RunPtrs> rp(n);
     for (int i = 0; i < n; ++i) {
         poro_ctx* c = runs[i];
-        rp[i] = RunPtrs{c->d_q0, c->d_econst, g->C > 1 ? c->d_qt : nullptr, c->d_iout};
+        rp[i] = RunPtrs{c->d_q0, c->d_econst, g->C > 1 ? c->d_qt : nullptr, c->d_iout,
+                        step_in_place(c) ? c->d_q0 : nullptr};
     }
     std::vector<int32_t> items, item_run;
     for (int64_t k = 0; k < g->cycle; ++k) {
@@ -1878,7 +1831,7 @@ poro_status poro_correct(poro_ctx* c, int32_t cluster) {
     if (!c->ready || !c->have_pred) return fail(c, PORO_ESTATE, "poro_correct: mesh set-up and a predictor first");
     if (cluster != -1 && cluster != 0) return fail(c, PORO_EINVAL, "poro_correct: no such cluster");
     cudaSetDevice(c->device);
-    int rc = poro::launch_corrector(c->cd, nullptr, c->n_elem, c->stream);
+    int rc = poro::launch_corrector(c->cd, true, nullptr, c->n_elem, c->stream);
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "poro_correct");
     return PORO_OK;
 }

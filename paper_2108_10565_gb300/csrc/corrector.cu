@@ -1,195 +1,279 @@
-// Corrector of the ADER-DG scheme (Eq. semi_discrete integrated over one
-// time step, Section "Temporal discretisation with ADER"), point source and
-// receivers, binary64.
+// Corrector of the ADER-DG scheme (Eq. semi_discrete integrated over one time
+// step, Section "Temporal discretisation with ADER"), point source and
+// receivers, in binary64 or (mixed-precision contexts) double-binary32.
 //
-// For element e with time-integrated predictor I (13 x B):
-//   dQ_pk = sum_j sum_l Kv^j_kl (A^j I)_pl              volume, Kv^j = M^{-1} K^{jT}
-//         + (E I)_pk                                    Darcy source term
-//         - sum_f c_f / M_kk [ sum_l Floc^f_kl (F^- I^e)_pl
-//                            + sum_l Fnb^{f,h,s}_kl (F^+ I^nb)_pl ]   Godunov flux
-// with A^j = A^{j*} / dt and E = E* / dt from the element constants,
-// c_f = 2 |S_f| / |J|, Floc^f / Fnb the face mass matrices of the local face
-// and of the (neighbour face h, vertex permutation s) pair.  One CTA per
-// element; the DOFs are updated in place (neighbours read I only).
+// With I the time-integrated predictor, A_n the normal Jacobian and the Godunov
+// flux F^- q_L + F^+ q_R of the paper's weak form, integration by parts gives
+//   dQ = E I - sum_j Khat^j A^j I                          volume and source
+//      + M^{-1} sum_f c_f Pf^T [ (A_n - F^-) tL - F^+ tR ]    faces
+// with c_f = 2 |S_f| / |J| and tL, tR the traces of both sides (Floc^f = Pf^T Pf).
+// The volume line is the predictor's own equation tested with 1, whose left
+// side is Q~(1) - Q: a time step's predictor therefore writes Q~(1) over Q and
+// the corrector adds the faces alone.  (After poro_correct's separate predictor,
+// and for the unrefined binary32 predictor, volume_kernel adds the line.)
+//
+// Only the 4 waves that enter the element enter the face term: A_n - F^- and
+// (interior) F^+ are the same matrix W V, W 13 x 4, V 4 x 13.  So each side is
+// reduced to 4 rows V I before its trace.  The traces use the Dubiner basis of
+// the triangle on each face with its vertices in increasing order, in which Pf
+// is sparse (N = 6: 3,060 of 9,408 entries); the neighbour's trace is taken on
+// its own face and then turned by the vertex permutation, block-diagonal by
+// degree.  Per element at N = 5 this is 55 thousand multiply-adds, against 246
+// thousand with dense traces, two 13 x 13 flux matrices and the volume term.
+//
+// One CTA per element; neighbours are read only through I (or, for another
+// cluster, the buffered sub-step sums or the predictor), so Q is updated in
+// place.  What bounds it: binary64, the FP64 pipe; double-binary32, issue slots.
 #include <cuda_runtime.h>
 
+#include "pair_device.cuh"
 #include "poro_internal.h"
 
 namespace poro {
 namespace {
 
-constexpr int CNT = 128;
+// a table entry: value (binary64, or (hi, lo) binary32) and column
+template <class P>
+__device__ __forceinline__ void load_entry(const int4* at, typename P::R& v, int& col);
+template <>
+__device__ __forceinline__ void load_entry<Bin64Base>(const int4* at, double& v, int& col) {
+    const int4 e = __ldg(at);
+    v = __hiloint2double(e.y, e.x);
+    col = e.z;
+}
+template <>
+__device__ __forceinline__ void load_entry<Bin32x2Base>(const int4* at, float2& v, int& col) {
+    const int4 e = __ldg(at);
+    v = make_float2(__int_as_float(e.x), __int_as_float(e.y));
+    col = e.z;
+}
 
-// the neighbour's trace source, integrated over this element's interval:
-// its own I (same cluster), the buffered sum of its sub-steps (smaller
-// neighbour) or its predictor integrated over the sub-interval (larger
-// neighbour); written to In[13][B]
 template <int N>
-__device__ void neighbour_integral(const CorrectorData& D, int64_t e, int64_t nbr, double* In, double* wts) {
+struct FaceShape {
+    // a thread takes whole columns of the first step (8 B of them)
+    static constexpr int NT = N == 1 ? 32 : N == 2 ? 96 : N <= 4 ? 160 : 224, NW = NT / 32;
+    static constexpr int B = n_modes(N), DF = face_modes(N), T = N + 1, TG = (DF + 7) / 8, BG = (B + 7) / 8;
+    // shared layout in 8-byte words: the factors V [13][4], W [13][4] of the
+    // four faces; Y [2 sides][4 faces][B][4]; traces [2][4][DF][4]
+    static constexpr int OFF_Y = 4 * FACE_FACTORS, OFF_T = OFF_Y + 2 * 4 * B * 4, END = OFF_T + 2 * 4 * DF * 4;
+    static constexpr int SMEM_BYTES = 8 * END;
+};
+
+// the neighbour across one face: where its time integral over this element's
+// interval comes from
+struct FaceSide {
+    const double* src;  // I or the buffered sum [13][B] (mode 1), or the predictor [13][B][T] (mode 2)
+    int mode;           // 0: boundary
+    int face, perm;     // its local face, the vertex permutation
+    double w[MAX_N + 1];  // mode 2: dt_r int_a^b chi_s
+};
+
+template <int N>
+__device__ void face_side(const CorrectorData& D, int64_t e, int f, FaceSide& S) {
     constexpr int B = n_modes(N), QB = NQ * B, T = N + 1;
+    const int64_t nbr = D.nb[e * 4 + f];
+    S.mode = 0;
+    if (nbr < 0) return;
+    const int tab = D.tab[e * 4 + f];
+    S.face = (tab / 6) & 3;
+    S.perm = tab % 6;
     const int c = D.cl ? D.cl[e] : 0, cr = D.cl ? D.cl[nbr] : 0;
+    S.mode = 1;
     if (cr == c) {
-        for (int i = threadIdx.x; i < QB; i += CNT) In[i] = D.iout[nbr * QB + i];
+        S.src = D.iout + nbr * QB;
     } else if (cr < c) {
-        const double* b = D.buf + (int64_t)D.slot[nbr * D.C + c] * QB;
-        for (int i = threadIdx.x; i < QB; i += CNT) In[i] = b[i];
+        S.src = D.buf + (int64_t)D.slot[nbr * D.C + c] * QB;
     } else {
         // larger neighbour: dt_r sum_s Qt_s int_a^b chi_s over the sub-interval
-        if (threadIdx.x == 0) {
-            const int64_t ks = D.tick + 1 - ((int64_t)1 << c);
-            const int64_t m = (ks >> cr) << cr;
-            const double a = (double)(ks - m) / (double)((int64_t)1 << cr);
-            const double bb = (double)(D.tick + 1 - m) / (double)((int64_t)1 << cr);
-            // int_a^b P_s(2 tau - 1) dtau = (1/2) [ (P_{s+1} - P_{s-1}) / (2s+1) ]_{2a-1}^{2b-1}
-            double P0[MAX_N + 3], P1[MAX_N + 3];
-            const double x0 = 2 * a - 1, x1 = 2 * bb - 1;
-            P0[0] = 1;
-            P0[1] = x0;
-            P1[0] = 1;
-            P1[1] = x1;
-            for (int n = 1; n <= T; ++n) {
-                P0[n + 1] = ((2 * n + 1) * x0 * P0[n] - n * P0[n - 1]) / (n + 1);
-                P1[n + 1] = ((2 * n + 1) * x1 * P1[n] - n * P1[n - 1]) / (n + 1);
-            }
-            wts[0] = 0.5 * (x1 - x0);
-            for (int sidx = 1; sidx < T; ++sidx)
-                wts[sidx] = 0.5 * ((P1[sidx + 1] - P1[sidx - 1]) - (P0[sidx + 1] - P0[sidx - 1])) / (2 * sidx + 1);
-        }
-        __syncthreads();
-        const int stride = elem_const_stride(N);
-        const double dtr = D.econst[nbr * stride + ec_scalars(N) + 2];
-        const double* qr = D.qt + nbr * (int64_t)QB * T;
-        for (int i = threadIdx.x; i < QB; i += CNT) {
-            double acc = 0.0;
-            for (int sidx = 0; sidx < T; ++sidx) acc = fma(qr[i * T + sidx], wts[sidx], acc);
-            In[i] = dtr * acc;
+        S.mode = 2;
+        S.src = D.qt + nbr * (int64_t)(QB * T);
+        const double dtr = D.econst[nbr * elem_const_stride(N) + ec_scalars(N) + 2];
+        const int64_t ks = D.tick + 1 - ((int64_t)1 << c);
+        const int64_t m = (ks >> cr) << cr;
+        const double h = __hiloint2double((1023 - cr) << 20, 0);  // 2^-cr
+        const double a = (double)(ks - m) * h, b = (double)(D.tick + 1 - m) * h;
+        // int_a^b P_s(2 tau - 1) dtau = (1/2) [ (P_{s+1} - P_{s-1}) / (2s+1) ]_{2a-1}^{2b-1}
+        const double x0 = 2 * a - 1, x1 = 2 * b - 1;
+        double p0 = 1, p1 = 1, q0 = x0, q1 = x1;  // P_{s-1}, P_s at both ends
+        S.w[0] = dtr * (0.5 * (x1 - x0));
+#pragma unroll
+        for (int s = 1; s < T; ++s) {
+            const double r0 = ((2 * s + 1) * x0 * q0 - s * p0) * (1.0 / (s + 1)),
+                         r1 = ((2 * s + 1) * x1 * q1 - s * p1) * (1.0 / (s + 1));
+            S.w[s] = dtr * (((r1 - p1) - (r0 - p0)) * (0.5 / (2 * s + 1)));
+            p0 = q0;
+            p1 = q1;
+            q0 = r0;
+            q1 = r1;
         }
     }
 }
 
-// Face terms through face traces.  Floc^f = Pf^T Pf and Fnb^{f,h,s} = Pf^T Pnb
-// with Pf, Pnb of df = (N+1)(N+2)/2 rows (traces in a basis orthonormal on
-// the reference triangle), so per face
-//   u_f = c_f (F^- (I Pf^T) + F^+ (I^nb Pnb^T))          [13 x df]
-//   dQ -= M^{-1} sum_f Pf^T u_f                          (one pass over all faces)
-template <int N, bool BATCH>
-__global__ void __launch_bounds__(CNT) corrector_kernel(const CorrectorData D1, const int32_t* elems, int64_t count,
-                                                        const CorrectorData* runs, const int32_t* item_run) {
-    constexpr int B = n_modes(N), QB = NQ * B, DF = (N + 1) * (N + 2) / 2, FQ = NQ * DF;
-    constexpr int stride = elem_const_stride(N);
-    extern __shared__ double sm[];
-    double* I = sm;             // [13][B]
-    double* Y = I + QB;         // [13][B]
-    double* dQ = Y + QB;        // [13][B]
-    double* In = dQ + QB;       // [13][B]
-    double* tL = In + QB;       // [4][13][DF] traces of I
-    double* tR = tL + 4 * FQ;   // [13][DF] neighbour trace
-    double* U = tR + FQ;        // [4][13][DF] flux values
-    __shared__ double F[2 * NQ * NQ];
-    __shared__ double wts[MAX_N + 1];
-    const int tid = threadIdx.x;
-    for (int64_t it = blockIdx.x; it < count; it += gridDim.x) {
-        // one run's data (D1), or item it's run of a batched launch over
-        // several runs (their tables in global memory)
-        const CorrectorData& D = BATCH ? runs[item_run[it]] : D1;
-        const int64_t e = elems ? elems[it] : it;
-        const double* ec = D.econst + e * stride;
-        const double dt = ec[ec_scalars(N) + 2];
-        const double ev = ec[ec_scalars(N)] / dt, gv = ec[ec_scalars(N) + 1] / dt;
-        for (int i = tid; i < QB; i += CNT) {
-            I[i] = D.iout[e * QB + i];
-            dQ[i] = 0.0;
-        }
-        __syncthreads();
-        // volume: X^j = A^j I (54-entry star pattern), dQ += Kv^j X^j
-        for (int j = 0; j < 3; ++j) {
-            const double* sj = ec + j * STAR_NNZ;
-            for (int l = tid; l < B; l += CNT) {
-                double qv[NQ], acc[NQ];
+template <int N, class P, bool BATCH>
+__global__ void __launch_bounds__(FaceShape<N>::NT)
+    face_kernel(const CorrectorData D1, const int32_t* elems, const CorrectorData* runs, const int32_t* item_run) {
+    using S = FaceShape<N>;
+    using R = typename P::R;
+    constexpr int B = S::B, DF = S::DF, T = S::T, NT = S::NT, NW = S::NW;
+    extern __shared__ __align__(16) double smf[];
+    R* VW = reinterpret_cast<R*>(smf);
+    R* Y = reinterpret_cast<R*>(smf) + S::OFF_Y;
+    R* tr = reinterpret_cast<R*>(smf) + S::OFF_T;
+    __shared__ FaceSide side[4];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // one run's data (D1), or the item's run of a batched launch over several
+    // runs (their tables in global memory)
+    const CorrectorData& D = BATCH ? runs[item_run[blockIdx.x]] : D1;
+    const int64_t e = elems ? elems[blockIdx.x] : (int64_t)blockIdx.x;
+    if (tid < 4) face_side<N>(D, e, tid, side[tid]);
+    {
+        const R* g = reinterpret_cast<const R*>(D.fvw) + e * (int64_t)(4 * FACE_FACTORS);
+        for (int i = tid; i < 4 * FACE_FACTORS; i += NT) VW[i] = g[i];
+    }
+    __syncthreads();
+    // Y[k][c] = sum_p V[p][c] I[p][k] of both sides of every face
+    for (int it = tid; it < 8 * B; it += NT) {
+        const int sf = it / B, k = it - sf * B, f = sf & 3;
+        const FaceSide& F = side[f];
+        if (sf >= 4 && F.mode == 0) continue;
+        const double* I = sf < 4 ? D.iout + e * (int64_t)(NQ * B) : F.src;
+        R v[NQ];
+        if (sf < 4 || F.mode == 1) {
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    qv[q] = I[q * B + l];
-                    acc[q] = 0.0;
-                }
+            for (int p = 0; p < NQ; ++p) v[p] = P::of(__ldg(I + p * B + k));
+        } else {
 #pragma unroll
-                for (int n = 0; n < STAR_NNZ; ++n) acc[star_row(n)] = fma(sj[n], qv[star_col(n)], acc[star_row(n)]);
+            for (int p = 0; p < NQ; ++p) {
+                double a = 0.0;
 #pragma unroll
-                for (int p = 0; p < NQ; ++p) Y[p * B + l] = acc[p] / dt;
+                for (int s = 0; s < T; ++s) a = ::fma(__ldg(I + (p * B + k) * T + s), F.w[s], a);
+                v[p] = P::of(a);
             }
-            __syncthreads();
-            const int32_t* vr = D.vrow + j * (B + 1);
-            for (int i = tid; i < QB; i += CNT) {
-                const int p = i / B, k = i - (i / B) * B;
-                double acc = 0.0;
-                for (int n = vr[k]; n < vr[k + 1]; ++n) acc = fma(D.vval[n], Y[p * B + D.vcol[n]], acc);
-                dQ[i] += acc;
-            }
-            __syncthreads();
         }
-        // Darcy source term E I: u rows from u_f, u_f rows from u_f
-        for (int i = tid; i < 6 * B; i += CNT) {
-            const int r = i / B, k = i - (i / B) * B;
-            if (r < 3) dQ[(QU + r) * B + k] += gv * I[(QUF + r) * B + k];
-            else dQ[(QUF + r - 3) * B + k] += ev * I[(QUF + r - 3) * B + k];
+        const R* V = VW + f * FACE_FACTORS;
+        R a[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) a[c] = P::mul(V[c], v[0]);
+#pragma unroll
+        for (int p = 1; p < NQ; ++p)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) a[c] = P::fma(V[4 * p + c], v[p], a[c]);
+        R* y = Y + (sf * B + k) * 4;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) y[c] = a[c];
+    }
+    __syncthreads();
+    // traces of the 4 rows: a warp takes 8 rows of a face (ordered by length),
+    // lanes (row, c)
+    const int rs = lane >> 2, c = lane & 3;
+    for (int t = warp; t < 8 * S::TG; t += NW) {
+        const int sf = t / S::TG, f = sf & 3;  // sides 0: own, 1: the neighbour's
+        if (sf >= 4 && side[f].mode == 0) continue;
+        const int ft = sf < 4 ? f : side[f].face;
+        const int4 row = __ldg(D.ftab + face_trace_slots(N) + (ft * S::TG + t % S::TG) * 8 + rs);
+        const R* y = Y + sf * B * 4 + c;
+        R a = P::zero();
+        for (int n = row.x; n < row.x + row.y; ++n) {
+            R v;
+            int k;
+            load_entry<P>(D.ftab + n, v, k);
+            a = P::fma(v, y[k * 4], a);
         }
-        // traces of I on the four faces: tL[f][p][a] = sum_k Pf[f][a][k] I[p][k]
-        for (int t = tid; t < 4 * FQ; t += CNT) {
-            const int f = t / FQ, r = t - f * FQ, p = r / DF, a = r - p * DF;
-            const double* row = D.Pf + ((size_t)f * DF + a) * B;
-            double acc = 0.0;
-#pragma unroll 4
-            for (int k = 0; k < B; ++k) acc = fma(__ldg(row + k), I[p * B + k], acc);
-            tL[t] = acc;
+        if (row.z >= 0) tr[(sf * DF + row.z) * 4 + c] = a;
+    }
+    __syncthreads();
+    // difference of the sides, the neighbour's turned by its permutation
+    for (int it = tid; it < 16 * DF; it += NT) {
+        const int f = it / (4 * DF), ac = it - f * (4 * DF);
+        if (side[f].mode == 0) continue;
+        const int4 row = __ldg(D.ftab + face_turn_slots(N) + side[f].perm * DF + (ac >> 2));
+        const R* t = tr + (4 + f) * DF * 4 + (ac & 3);
+        R a = P::zero();
+        for (int n = row.x; n < row.x + row.y; ++n) {
+            R v;
+            int k;
+            load_entry<P>(D.ftab + n, v, k);
+            a = P::fma(v, t[k * 4], a);
         }
-        __syncthreads();
+        R* o = tr + f * DF * 4 + ac;
+        *o = P::sub(*o, a);
+    }
+    __syncthreads();
+    // M^{-1} Pf^T of the 4 rows, into the own side of Y
+    for (int t = warp; t < 4 * S::BG; t += NW) {
+        const int f = t / S::BG;
+        const int4 row = __ldg(D.ftab + face_back_slots(N) + t * 8 + rs);
+        const R* x = tr + f * DF * 4 + c;
+        R a = P::zero();
+        for (int n = row.x; n < row.x + row.y; ++n) {
+            R v;
+            int k;
+            load_entry<P>(D.ftab + n, v, k);
+            a = P::fma(v, x[k * 4], a);
+        }
+        if (row.z >= 0) Y[(f * B + row.z) * 4 + c] = a;
+    }
+    __syncthreads();
+    // Q[p][k] += sum_f sum_c (c_f W_f)[p][c] Y[f][k][c]
+    double* q = D.q + e * (int64_t)(NQ * B);
+    for (int it = tid; it < NQ * B; it += NT) {
+        const int p = it / B, k = it - p * B;
+        const double q0 = q[it];
+        R a[2] = {P::zero(), P::zero()};
+#pragma unroll
         for (int f = 0; f < 4; ++f) {
-            const int64_t nbr = D.nb[e * 4 + f];
-            const double cf = D.fc[e * 4 + f];
-            const double* Fm = D.fF + ((e * 4 + f) * 2) * NQ * NQ;
-            const bool inner = nbr >= 0;
-            for (int i = tid; i < (inner ? 2 : 1) * NQ * NQ; i += CNT) F[i] = Fm[i];
-            if (inner) {
-                neighbour_integral<N>(D, e, nbr, In, wts);
-                __syncthreads();
-                const double* Pn = D.Pnb + (size_t)D.tab[e * 4 + f] * DF * B;
-                for (int t = tid; t < FQ; t += CNT) {
-                    const int p = t / DF, a = t - p * DF;
-                    const double* row = Pn + (size_t)a * B;
-                    double acc = 0.0;
-#pragma unroll 4
-                    for (int k = 0; k < B; ++k) acc = fma(__ldg(row + k), In[p * B + k], acc);
-                    tR[t] = acc;
-                }
-            }
-            __syncthreads();
-            // u = c_f (F^- tL + F^+ tR)
-            for (int t = tid; t < FQ; t += CNT) {
-                const int p = t / DF, a = t - p * DF;
-                double acc = 0.0;
+            const R* W = VW + f * FACE_FACTORS + 4 * NQ + 4 * p;
+            const R* y = Y + (f * B + k) * 4;
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) acc = fma(F[p * NQ + q], tL[f * FQ + q * DF + a], acc);
-                if (inner) {
-#pragma unroll
-                    for (int q = 0; q < NQ; ++q) acc = fma(F[NQ * NQ + p * NQ + q], tR[q * DF + a], acc);
-                }
-                U[f * FQ + t] = cf * acc;
-            }
-            __syncthreads();
+            for (int cc = 0; cc < 4; ++cc) a[cc & 1] = P::fma(W[cc], y[cc], a[cc & 1]);
         }
-        // dQ[p][k] -= M_kk^{-1} sum_f sum_a Pf[f][a][k] U[f][p][a], then Q += dQ
-        for (int i = tid; i < QB; i += CNT) {
-            const int p = i / B, k = i - (i / B) * B;
-            double acc = 0.0;
+        q[it] = q0 + P::value(P::normal(P::add(a[0], a[1])));
+    }
+}
+
+// Q += E I - sum_j Khat^j A^j I in binary64: the volume line for a predictor
+// that did not write Q~(1) itself
+constexpr int VNT = 128;
+template <bool BATCH>
+__global__ void __launch_bounds__(VNT) volume_kernel(int N, const CorrectorData D1, const int32_t* elems,
+                                                     const CorrectorData* runs, const int32_t* item_run) {
+    extern __shared__ double smv[];
+    const int B = n_modes(N), QB = NQ * B;
+    double* I = smv;      // [13][B]
+    double* X = I + QB;   // [13][B]
+    const int tid = threadIdx.x;
+    const CorrectorData& D = BATCH ? runs[item_run[blockIdx.x]] : D1;
+    const int64_t e = elems ? elems[blockIdx.x] : (int64_t)blockIdx.x;
+    const double* ec = D.econst + e * elem_const_stride(N);
+    const double* sc = ec + ec_scalars(N);
+    const double ev = sc[0] / sc[2], gv = sc[1] / sc[2];
+    double* q = D.q + e * QB;
+    for (int i = tid; i < QB; i += VNT) I[i] = D.iout[e * QB + i];
+    for (int j = 0; j < 3; ++j) {
+        __syncthreads();
+        const double* sj = ec + j * STAR_NNZ;
+        for (int l = tid; l < B; l += VNT) {
+            double acc[NQ];
 #pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                const double* col = D.Pf + (size_t)f * DF * B + k;
-                const double* u = U + f * FQ + p * DF;
-#pragma unroll 4
-                for (int a = 0; a < DF; ++a) acc = fma(__ldg(col + (size_t)a * B), u[a], acc);
-            }
-            D.q[e * QB + i] += dQ[i] - D.minv[k] * acc;
+            for (int p = 0; p < NQ; ++p) acc[p] = 0.0;
+#pragma unroll
+            for (int n = 0; n < STAR_NNZ; ++n) acc[star_row(n)] = fma(sj[n], I[star_col(n) * B + l], acc[star_row(n)]);
+#pragma unroll
+            for (int p = 0; p < NQ; ++p) X[p * B + l] = acc[p] / sc[2];
         }
         __syncthreads();
+        const int32_t* kr = D.krow + j * (B + 1);
+        for (int i = tid; i < QB; i += VNT) {
+            const int p = i / B, k = i - p * B;
+            double acc = 0.0;
+            for (int n = kr[k]; n < kr[k + 1]; ++n) acc = fma(D.kval[n], X[p * B + D.kcol[n]], acc);
+            if (j == 0) {
+                // Darcy source term E I: u rows from u_f, u_f rows from u_f
+                if (p >= QU && p <= QW) acc = fma(-gv, I[(p + QUF - QU) * B + k], acc);
+                if (p >= QUF) acc = fma(-ev, I[i], acc);
+            }
+            q[i] -= acc;
+        }
     }
 }
 
@@ -286,32 +370,42 @@ __global__ void receiver_kernel(int B, const double* q, int32_t nrec, const int6
     out[r * stride_out + p] = acc;
 }
 
-template <int N>
-int launch_corr_n(const CorrectorData& d, const int32_t* elems, int64_t count, void* stream, const CorrectorData* runs,
-                  const int32_t* item_run) {
-    constexpr int B = n_modes(N), DF = (N + 1) * (N + 2) / 2;
-    const size_t smem = sizeof(double) * (4 * NQ * B + 9 * NQ * DF);
-    auto* kern = runs ? corrector_kernel<N, true> : corrector_kernel<N, false>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int N, class P>
+int launch_faces_p(const CorrectorData& d, const int32_t* elems, int64_t count, void* stream, const CorrectorData* runs,
+                   const int32_t* item_run) {
+    using S = FaceShape<N>;
+    auto* kern = runs ? face_kernel<N, P, true> : face_kernel<N, P, false>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BYTES);
     if (err != cudaSuccess) return (int)err;
-    const int64_t grid = count < (int64_t)(1u << 30) ? count : (int64_t)(1u << 30);
-    kern<<<(unsigned)grid, CNT, smem, (cudaStream_t)stream>>>(d, elems, count, runs, item_run);
+    kern<<<(unsigned)count, S::NT, S::SMEM_BYTES, (cudaStream_t)stream>>>(d, elems, runs, item_run);
     return (int)cudaGetLastError();
+}
+
+template <int N>
+int launch_faces_n(const CorrectorData& d, const int32_t* elems, int64_t count, void* stream, const CorrectorData* runs,
+                   const int32_t* item_run) {
+    return d.dw ? launch_faces_p<N, Bin32x2Base>(d, elems, count, stream, runs, item_run)
+                : launch_faces_p<N, Bin64Base>(d, elems, count, stream, runs, item_run);
 }
 
 }  // namespace
 
-int launch_corrector(const CorrectorData& d, const int32_t* elems, int64_t count, void* stream,
+int launch_corrector(const CorrectorData& d, bool volume, const int32_t* elems, int64_t count, void* stream,
                      const CorrectorData* runs, const int32_t* item_run) {
     if (count <= 0) return 0;
-    if (d.dw) return launch_corrector_dw(d, elems, count, stream, runs, item_run);
+    if (volume) {
+        const size_t smem = sizeof(double) * 2 * NQ * n_modes(d.N);
+        auto* kern = runs ? volume_kernel<true> : volume_kernel<false>;
+        kern<<<(unsigned)count, VNT, smem, (cudaStream_t)stream>>>(d.N, d, elems, runs, item_run);
+        if (const cudaError_t err = cudaGetLastError()) return (int)err;
+    }
     switch (d.N) {
-        case 1: return launch_corr_n<1>(d, elems, count, stream, runs, item_run);
-        case 2: return launch_corr_n<2>(d, elems, count, stream, runs, item_run);
-        case 3: return launch_corr_n<3>(d, elems, count, stream, runs, item_run);
-        case 4: return launch_corr_n<4>(d, elems, count, stream, runs, item_run);
-        case 5: return launch_corr_n<5>(d, elems, count, stream, runs, item_run);
-        case 6: return launch_corr_n<6>(d, elems, count, stream, runs, item_run);
+        case 1: return launch_faces_n<1>(d, elems, count, stream, runs, item_run);
+        case 2: return launch_faces_n<2>(d, elems, count, stream, runs, item_run);
+        case 3: return launch_faces_n<3>(d, elems, count, stream, runs, item_run);
+        case 4: return launch_faces_n<4>(d, elems, count, stream, runs, item_run);
+        case 5: return launch_faces_n<5>(d, elems, count, stream, runs, item_run);
+        case 6: return launch_faces_n<6>(d, elems, count, stream, runs, item_run);
         default: return (int)cudaErrorInvalidValue;
     }
 }

@@ -176,27 +176,27 @@ void traction_rows(const double n[3], ld C[][NQ], int& rows, bool full) {
 }
 }  // namespace
 
-bool flux_solver(const poro_material& mL, const poro_material* mR, const double n[3], int kind, double* Fm,
-                 double* Fp, std::string& err) {
-    Scaled SL;
+namespace {
+// The 4 waves that enter element L through its face with outward normal n,
+// R [13][4], and their amplitudes G [4][13]: interior faces G (q_R - q_L), free
+// surface -G q_L, absorbing faces -G q_L (all of them are absorbed).
+bool incoming_waves(const poro_material& mL, const poro_material* mR, const double n[3], int kind, Scaled& SL,
+                    std::vector<ld>& RmL, ld G[4][NQ], std::string& err) {
     ld sigL;
     if (!scaled_normal_jacobian(mL, n, SL, sigL, err)) return false;
-    std::memset(Fp, 0, sizeof(double) * NQ * NQ);
-    if (kind == PORO_FACE_ABSORBING) {
-        std::vector<ld> P;
-        if (!projector(SL, sigL, true, P)) { err = "flux: sign iteration failed"; return false; }
-        // A_n^+ = A_n P^+ (physical frame: S (A_s P_s) S^{-1})
-        std::vector<ld> AP(NQ * NQ);
-        matmul(NQ, SL.A.data(), P.data(), AP.data());
-        for (int i = 0; i < NQ; ++i)
-            for (int j = 0; j < NQ; ++j) Fm[i * NQ + j] = (double)(AP[i * NQ + j] * SL.s[i] / SL.s[j]);
-        return true;
-    }
-    std::vector<ld> Pm, RmL;
+    std::vector<ld> Pm;
     if (!projector(SL, sigL, false, Pm)) { err = "flux: sign iteration failed"; return false; }
     range_basis(NQ, Pm, 4, RmL);
+    if (kind == PORO_FACE_ABSORBING)  // P^- = R (R^T P^-), R orthonormal in the scaled frame
+        for (int a = 0; a < 4; ++a)
+            for (int q = 0; q < NQ; ++q) {
+                ld s = 0;
+                for (int i = 0; i < NQ; ++i) s += RmL[i * 4 + a] * Pm[i * NQ + q];
+                G[a][q] = s / SL.s[q];
+            }
     for (int i = 0; i < NQ; ++i)
         for (int c = 0; c < 4; ++c) RmL[i * 4 + c] *= SL.s[i];  // physical frame
+    if (kind == PORO_FACE_ABSORBING) return true;
     ld C[8][NQ];
     int rows;
     const bool interior = (kind == PORO_FACE_INTERIOR);
@@ -237,13 +237,52 @@ bool flux_solver(const poro_material& mL, const poro_material* mR, const double 
     }
     if (!inverse_ld(nu, Mx.data(), Minv.data())) { err = "flux: singular interface system"; return false; }
     // G = first 4 rows of M^{-1} C  (alpha = G (q_R - q_L), or alpha = -G q_L)
-    ld G[4][NQ];
     for (int a = 0; a < 4; ++a)
         for (int q = 0; q < NQ; ++q) {
             ld s = 0;
             for (int r = 0; r < nu; ++r) s += Minv[a * nu + r] * Cs[r * NQ + q];
             G[a][q] = s;
         }
+    return true;
+}
+}  // namespace
+
+bool flux_factors(const poro_material& mL, const poro_material* mR, const double n[3], int kind, double* V, double* W,
+                  std::string& err) {
+    Scaled SL;
+    std::vector<ld> R;
+    ld G[4][NQ];
+    if (!incoming_waves(mL, mR, n, kind, SL, R, G, err)) return false;
+    for (int p = 0; p < NQ; ++p)
+        for (int a = 0; a < 4; ++a) {
+            ld s = 0;
+            for (int q = 0; q < NQ; ++q) s += SL.An[p * NQ + q] * R[q * 4 + a];
+            V[p * 4 + a] = (double)G[a][p];
+            W[p * 4 + a] = (double)s;
+        }
+    return true;
+}
+
+bool flux_solver(const poro_material& mL, const poro_material* mR, const double n[3], int kind, double* Fm,
+                 double* Fp, std::string& err) {
+    Scaled SL;
+    std::memset(Fp, 0, sizeof(double) * NQ * NQ);
+    if (kind == PORO_FACE_ABSORBING) {
+        ld sigL;
+        if (!scaled_normal_jacobian(mL, n, SL, sigL, err)) return false;
+        std::vector<ld> P;
+        if (!projector(SL, sigL, true, P)) { err = "flux: sign iteration failed"; return false; }
+        // A_n^+ = A_n P^+ (physical frame: S (A_s P_s) S^{-1})
+        std::vector<ld> AP(NQ * NQ);
+        matmul(NQ, SL.A.data(), P.data(), AP.data());
+        for (int i = 0; i < NQ; ++i)
+            for (int j = 0; j < NQ; ++j) Fm[i * NQ + j] = (double)(AP[i * NQ + j] * SL.s[i] / SL.s[j]);
+        return true;
+    }
+    std::vector<ld> RmL;
+    ld G[4][NQ];
+    if (!incoming_waves(mL, mR, n, kind, SL, RmL, G, err)) return false;
+    const bool interior = (kind == PORO_FACE_INTERIOR);
     // K = R_L^- G ;  F^- = A_n (I - K),  F^+ = A_n K (interior)
     ld K[NQ][NQ];
     for (int i = 0; i < NQ; ++i)
@@ -360,45 +399,24 @@ void triangle_rule(int N, std::vector<double>& a, std::vector<double>& b, std::v
 //   phi_k(chi_f(t)) = sum_a Pf[f][a][k] psi_a(t)   exactly, and
 //   Floc[f] = Pf[f]^T Pf[f],  Fnb[f,h,s] = Pf[f]^T Pnb[f,h,s]
 // with Pnb the neighbour's trace seen in this face's parameters.
-void face_traces(int N, std::vector<double>& Pf, std::vector<double>& Pnb) {
-    const int B = n_modes(N), df = (N + 1) * (N + 2) / 2;
+void face_traces(int N, std::vector<double>& Pf, std::vector<double>& turn) {
+    const int B = n_modes(N), df = face_modes(N);
     std::vector<double> qa, qb, qw;
     triangle_rule(N, qa, qb, qw);
     const int nq = (int)qw.size();
-    // psi at the quadrature points: [nq][df]; the starting functions are the
-    // collapsed-coordinate (Dubiner) polynomials of the triangle, already
-    // orthogonal, so the Cholesky step only normalises them
-    std::vector<long double> m((size_t)nq * df), G((size_t)df * df, 0.0L), Lc((size_t)df * df, 0.0L);
+    // the triangle's Dubiner polynomials at barycentrics (., a, b), orthogonal
+    auto poly = [&](long double a, long double b, long double* out) {
+        for (int g = 0, i = 0; g <= N; ++g)
+            for (int jj = 0; jj <= g; ++jj)
+                out[i++] = hjacobi(g - jj, 0, 0, 2 * a - (1 - b), 1 - b) * hjacobi(jj, 2 * (g - jj) + 1, 0, 2 * b - 1, 1);
+    };
+    std::vector<long double> m((size_t)nq * df), norm(df, 0.0L), t(df);
     for (int q = 0; q < nq; ++q) {
-        int i = 0;
-        const long double a = qa[q], b = qb[q];
-        for (int g = 0; g <= N; ++g)
-            for (int e = 0; e <= g; ++e) {
-                const int ii = g - e, jj = e;
-                m[(size_t)q * df + i++] = hjacobi(ii, 0, 0, 2 * a - (1 - b), 1 - b) * hjacobi(jj, 2 * ii + 1, 0, 2 * b - 1, 1);
-            }
+        poly(qa[q], qb[q], &m[(size_t)q * df]);
+        for (int a = 0; a < df; ++a) norm[a] += qw[q] * m[(size_t)q * df + a] * m[(size_t)q * df + a];
     }
-    for (int q = 0; q < nq; ++q)
-        for (int i = 0; i < df; ++i)
-            for (int j = 0; j < df; ++j) G[i * df + j] += qw[q] * m[(size_t)q * df + i] * m[(size_t)q * df + j];
-    for (int j = 0; j < df; ++j) {
-        long double d = G[j * df + j];
-        for (int k = 0; k < j; ++k) d -= Lc[j * df + k] * Lc[j * df + k];
-        Lc[j * df + j] = std::sqrt(d);
-        for (int i = j + 1; i < df; ++i) {
-            long double v = G[i * df + j];
-            for (int k = 0; k < j; ++k) v -= Lc[i * df + k] * Lc[j * df + k];
-            Lc[i * df + j] = v / Lc[j * df + j];
-        }
-    }
-    std::vector<long double> psi((size_t)nq * df);
-    for (int q = 0; q < nq; ++q)
-        for (int i = 0; i < df; ++i) {
-            long double v = m[(size_t)q * df + i];
-            for (int k = 0; k < i; ++k) v -= Lc[i * df + k] * psi[(size_t)q * df + k];
-            psi[(size_t)q * df + i] = v / Lc[i * df + i];
-        }
-    std::vector<long double> acc((size_t)4 * df * B, 0.0L), accn((size_t)96 * df * B, 0.0L);
+    for (int a = 0; a < df; ++a) norm[a] = 1.0L / std::sqrt(norm[a]);
+    std::vector<long double> acc((size_t)4 * df * B, 0.0L), acct((size_t)6 * df * df, 0.0L);
     std::vector<double> ph(B);
     for (int q = 0; q < nq; ++q) {
         const double lam[3] = {1 - qa[q] - qb[q], qa[q], qb[q]};
@@ -407,26 +425,83 @@ void face_traces(int N, std::vector<double>& Pf, std::vector<double>& Pnb) {
             face_point(f, lam, xi);
             basis_at(N, xi, ph.data());
             for (int a = 0; a < df; ++a) {
-                const long double c = qw[q] * psi[(size_t)q * df + a];
+                const long double c = qw[q] * norm[a] * m[(size_t)q * df + a];
                 for (int k = 0; k < B; ++k) acc[((size_t)f * df + a) * B + k] += c * ph[k];
             }
-            for (int h = 0; h < 4; ++h)
-                for (int s = 0; s < 6; ++s) {
-                    double mu[3];
-                    for (int i = 0; i < 3; ++i) mu[PERM[s][i]] = lam[i];
-                    double xr[3];
-                    face_point(h, mu, xr);
-                    basis_at(N, xr, ph.data());
-                    const size_t t = ((size_t)f * 4 + h) * 6 + s;
-                    for (int a = 0; a < df; ++a) {
-                        const long double c = qw[q] * psi[(size_t)q * df + a];
-                        for (int l = 0; l < B; ++l) accn[(t * df + a) * B + l] += c * ph[l];
-                    }
-                }
+        }
+        // the same point on the neighbour's face under permutation s
+        for (int s = 0; s < 6; ++s) {
+            double mu[3];
+            for (int i = 0; i < 3; ++i) mu[PERM[s][i]] = lam[i];
+            poly(mu[1], mu[2], t.data());
+            for (int a = 0; a < df; ++a)
+                for (int b = 0; b < df; ++b)
+                    acct[((size_t)s * df + a) * df + b] += qw[q] * norm[a] * m[(size_t)q * df + a] * norm[b] * t[b];
         }
     }
-    Pf.assign(acc.begin(), acc.end());
-    Pnb.assign(accn.begin(), accn.end());
+    // entries that vanish exactly come out at rounding size
+    auto clean = [](const std::vector<long double>& x, std::vector<double>& o) {
+        o.resize(x.size());
+        for (size_t i = 0; i < x.size(); ++i) o[i] = std::fabs(x[i]) < 1e-12L ? 0.0 : (double)x[i];
+    };
+    clean(acc, Pf);
+    clean(acct, turn);
+}
+
+void face_tables(int N, const std::vector<double>& mass, bool dw, std::vector<int32_t>& words) {
+    const int B = n_modes(N), df = face_modes(N), TG = (df + 7) / 8, BG = (B + 7) / 8;
+    std::vector<double> Pf, turn;
+    face_traces(N, Pf, turn);
+    const int32_t entries = face_turn_slots(N) + 6 * df;
+    words.assign((size_t)4 * entries, 0);
+    int32_t at = entries;
+    // one row (its non-zeros in order) into slot `slot` as row `id`
+    auto put_row = [&](int slot, int id, const std::vector<double>& row) {
+        const int32_t first = at;
+        for (int c = 0; c < (int)row.size(); ++c) {
+            if (row[c] == 0.0) continue;
+            int32_t w[4] = {0, 0, c, 0};
+            if (dw) {
+                const float h = (float)row[c], l = (float)(row[c] - (double)h);
+                std::memcpy(&w[0], &h, 4);
+                std::memcpy(&w[1], &l, 4);
+            } else {
+                std::memcpy(w, &row[c], 8);
+            }
+            words.insert(words.end(), w, w + 4);
+            ++at;
+        }
+        const int32_t s[4] = {first, at - first, id, 0};
+        std::memcpy(&words[(size_t)4 * slot], s, sizeof s);
+    };
+    // rows longest first, so that the 8 rows of a group are of like length
+    auto put_sorted = [&](int slot0, int slots, const std::vector<std::vector<double>>& rows) {
+        std::vector<int> order(rows.size()), len(rows.size());
+        for (size_t i = 0; i < rows.size(); ++i) {
+            order[i] = (int)i;
+            len[i] = (int)std::count_if(rows[i].begin(), rows[i].end(), [](double v) { return v != 0.0; });
+        }
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return len[a] > len[b]; });
+        for (int i = 0; i < slots; ++i) {
+            if (i < (int)order.size()) put_row(slot0 + i, order[i], rows[order[i]]);
+            else words[(size_t)4 * (slot0 + i) + 2] = -1;
+        }
+    };
+    for (int f = 0; f < 4; ++f) {
+        std::vector<std::vector<double>> tr(df, std::vector<double>(B)), bk(B, std::vector<double>(df));
+        for (int a = 0; a < df; ++a)
+            for (int k = 0; k < B; ++k) {
+                tr[a][k] = Pf[((size_t)f * df + a) * B + k];
+                bk[k][a] = tr[a][k] / mass[k];
+            }
+        put_sorted(face_trace_slots(N) + f * TG * 8, TG * 8, tr);
+        put_sorted(face_back_slots(N) + f * BG * 8, BG * 8, bk);
+    }
+    for (int s = 0; s < 6; ++s)
+        for (int a = 0; a < df; ++a) {
+            const double* r = &turn[((size_t)s * df + a) * df];
+            put_row(face_turn_slots(N) + s * df + a, a, std::vector<double>(r, r + df));
+        }
 }
 
 void face_matrices(int N, std::vector<double>& Floc, std::vector<double>& Fnb) {

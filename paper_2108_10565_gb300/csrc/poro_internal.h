@@ -11,6 +11,7 @@
 // the CUDA runtime's graph-exec handle (cudaGraphExec_t points to it),
 // declared here for the host translation units built without CUDA headers
 struct CUgraphExec_st;
+struct int4;
 
 namespace poro {
 
@@ -212,9 +213,24 @@ void basis_at(int N, const double xi[3], double* phi);
 // Floc[4][B][B] = int_face phi_k phi_l, Fnb[4][4][6][B][B] = int_face phi_k(L) phi_l(R)
 // for local face f, neighbour face h, vertex permutation s
 void face_matrices(int N, std::vector<double>& Floc, std::vector<double>& Fnb);
-// Pf[4][df][B], Pnb[96][df][B] with Floc[f] = Pf^T Pf, Fnb[f,h,s] = Pf^T Pnb,
-// df = (N+1)(N+2)/2 (traces in a basis orthonormal on the reference triangle)
-void face_traces(int N, std::vector<double>& Pf, std::vector<double>& Pnb);
+// the same face in factors: A_n^L - F^- = W V (every kind) and, on interior
+// faces, F^+ = W V; V and W as [13][4]
+bool flux_factors(const poro_material& mL, const poro_material* mR, const double n[3], int kind, double* V, double* W,
+                  std::string& err);
+// Pf[4][df][B] with Floc[f] = Pf^T Pf, df = (N+1)(N+2)/2: traces in the
+// normalised Dubiner basis of the reference triangle on each face (its vertices
+// in increasing local order); turn[6][df][df] with Fnb[f,h,s] = Pf[f]^T turn[s] Pf[h]
+void face_traces(int N, std::vector<double>& Pf, std::vector<double>& turn);
+// The corrector's table of 16-byte words (value as binary64 or as (hi, lo)
+// binary32, column): first the slots (first entry, entries, row; row -1: none)
+// of the traces, rows of Pf[f] in groups of 8, longest first; of M^{-1} Pf^T,
+// likewise; of the turns; then their entries.
+PORO_HD constexpr int face_modes(int N) { return (N + 1) * (N + 2) / 2; }
+PORO_HD constexpr int face_trace_slots(int) { return 0; }
+PORO_HD constexpr int face_back_slots(int N) { return 4 * ((face_modes(N) + 7) / 8) * 8; }
+PORO_HD constexpr int face_turn_slots(int N) { return face_back_slots(N) + 4 * ((n_modes(N) + 7) / 8) * 8; }
+constexpr int FACE_FACTORS = 2 * 4 * NQ;  // V and W of one face
+void face_tables(int N, const std::vector<double>& mass, bool dw, std::vector<int32_t>& words);
 int face_permutation_index(const int p[3]);
 
 // ----- device side (kernels) -----
@@ -253,6 +269,7 @@ struct RunPtrs {
     const double* econst;  // [ne][stride]
     double* qt;            // [ne][13][B][T] or nullptr
     double* iout;          // [ne][13][B] or nullptr
+    double* qend;          // [ne][13][B] or nullptr: Q~(1), the sum over the time modes (may be q0)
 };
 
 // Launch the mixed-precision predictor for `count` elements: binary32 sweeps
@@ -260,7 +277,7 @@ struct RunPtrs {
 // (device array) and `item_run`, the items come from several runs and q0,
 // econst, qt, iout are ignored.
 int launch_stp_mixed(const MixedReference& ref, int refine, const int32_t* elems, int64_t count,
-                     const double* q0, const double* econst, double* qt, double* iout, void* stream,
+                     const double* q0, const double* econst, double* qt, double* iout, double* qend, void* stream,
                      int variant = 0, const RunPtrs* runs = nullptr, const int32_t* item_run = nullptr);
 
 // Dense-LU comparator: reference data and per-batch scratch (factors,
@@ -312,22 +329,14 @@ struct CorrectorData {
     double* q = nullptr;              // [ne][13][B] DOFs, updated in place
     const int32_t* nb = nullptr;      // [ne][4]
     const int32_t* tab = nullptr;     // [ne][4] neighbour table index f*24 + h*6 + s, or -1
-    const double* fc = nullptr;       // [ne][4] 2 |S_f| / |J|
-    const double* fF = nullptr;       // [ne][4][2][169] flux solver matrices
-    const int32_t* vrow = nullptr;    // volume CSR rows [3][B+1] (absolute)
-    const int32_t* vcol = nullptr;
-    const double* vval = nullptr;     // Kv^j_kl = M_ll Khat^j_lk / M_kk
-    const double* minv = nullptr;     // [B] 1 / M_kk
-    // face traces (df = (N+1)(N+2)/2): Floc^f = Pf^T Pf, Fnb^{f,h,s} = Pf^T Pnb
-    const double* Pf = nullptr;       // [4][df][B]
-    const double* Pnb = nullptr;      // [96][df][B]
-    // double-binary32 (hi, lo) copies for the mixed-precision form (dw = true:
-    // the corrector runs in double-binary32 and fF is not needed)
-    bool dw = false;
-    const float* fF2 = nullptr;       // [ne][4][2][169] pairs
-    const float* Pf2 = nullptr;       // [4][df][B] pairs
-    const float* Pnb2 = nullptr;      // [96][df][B] pairs
-    const float* vval2 = nullptr;     // Kv^j values, pairs
+    bool dw = false;                  // double-binary32 (mixed-precision contexts), else binary64
+    // [ne][4][2][13][4]: V, then c_f W (c_f = 2 |S_f| / |J|), of each face in
+    // 8-byte words (binary64, or (hi, lo) binary32)
+    const void* fvw = nullptr;
+    const int4* ftab = nullptr;       // face_tables
+    const int32_t* krow = nullptr;    // full-row CSR of Khat^j [3][B+1] (absolute)
+    const int32_t* kcol = nullptr;
+    const double* kval = nullptr;
     // clustered local time stepping (all nullptr / 1 for global time stepping)
     int C = 1;                        // number of clusters
     const int32_t* cl = nullptr;      // [ne] cluster of each element
@@ -338,13 +347,13 @@ struct CorrectorData {
 };
 int launch_lts_buffers(int N, int C, const int32_t* elems, int64_t count, const int32_t* slot, const double* iout,
                        double* buf, int64_t tick, void* stream);
-// `runs` (device array, nullable) / `item_run`: a launch over several runs;
-// item i is element elems[i] of the run whose data is runs[item_run[i]] (d
-// then only selects the precision and degree)
-int launch_corrector(const CorrectorData& d, const int32_t* elems, int64_t count, void* stream,
+// The faces' part of the corrector; with `volume` first the volume and source
+// part (for a predictor that did not write Q~(1)).  `runs` (device array,
+// nullable) / `item_run`: a launch over several runs; item i is element
+// elems[i] of the run whose data is runs[item_run[i]] (d then only selects the
+// precision and degree)
+int launch_corrector(const CorrectorData& d, bool volume, const int32_t* elems, int64_t count, void* stream,
                      const CorrectorData* runs = nullptr, const int32_t* item_run = nullptr);
-int launch_corrector_dw(const CorrectorData& d, const int32_t* elems, int64_t count, void* stream,
-                        const CorrectorData* runs = nullptr, const int32_t* item_run = nullptr);
 int launch_point_source(int N, double* q, int64_t elem, const double* coef, double amp, void* stream);
 // One point source or receiver of one run, for the launches of a batched
 // group that serve all its runs' sources (then receivers) of a tick.
@@ -403,17 +412,17 @@ int upload_direct_tables(int N, const std::vector<int32_t>& ent, const std::vect
 // result NaN; status, wait_limit: the bounded wait of the double-binary32 form.
 int launch_stp_direct(const DeviceReference& ref, bool dw, bool whole_nan, int32_t* status, long long wait_limit,
                       const int32_t* elems, int64_t count, const double* q0, const double* econst, double* qt,
-                      double* iout, void* stream, int variant, const RunPtrs* runs,
+                      double* iout, double* qend, void* stream, int variant, const RunPtrs* runs,
                       const int32_t* item_run);
 
 // Launch the FP64 Algorithm-3 predictor for `count` elements.
-// q0[count][13][B], econst[count][stride], qt, iout nullable.
+// q0[count][13][B], econst[count][stride], qt, iout, qend (Q~(1), may be q0) nullable.
 // `elems` (nullable): element index list; outputs are indexed by element.
 // `variant` selects the CTA size (0: default, 1: the alternative the
 // autotuner may pick).  `runs` / `item_run`: items of several runs, as for
 // launch_stp_mixed.
 int launch_stp_fp64(const DeviceReference& ref, const int32_t* elems, int64_t count, const double* q0,
-                    const double* econst, double* qt, double* iout, void* stream, int variant = 0,
+                    const double* econst, double* qt, double* iout, double* qend, void* stream, int variant = 0,
                     const RunPtrs* runs = nullptr, const int32_t* item_run = nullptr);
 // The same kernel for the damped Maxwell system (q0 [count][6][B], econst
 // [count][maxwell::elem_const_stride(N)], qt [count][6][B][T]).

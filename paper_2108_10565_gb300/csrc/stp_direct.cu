@@ -86,6 +86,7 @@ struct DirectParams {
     const double* econst;
     double* qt;
     double* iout;
+    double* qend;           // Q~(1) [ne][13][B], may be q0
     int64_t count;
     int stride;
     const double* inv_d;    // [B] 1 / d_l
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
 
     const int64_t it0 = blockIdx.x;
     const int64_t e = A.elems ? (int64_t)A.elems[it0] : it0;
-    RunPtrs run{A.q0, A.econst, A.qt, A.iout};
+    RunPtrs run{A.q0, A.econst, A.qt, A.iout, A.qend};
     if (A.runs) run = A.runs[A.item_run[it0]];
     const double* q0 = run.q0 + e * (int64_t)(NQ * B);
     const double* ec = run.econst + e * (int64_t)A.stride + S::EC0;
@@ -230,6 +231,7 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
     const double dt = raw[T * T + 2];
     double* qo = run.qt ? run.qt + e * (int64_t)(B * PT) : nullptr;
     double* io = run.iout ? run.iout + e * (int64_t)(NQ * B) : nullptr;
+    double* qe = run.qend ? run.qend + e * (int64_t)(NQ * B) : nullptr;
     int buf = 0;
 #pragma unroll 1
     for (int g = N; g >= 0; --g) {
@@ -242,7 +244,7 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
             const int m = o + min(mb + min(grp, G - 1), d - 1);
             R* c = C + m * PT + u;
             // lane u of a group loads entry u of the task's q0
-            auto load = [&](int q) { return P::of(__ldg(q0 + q * B + m)); };
+            auto load = [&](int q) { return P::of(q0[q * B + m]); };
             // b = S^{-1}w q0 + a, with entry i of the task's q0
             auto rhs = [&](R ql, int i, R a) { return P::fma1(sw, P::shfl(ql, base + i), a); };
             auto plain = [&](R b) {
@@ -258,6 +260,14 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                     const double v64 = P::value(x);
                     if (qo) qo[(q * B + m) * T + u] = v64;
                     if (io && u == 0) io[q * B + m] = dt * v64;
+                }
+                if (qe) {
+                    // Q~(1): the sum over u, chi_u(1) = 1 (the modes of q0 read by
+                    // this task are the ones written)
+                    R s = P::shfl(x, base + T - 1);
+#pragma unroll
+                    for (int n = T - 2; n >= 0; --n) s = P::add(s, P::shfl(x, base + n));
+                    if (act && u == 0) qe[q * B + m] = P::value(P::normal(s));
                 }
             };
             if (kind == 0) {
@@ -389,8 +399,10 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
     __syncthreads();
     if (flag[0]) {
         const double nan = __longlong_as_double(0x7FF8000000000000LL);
-        if (io)
-            for (int i = tid; i < NQ * B; i += NT) io[i] = nan;
+        for (int i = tid; i < NQ * B; i += NT) {
+            if (io) io[i] = nan;
+            if (qe) qe[i] = nan;
+        }
         if (qo)
             for (int i = tid; i < B * PT; i += NT) qo[i] = nan;
     }
@@ -520,7 +532,8 @@ int upload_direct_tables(int N, const std::vector<int32_t>& ent, const std::vect
 
 int launch_stp_direct(const DeviceReference& ref, bool dw, bool whole_nan, int32_t* status, long long wait_limit,
                       const int32_t* elems, int64_t count, const double* q0, const double* econst, double* qt,
-                      double* iout, void* stream, int variant, const RunPtrs* runs, const int32_t* item_run) {
+                      double* iout, double* qend, void* stream, int variant, const RunPtrs* runs,
+                      const int32_t* item_run) {
     if (count <= 0) return 0;
     DirectParams A;
     A.elems = elems;
@@ -528,6 +541,7 @@ int launch_stp_direct(const DeviceReference& ref, bool dw, bool whole_nan, int32
     A.econst = econst;
     A.qt = qt;
     A.iout = iout;
+    A.qend = qend;
     A.count = count;
     A.stride = elem_const_stride(ref.N);
     A.inv_d = ref.inv_d;

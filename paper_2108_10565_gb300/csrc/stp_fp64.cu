@@ -134,9 +134,9 @@ int launch_stp_fp64_visco(const DeviceReference& ref, int64_t count, const doubl
 }
 
 int launch_stp_fp64(const DeviceReference& ref, const int32_t* elems, int64_t count, const double* q0,
-                    const double* econst, double* qt, double* iout, void* stream, int variant,
+                    const double* econst, double* qt, double* iout, double* qend, void* stream, int variant,
                     const RunPtrs* runs, const int32_t* item_run) {
-    return launch_stp_direct(ref, false, false, nullptr, 0, elems, count, q0, econst, qt, iout, stream, variant,
+    return launch_stp_direct(ref, false, false, nullptr, 0, elems, count, q0, econst, qt, iout, qend, stream, variant,
                              runs, item_run);
 }
 

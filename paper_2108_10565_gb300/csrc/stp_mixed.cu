@@ -616,13 +616,13 @@ int launch_n(const MixedReference& ref, int variant, const int32_t* elems, int64
 }  // namespace
 
 int launch_stp_mixed(const MixedReference& ref, int refine, const int32_t* elems, int64_t count, const double* q0,
-                     const double* econst, double* qt, double* iout, void* stream, int variant, const RunPtrs* runs,
+                     const double* econst, double* qt, double* iout, double* qend, void* stream, int variant, const RunPtrs* runs,
                      const int32_t* item_run) {
     if (refine == 1)
         return launch_stp_direct(*ref.base, true, true, ref.status, ref.wait_limit, elems, count, q0, econst, qt, iout,
-                                 stream, variant, runs, item_run);
+                                 qend, stream, variant, runs, item_run);
     if (refine == 2)
-        return launch_stp_direct(*ref.base, false, true, nullptr, 0, elems, count, q0, econst, qt, iout, stream,
+        return launch_stp_direct(*ref.base, false, true, nullptr, 0, elems, count, q0, econst, qt, iout, qend, stream,
                                  variant, runs, item_run);
     switch (ref.base->N) {
         case 1: return launch_n<1>(ref, variant, elems, count, q0, econst, qt, iout, stream, runs, item_run);

@@ -1,5 +1,5 @@
-"""GPU tests of the fixed-point predictor of Biot's system beyond the oracle parity tests: scale invariance to the last
-bit, the widest ranges, non-finite rows."""
+"""GPU tests of the fixed-point predictor of Biot's system and of the face corrector, beyond the oracle parity tests:
+scale invariance to the last bit, the widest ranges, and the corrector's two ways to the volume term."""
 import numpy as np
 import pytest
 
@@ -77,3 +77,39 @@ def test_non_finite_binary64_rows(L, bad, mode):
     assert not np.isfinite(dirty[2, 7]).all()
     if mode == -1:  # the last mode feeds the lower ones
         assert not np.isfinite(dirty[2, :, 0]).all()
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("precision,sweeps,tol", [(0, 1, 1e-13), (1, 1, 1e-11), (2, 2, 1e-11), (1, 0, 1e-4), (2, 0, 1e-2)])
+def test_step_equals_predict_and_correct(L, N, precision, sweeps, tol):
+    """One time step of poro_advance (the predictor writes Q~(1), the corrector adds the faces) against poro_predict and
+    poro_correct (volume term from the time integral, then the faces); with no refinement sweep both take the second
+    way, and the step is compared with binary64's.  Free surface, absorbing and interior faces of two materials."""
+    from paper_2108_10565_gb300 import inputs
+
+    mesh = inputs.kuhn_box_mesh((3, 2, 2), lo=(0, 0, -1), hi=(1.5, 1.2, 0), periodic=(True, False, False), tags={"z+": 1})
+    ne = mesh["tets"].shape[0]
+    z = mesh["vertices"][mesh["tets"]].mean(axis=1)[:, 2]
+    mats = np.where((z > -0.5)[:, None], inputs.REFERENCE_MATERIAL, inputs.HALFSPACE_MATERIAL)
+    q0 = np.random.default_rng(N).standard_normal((ne, 13, (N + 1) * (N + 2) * (N + 3) // 6))
+
+    def run(prec, advance):
+        ctx = L.poro_create(0, N, prec)
+        try:
+            if prec:
+                L.poro_set_refinement(ctx, sweeps)
+            L.poro_set_mesh(ctx, mesh["vertices"], mesh["tets"], mesh["neighbors"], mesh["face_tag"])
+            L.poro_set_materials(ctx, mats)
+            dt, _ = L.poro_set_clusters(ctx, 0.5, 1)
+            L.poro_set_dofs(ctx, q0)
+            if advance:
+                L.poro_advance(ctx, 1.5 * dt)
+            else:
+                L.poro_predict(ctx)
+                L.poro_correct(ctx)
+            return L.poro_get_dofs(ctx)
+        finally:
+            L.poro_destroy(ctx)
+
+    a, b = run(precision, True), run(precision if sweeps else 0, False)
+    assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b), np.linalg.norm(a - b) / np.linalg.norm(b)
