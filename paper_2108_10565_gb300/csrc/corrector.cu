@@ -48,6 +48,34 @@ __device__ __forceinline__ void load_entry<Bin32x2Base>(const int4* at, float2& 
     col = e.z;
 }
 
+// sum over one row's entries of value times x[4 column], `width` rows a step;
+// the next 4 entries load while 4 are used
+template <class P>
+__device__ __forceinline__ typename P::R row_sum(const int4* ent, int steps, int width, const typename P::R* x) {
+    typename P::R a = P::zero(), b = P::zero(), v[4];
+    int k[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) load_entry<P>(ent + i * width, v[i], k[i]);
+    for (int n = 4; n <= steps; n += 4) {
+        typename P::R w[4];
+        int m[4];
+        const int4* next = ent + (n < steps ? n : 0) * width;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) load_entry<P>(next + i * width, w[i], m[i]);
+#pragma unroll
+        for (int i = 0; i < 4; i += 2) {
+            a = P::fma(v[i], x[k[i] * 4], a);
+            b = P::fma(v[i + 1], x[k[i + 1] * 4], b);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v[i] = w[i];
+            k[i] = m[i];
+        }
+    }
+    return P::add(a, b);
+}
+
 template <int N>
 struct FaceShape {
     // a thread takes whole columns of the first step (8 B of them)
@@ -171,14 +199,7 @@ __global__ void __launch_bounds__(FaceShape<N>::NT)
         if (sf >= 4 && side[f].mode == 0) continue;
         const int ft = sf < 4 ? f : side[f].face;
         const int4 row = __ldg(D.ftab + face_trace_slots(N) + (ft * S::TG + t % S::TG) * 8 + rs);
-        const R* y = Y + sf * B * 4 + c;
-        R a = P::zero();
-        for (int n = row.x; n < row.x + row.y; ++n) {
-            R v;
-            int k;
-            load_entry<P>(D.ftab + n, v, k);
-            a = P::fma(v, y[k * 4], a);
-        }
+        const R a = row_sum<P>(D.ftab + row.x + rs, row.y, 8, Y + sf * B * 4 + c);
         if (row.z >= 0) tr[(sf * DF + row.z) * 4 + c] = a;
     }
     __syncthreads();
@@ -187,30 +208,15 @@ __global__ void __launch_bounds__(FaceShape<N>::NT)
         const int f = it / (4 * DF), ac = it - f * (4 * DF);
         if (side[f].mode == 0) continue;
         const int4 row = __ldg(D.ftab + face_turn_slots(N) + side[f].perm * DF + (ac >> 2));
-        const R* t = tr + (4 + f) * DF * 4 + (ac & 3);
-        R a = P::zero();
-        for (int n = row.x; n < row.x + row.y; ++n) {
-            R v;
-            int k;
-            load_entry<P>(D.ftab + n, v, k);
-            a = P::fma(v, t[k * 4], a);
-        }
         R* o = tr + f * DF * 4 + ac;
-        *o = P::sub(*o, a);
+        *o = P::sub(*o, row_sum<P>(D.ftab + row.x, row.y, 1, tr + (4 + f) * DF * 4 + (ac & 3)));
     }
     __syncthreads();
     // M^{-1} Pf^T of the 4 rows, into the own side of Y
     for (int t = warp; t < 4 * S::BG; t += NW) {
         const int f = t / S::BG;
         const int4 row = __ldg(D.ftab + face_back_slots(N) + t * 8 + rs);
-        const R* x = tr + f * DF * 4 + c;
-        R a = P::zero();
-        for (int n = row.x; n < row.x + row.y; ++n) {
-            R v;
-            int k;
-            load_entry<P>(D.ftab + n, v, k);
-            a = P::fma(v, x[k * 4], a);
-        }
+        const R a = row_sum<P>(D.ftab + row.x + rs, row.y, 8, tr + f * DF * 4 + c);
         if (row.z >= 0) Y[(f * B + row.z) * 4 + c] = a;
     }
     __syncthreads();

@@ -455,36 +455,47 @@ void face_tables(int N, const std::vector<double>& mass, bool dw, std::vector<in
     const int32_t entries = face_turn_slots(N) + 6 * df;
     words.assign((size_t)4 * entries, 0);
     int32_t at = entries;
-    // one row (its non-zeros in order) into slot `slot` as row `id`
-    auto put_row = [&](int slot, int id, const std::vector<double>& row) {
-        const int32_t first = at;
-        for (int c = 0; c < (int)row.size(); ++c) {
-            if (row[c] == 0.0) continue;
-            int32_t w[4] = {0, 0, c, 0};
-            if (dw) {
-                const float h = (float)row[c], l = (float)(row[c] - (double)h);
-                std::memcpy(&w[0], &h, 4);
-                std::memcpy(&w[1], &l, 4);
-            } else {
-                std::memcpy(w, &row[c], 8);
-            }
-            words.insert(words.end(), w, w + 4);
-            ++at;
+    auto put_entry = [&](double v, int c) {
+        int32_t w[4] = {0, 0, c, 0};
+        if (dw) {
+            const float h = (float)v, l = (float)(v - (double)h);
+            std::memcpy(&w[0], &h, 4);
+            std::memcpy(&w[1], &l, 4);
+        } else {
+            std::memcpy(w, &v, 8);
         }
-        const int32_t s[4] = {first, at - first, id, 0};
-        std::memcpy(&words[(size_t)4 * slot], s, sizeof s);
+        words.insert(words.end(), w, w + 4);
+        ++at;
     };
-    // rows longest first, so that the 8 rows of a group are of like length
-    auto put_sorted = [&](int slot0, int slots, const std::vector<std::vector<double>>& rows) {
-        std::vector<int> order(rows.size()), len(rows.size());
+    // rows in groups of `width` slots, longest first (so that a group's rows are
+    // of like length): a group's entries are step by step the next non-zero of
+    // each of its rows, zeros after a row's end, a multiple of 4 steps
+    auto put_rows = [&](int slot0, int slots, int width, bool sorted, const std::vector<std::vector<double>>& rows) {
+        std::vector<std::vector<int>> cols(rows.size());
+        std::vector<int> order(rows.size());
         for (size_t i = 0; i < rows.size(); ++i) {
             order[i] = (int)i;
-            len[i] = (int)std::count_if(rows[i].begin(), rows[i].end(), [](double v) { return v != 0.0; });
+            for (int c = 0; c < (int)rows[i].size(); ++c)
+                if (rows[i][c] != 0.0) cols[i].push_back(c);
         }
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return len[a] > len[b]; });
-        for (int i = 0; i < slots; ++i) {
-            if (i < (int)order.size()) put_row(slot0 + i, order[i], rows[order[i]]);
-            else words[(size_t)4 * (slot0 + i) + 2] = -1;
+        if (sorted)
+            std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cols[a].size() > cols[b].size(); });
+        for (int g = 0; g < slots / width; ++g) {
+            size_t steps = 0;
+            for (int r = 0; r < width; ++r)
+                if (g * width + r < (int)order.size()) steps = std::max(steps, cols[order[g * width + r]].size());
+            steps = (steps + 3) / 4 * 4;
+            for (int r = 0; r < width; ++r) {
+                const int i = g * width + r;
+                const int32_t s[4] = {at, (int32_t)steps, i < (int)order.size() ? order[i] : -1, 0};
+                std::memcpy(&words[(size_t)4 * (slot0 + i)], s, sizeof s);
+            }
+            for (size_t n = 0; n < steps; ++n)
+                for (int r = 0; r < width; ++r) {
+                    const int i = g * width + r;
+                    const bool in = i < (int)order.size() && n < cols[order[i]].size();
+                    put_entry(in ? rows[order[i]][cols[order[i]][n]] : 0.0, in ? cols[order[i]][n] : 0);
+                }
         }
     };
     for (int f = 0; f < 4; ++f) {
@@ -494,14 +505,17 @@ void face_tables(int N, const std::vector<double>& mass, bool dw, std::vector<in
                 tr[a][k] = Pf[((size_t)f * df + a) * B + k];
                 bk[k][a] = tr[a][k] / mass[k];
             }
-        put_sorted(face_trace_slots(N) + f * TG * 8, TG * 8, tr);
-        put_sorted(face_back_slots(N) + f * BG * 8, BG * 8, bk);
+        put_rows(face_trace_slots(N) + f * TG * 8, TG * 8, 8, true, tr);
+        put_rows(face_back_slots(N) + f * BG * 8, BG * 8, 8, true, bk);
     }
-    for (int s = 0; s < 6; ++s)
+    for (int s = 0; s < 6; ++s) {
+        std::vector<std::vector<double>> rows(df);
         for (int a = 0; a < df; ++a) {
             const double* r = &turn[((size_t)s * df + a) * df];
-            put_row(face_turn_slots(N) + s * df + a, a, std::vector<double>(r, r + df));
+            rows[a].assign(r, r + df);
         }
+        put_rows(face_turn_slots(N) + s * df, df, 1, false, rows);
+    }
 }
 
 void face_matrices(int N, std::vector<double>& Floc, std::vector<double>& Fnb) {

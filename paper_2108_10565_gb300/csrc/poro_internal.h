@@ -221,10 +221,11 @@ bool flux_factors(const poro_material& mL, const poro_material* mR, const double
 // normalised Dubiner basis of the reference triangle on each face (its vertices
 // in increasing local order); turn[6][df][df] with Fnb[f,h,s] = Pf[f]^T turn[s] Pf[h]
 void face_traces(int N, std::vector<double>& Pf, std::vector<double>& turn);
-// The corrector's table of 16-byte words (value as binary64 or as (hi, lo)
-// binary32, column): first the slots (first entry, entries, row; row -1: none)
-// of the traces, rows of Pf[f] in groups of 8, longest first; of M^{-1} Pf^T,
-// likewise; of the turns; then their entries.
+// The corrector's table of 16-byte words: first the slots (first entry, steps, row;
+// row -1: none) of the traces, rows of Pf[f] in groups of 8, longest first; of
+// M^{-1} Pf^T, likewise; of the turns, one row each; then their entries (value as
+// binary64 or as (hi, lo) binary32, column), step by step for the rows of a group,
+// padded with zeros to a multiple of 4 steps.
 PORO_HD constexpr int face_modes(int N) { return (N + 1) * (N + 2) / 2; }
 PORO_HD constexpr int face_trace_slots(int) { return 0; }
 PORO_HD constexpr int face_back_slots(int N) { return 4 * ((face_modes(N) + 7) / 8) * 8; }

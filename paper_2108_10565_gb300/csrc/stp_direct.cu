@@ -251,7 +251,11 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 const R lo = P::shfl(b, lane - 1), hi = P::shfl(b, lane + 1);
                 return P::fma(z_hi, P::select(u == T - 1, b, hi), P::mul(z_lo, P::select(u == 0, b, lo)));
             };
-            auto put = [&](int q, R x) {
+            // x: row q of Q; end: in lane u = 0 its value at the end of the step,
+            // Q~(1) = b_0 + (E* Q)_0 (the columns of Z^{-1} but the first sum to
+            // zero).  q0 may be the array written: its entries read by this task
+            // are the ones it writes.
+            auto put = [&](int q, R x, R end) {
                 x = P::normal(x);
                 if (act) {
                     atomicMax(qmax + buf * PT + q * T + u, P::abs_bits(x));
@@ -261,14 +265,7 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                     if (qo) qo[(q * B + m) * T + u] = v64;
                     if (io && u == 0) io[q * B + m] = dt * v64;
                 }
-                if (qe) {
-                    // Q~(1): the sum over u, chi_u(1) = 1 (the modes of q0 read by
-                    // this task are the ones written)
-                    R s = P::shfl(x, base + T - 1);
-#pragma unroll
-                    for (int n = T - 2; n >= 0; --n) s = P::add(s, P::shfl(x, base + n));
-                    if (act && u == 0) qe[q * B + m] = P::value(P::normal(s));
-                }
+                if (qe && act && u == 0) qe[q * B + m] = P::value(P::normal(end));
             };
             if (kind == 0) {
                 // normal stresses and pressure from D, Df, n_x u, n_y v
@@ -278,20 +275,17 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 const R D = c[0], Df = c[T], gx = c[2 * T], gy = c[9 * T];
                 const R gz = P::sub(P::sub(D, gx), gy);
                 const R Lm = P::neg(P::fma(iso[10], Df, P::mul(iso[9], D)));
-                const R x0 = plain(rhs(q[0], 0, P::fma1(-2.f, gx, Lm)));
-                const R x1 = plain(rhs(q[1 / T], 1 % T, P::fma1(-2.f, gy, Lm)));
-                const R x2 = plain(rhs(q[2 / T], 2 % T, P::fma1(-2.f, gz, Lm)));
-                const R x3 = plain(rhs(q[3 / T], 3 % T, P::fma(iso[11], Df, P::mul(iso[10], D))));
-                put(SXX, x0);
-                put(SYY, x1);
-                put(SZZ, x2);
-                put(QP, x3);
+                const R b[4] = {rhs(q[0], 0, P::fma1(-2.f, gx, Lm)), rhs(q[1 / T], 1 % T, P::fma1(-2.f, gy, Lm)),
+                                rhs(q[2 / T], 2 % T, P::fma1(-2.f, gz, Lm)),
+                                rhs(q[3 / T], 3 % T, P::fma(iso[11], Df, P::mul(iso[10], D)))};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) put(i < 3 ? SXX + i : QP, plain(b[i]), b[i]);
             } else {
                 // one pair (u, u_f) of velocities and one shear stress
                 const int i = kind - 1;
                 const R q = load(u == 0 ? QU + i : u == 1 ? QUF + i : SXY + i);
                 const R qs = T > 2 ? q : load(SXY + i);
-                const R x = plain(rhs(qs, T > 2 ? 2 : 0, P::neg(c[(SXY + i) * T])));
+                const R bs = rhs(qs, T > 2 ? 2 : 0, P::neg(c[(SXY + i) * T]));
                 const R Sg = c[(QU + i) * T], Gp = c[(QUF + i) * T];
                 const R bu = rhs(q, 0, P::neg(P::fma(iso[13], Gp, P::mul(iso[12], Sg))));
                 const R bf = rhs(q, 1, P::fma(iso[14], Gp, P::mul(iso[13], Sg)));
@@ -299,10 +293,10 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
 #pragma unroll
                 for (int s = 1; s < T; ++s) xf = P::fma(zuf[u * T + s], P::shfl(bf, base + s), xf);
                 xf = P::normal(xf);
-                const R xu = plain(P::fma(K[T * T + 1], xf, bu));  // + g Q_uf
-                put(SXY + i, x);
-                put(QUF + i, xf);
-                put(QU + i, xu);
+                const R by = P::fma(K[T * T + 1], xf, bu);  // + g Q_uf
+                put(SXY + i, plain(bs), bs);
+                put(QUF + i, xf, qe ? P::fma(K[T * T], xf, bf) : bf);
+                put(QU + i, plain(by), by);
             }
         }
         __syncthreads();
