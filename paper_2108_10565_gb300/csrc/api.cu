@@ -87,6 +87,16 @@ struct poro_ctx {
     int32_t* d_cnt = nullptr;
     int64_t seis_cap = 0;                      // samples per receiver d_seis holds
     size_t rp_n = 0;                           // receivers uploaded to d_rp
+    // sources, then receivers, by cluster (rebuilt when either or their
+    // buffers change); [offset, count] per cluster
+    poro::TickItem* d_tick_items = nullptr;
+    bool tick_items_ok = false;
+    std::vector<std::pair<int32_t, int32_t>> src_of, rec_of;
+    // one cycle as a CUDA graph, for the settings in exec_key, and the cycles
+    // run with these settings
+    cudaGraphExec_t exec = nullptr;
+    std::vector<int64_t> exec_key;
+    int64_t exec_cycles = 0;
     std::vector<double> h_seis;                // staging for the D2H copy
 };
 
@@ -133,6 +143,11 @@ void free_mesh_device(poro_ctx* c) {
     dfree(c->d_rp);
     dfree(c->d_seis);
     dfree(c->d_cnt);
+    dfree(c->d_tick_items);
+    c->tick_items_ok = false;
+    if (c->exec) cudaGraphExecDestroy(c->exec);
+    c->exec = nullptr;
+    c->exec_key.clear();
     c->seis_cap = 0;
     c->rp_n = 0;
     c->ready = false;
@@ -1266,6 +1281,7 @@ poro_status poro_add_point_source(poro_ctx* c, const double xyz[3], const double
     cudaError_t er = upload((void**)&s.d_coef, coef.data(), coef.size() * sizeof(double));
     if (er != cudaSuccess) return cuda_fail(c, er, "poro_add_point_source");
     c->sources.push_back(s);
+    c->tick_items_ok = false;
     return PORO_OK;
 }
 
@@ -1321,11 +1337,10 @@ static bool step_in_place(const poro_ctx* c) { return c->prec == PORO_FP64 || c-
 
 enum : unsigned { TICK_PREDICT = 1, TICK_BUFFERS = 2, TICK_CORRECT = 4, TICK_SOURCES = 8, TICK_ALL = 15 };
 
-static int enqueue_tick(poro_ctx* c, int64_t k, unsigned what, const double* d_rp, double* d_seis, int64_t cap,
-                        int32_t* d_cnt, cudaStream_t st, std::vector<ClusterEvent>* prof = nullptr) {
+static int enqueue_tick(poro_ctx* c, int64_t k, unsigned what, cudaStream_t st,
+                        std::vector<ClusterEvent>* prof = nullptr) {
     const bool predict = (what & TICK_PREDICT) != 0;
     const int C = c->C;
-    const int nrec = (int)c->rec_elem.size();
     const bool want_qt = C > 1;
     const bool in_place = step_in_place(c);
     int rc = 0;
@@ -1360,24 +1375,20 @@ static int enqueue_tick(poro_ctx* c, int64_t k, unsigned what, const double* d_r
                 if (rc == 0) rc = mark(prof, cl, false, st);
                 continue;
             }
-            for (auto& src : c->sources)
-                if (rc == 0 && c->h_cl[src.elem] == cl)
-                    rc = poro::launch_point_source_tick(c->N, c->d_q0, src.elem, src.d_coef, src.f0, src.t0, c->dt, len,
-                                                        k, c->d_tick, st);
-            for (int r = 0; r < nrec && rc == 0; ++r)
-                if (c->h_cl[c->rec_elem[r]] == cl)
-                    rc = poro::launch_receiver_count(c->N, c->d_q0, c->rec_elem[r], d_rp + (size_t)r * c->B,
-                                                     d_seis + (size_t)r * cap * NQ, d_cnt + r, st);
+            if (rc == 0)
+                rc = poro::launch_source_list(c->N, c->d_tick_items + c->src_of[cl].first, c->src_of[cl].second, k, st);
+            if (rc == 0)
+                rc = poro::launch_tick_receivers(c->N, c->d_tick_items + c->rec_of[cl].first, c->rec_of[cl].second, st);
             if (rc == 0) rc = mark(prof, cl, false, st);
         }
     }
     return rc;
 }
 
-static int enqueue_cycle(poro_ctx* c, const double* d_rp, double* d_seis, int64_t cap, int32_t* d_cnt) {
+static int enqueue_cycle(poro_ctx* c) {
     const int64_t cycle = (int64_t)1 << (c->C - 1);
     int rc = 0;
-    for (int64_t k = 0; k < cycle && rc == 0; ++k) rc = enqueue_tick(c, k, TICK_ALL, d_rp, d_seis, cap, d_cnt, c->stream);
+    for (int64_t k = 0; k < cycle && rc == 0; ++k) rc = enqueue_tick(c, k, TICK_ALL, c->stream);
     if (rc == 0) rc = poro::launch_tick_advance(c->d_tick, cycle, c->stream);
     return rc;
 }
@@ -1400,6 +1411,7 @@ static poro_status prepare_advance(poro_ctx* c, int64_t ticks, cudaStream_t st, 
                 (er = cudaMalloc((void**)&c->d_cnt, nrec * sizeof(int32_t))) != cudaSuccess)
                 return cuda_fail(c, er, who);
             c->rp_n = nrec;
+            c->tick_items_ok = false;
             dfree(c->d_seis);
             c->seis_cap = 0;
         }
@@ -1409,8 +1421,50 @@ static poro_status prepare_advance(poro_ctx* c, int64_t ticks, cudaStream_t st, 
             if ((er = cudaMalloc((void**)&c->d_seis, (size_t)nrec * ticks * NQ * sizeof(double))) != cudaSuccess)
                 return cuda_fail(c, er, who);
             c->seis_cap = ticks;
+            c->tick_items_ok = false;
         }
         if ((er = cudaMemsetAsync(c->d_cnt, 0, nrec * sizeof(int32_t), st)) != cudaSuccess) return cuda_fail(c, er, who);
+    }
+    if (!c->tick_items_ok) {
+        std::vector<poro::TickItem> items;
+        c->src_of.clear();
+        c->rec_of.clear();
+        for (int cl = 0; cl < c->C; ++cl) {
+            const int32_t first = (int32_t)items.size();
+            for (const auto& s : c->sources) {
+                if (c->h_cl[s.elem] != cl) continue;
+                poro::TickItem it;
+                it.q = c->d_q0;
+                it.vec = s.d_coef;
+                it.tick = c->d_tick;
+                it.elem = s.elem;
+                it.len = (int64_t)1 << cl;
+                it.f0 = s.f0;
+                it.tc = s.t0;
+                it.dt = c->dt;
+                items.push_back(it);
+            }
+            c->src_of.push_back({first, (int32_t)items.size() - first});
+        }
+        for (int cl = 0; cl < c->C; ++cl) {
+            const int32_t first = (int32_t)items.size();
+            for (int r = 0; r < nrec; ++r) {
+                if (c->h_cl[c->rec_elem[r]] != cl) continue;
+                poro::TickItem it;
+                it.q = c->d_q0;
+                it.vec = c->d_rp + (size_t)r * c->B;
+                it.out = c->d_seis + (size_t)r * c->seis_cap * NQ;
+                it.counter = c->d_cnt + r;
+                it.elem = c->rec_elem[r];
+                items.push_back(it);
+            }
+            c->rec_of.push_back({first, (int32_t)items.size() - first});
+        }
+        if ((er = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(c, er, who);
+        dfree(c->d_tick_items);
+        if ((er = upload((void**)&c->d_tick_items, items.data(), items.size() * sizeof(poro::TickItem))) != cudaSuccess)
+            return cuda_fail(c, er, who);
+        c->tick_items_ok = true;
     }
     return PORO_OK;
 }
@@ -1452,33 +1506,34 @@ poro_status poro_advance(poro_ctx* c, double t_end) {
     if (n_cycles <= 0) return PORO_OK;
     const int64_t ticks = n_cycles * cycle;
     if (poro_status st = prepare_advance(c, ticks, c->stream, "poro_advance")) return st;
-    double* d_rp = c->d_rp;
-    double* d_seis = c->d_seis;
-    int32_t* d_cnt = c->d_cnt;
-    const int64_t cap = c->seis_cap;
+    // The first cycle after a change of the settings runs directly (it also
+    // sets the kernels' attributes); the others, of this call and of later
+    // ones, replay a CUDA graph of one cycle.
+    const std::vector<int64_t> key = {c->variant, c->refine, c->mref.wait_limit, (int64_t)(intptr_t)c->d_tick_items,
+                                      (int64_t)c->sources.size(), (int64_t)c->rec_elem.size()};
+    if (key != c->exec_key) {
+        if (c->exec) cudaGraphExecDestroy(c->exec);
+        c->exec = nullptr;
+        c->exec_key = key;
+        c->exec_cycles = 0;
+    }
     cudaError_t er = cudaSuccess;
-    // the first cycle runs directly (it also sets the kernels' attributes);
-    // the others replay a CUDA graph of one cycle
-    int rc = enqueue_cycle(c, d_rp, d_seis, cap, d_cnt);
-    if (rc == 0 && n_cycles > 1) {
-        if (c->use_graphs) {
+    int rc = 0;
+    for (int64_t n = 0; n < n_cycles && rc == 0; ++n) {
+        if (c->use_graphs && !c->exec && c->exec_cycles > 0) {
             cudaGraph_t graph = nullptr;
-            cudaGraphExec_t exec = nullptr;
-            er = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
-            if (er == cudaSuccess) {
-                rc = enqueue_cycle(c, d_rp, d_seis, cap, d_cnt);
-                cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
-                if (rc == 0 && e2 != cudaSuccess) rc = (int)e2;
-            } else {
-                rc = (int)er;
+            rc = (int)cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
+            if (rc == 0) {
+                rc = enqueue_cycle(c);
+                const cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
+                if (rc == 0) rc = (int)e2;
             }
-            if (rc == 0) rc = (int)cudaGraphInstantiate(&exec, graph, 0);
-            for (int64_t k = 1; k < n_cycles && rc == 0; ++k) rc = (int)cudaGraphLaunch(exec, c->stream);
-            if (exec) cudaGraphExecDestroy(exec);
+            if (rc == 0) rc = (int)cudaGraphInstantiate(&c->exec, graph, 0);
+            if (rc != 0) c->exec = nullptr;
             if (graph) cudaGraphDestroy(graph);
-        } else {
-            for (int64_t k = 1; k < n_cycles && rc == 0; ++k) rc = enqueue_cycle(c, d_rp, d_seis, cap, d_cnt);
         }
+        if (rc == 0) rc = c->use_graphs && c->exec ? (int)cudaGraphLaunch(c->exec, c->stream) : enqueue_cycle(c);
+        ++c->exec_cycles;
     }
     if (rc == 0) er = stage_seismograms(c, c->stream);
     if (rc == 0 && er == cudaSuccess) er = cudaStreamSynchronize(c->stream);
@@ -1544,7 +1599,7 @@ static int enqueue_group_cycle(RunGroup* g) {
                                       g->stream, lead->variant, g->d_runs, ir);
         }
         for (poro_ctx* c : g->runs)
-            if (rc == 0) rc = enqueue_tick(c, k, TICK_BUFFERS, c->d_rp, c->d_seis, c->seis_cap, c->d_cnt, g->stream);
+            if (rc == 0) rc = enqueue_tick(c, k, TICK_BUFFERS, g->stream);
         const int64_t cc = g->ck_cnt[k];
         if (rc == 0 && cc > 0)
             rc = launch_corrector(lead->cd, !step_in_place(lead), g->d_citems + g->ck_off[k], cc, g->stream,
@@ -1800,7 +1855,7 @@ poro_status poro_cluster_times(poro_ctx* c, double t_end, double* ms_out) {
     int rc = 0;
     for (int64_t n = 0; n < n_cycles && rc == 0; ++n) {
         for (int64_t k = 0; k < cycle && rc == 0; ++k)
-            rc = enqueue_tick(c, k, TICK_ALL, c->d_rp, c->d_seis, c->seis_cap, c->d_cnt, c->stream, &prof);
+            rc = enqueue_tick(c, k, TICK_ALL, c->stream, &prof);
         if (rc == 0) rc = poro::launch_tick_advance(c->d_tick, cycle, c->stream);
     }
     cudaError_t er = cudaSuccess;

@@ -300,31 +300,21 @@ __global__ void lts_buffer_kernel(int QB, int C, const int32_t* elems, int64_t c
     }
 }
 
-// point source with the amplitude of the step computed on the device:
-// int_{t0}^{t1} s dt = S(t1) - S(t0), S(t) = (t - tc) exp(-(pi f0 (t - tc))^2),
-// the step [ (k+1-len) dt, (k+1) dt ], k = *tick + k_rel
-__global__ void point_source_tick_kernel(int QB, double* q, int64_t elem, const double* coef, double f0, double tc,
-                                         double dt, int64_t len, int64_t k_rel, const int64_t* tick) {
-    const int64_t k = *tick + k_rel;
-    const double t1 = (double)(k + 1) * dt, t0 = (double)(k + 1 - len) * dt;
-    const double a1 = 3.14159265358979323846 * f0 * (t1 - tc), a0 = 3.14159265358979323846 * f0 * (t0 - tc);
-    const double amp = (t1 - tc) * exp(-a1 * a1) - (t0 - tc) * exp(-a0 * a0);
-    for (int i = threadIdx.x; i < QB; i += blockDim.x) q[elem * QB + i] += amp * coef[i];
-}
-
-// receiver sample at the position given by a device counter
-__global__ void receiver_count_kernel(int B, const double* q, int64_t elem, const double* phi, double* out,
-                                      int32_t* counter) {
-    const int p = threadIdx.x;
-    const int32_t idx = *counter;
-    if (p < NQ) {
-        const double* qe = q + elem * (int64_t)(NQ * B) + p * B;
-        double acc = 0.0;
-        for (int l = 0; l < B; ++l) acc = fma(qe[l], phi[l], acc);
-        out[(int64_t)idx * NQ + p] = acc;
+// q[elem] += (S(t1) - S(t0)) vec over the step [(k+1-len) dt, (k+1) dt] with S the
+// antiderivative of the Ricker wavelet, S(t) = (t - tc) exp(-(pi f0 (t - tc))^2), k = *tick
+// + k_rel + k_add; one CTA
+__device__ void add_source(int QB, const TickItem& it, int64_t k_add) {
+    __shared__ double S[2];
+    if (threadIdx.x < 2) {  // S(t0), S(t1)
+        const int64_t k = *it.tick + it.k_rel + k_add;
+        const double t = (double)(threadIdx.x == 0 ? k + 1 - it.len : k + 1) * it.dt;
+        const double a = 3.14159265358979323846 * it.f0 * (t - it.tc);
+        S[threadIdx.x] = (t - it.tc) * exp(-a * a);
     }
     __syncthreads();
-    if (p == 0) *counter = idx + 1;
+    const double amp = S[1] - S[0];
+    double* q = it.q + it.elem * QB;
+    for (int i = threadIdx.x; i < QB; i += blockDim.x) q[i] += amp * it.vec[i];
 }
 
 __global__ void tick_advance_kernel(int64_t* tick, int64_t n) { *tick += n; }
@@ -334,46 +324,33 @@ __global__ void ticks_advance_kernel(int64_t* const* ticks, int count, int64_t n
     if (i < count) *ticks[i] += n;
 }
 
-// one CTA per source item of a batched group: the arithmetic of
-// point_source_tick_kernel
-__global__ void source_items_kernel(int QB, const TickItem* items) {
-    const TickItem& it = items[blockIdx.x];
-    const int64_t k = *it.tick + it.k_rel;
-    const double t1 = (double)(k + 1) * it.dt, t0 = (double)(k + 1 - it.len) * it.dt;
-    const double a1 = 3.14159265358979323846 * it.f0 * (t1 - it.tc), a0 = 3.14159265358979323846 * it.f0 * (t0 - it.tc);
-    const double amp = (t1 - it.tc) * exp(-a1 * a1) - (t0 - it.tc) * exp(-a0 * a0);
-    double* q = it.q + it.elem * QB;
-    for (int i = threadIdx.x; i < QB; i += blockDim.x) q[i] += amp * it.vec[i];
+// one CTA per source item (of several runs), or one CTA for a run's list (its
+// sources may share an element)
+__global__ void source_items_kernel(int QB, const TickItem* items) { add_source(QB, items[blockIdx.x], 0); }
+__global__ void source_list_kernel(int QB, const TickItem* items, int count, int64_t k_add) {
+    for (int i = 0; i < count; ++i) {
+        add_source(QB, items[i], k_add);
+        __syncthreads();
+    }
 }
 
-// one CTA per receiver item: the arithmetic of receiver_count_kernel
-__global__ void receiver_items_kernel(int B, const TickItem* items) {
+// one CTA per receiver item: out[*counter] = Q[elem] phi, then ++*counter; a warp per
+// quantity, lanes over the modes
+constexpr int RNT = 128;
+__global__ void __launch_bounds__(RNT) receiver_items_kernel(int B, const TickItem* items) {
     const TickItem& it = items[blockIdx.x];
-    const int p = threadIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t idx = *it.counter;
-    if (p < NQ) {
-        const double* qe = it.q + it.elem * (int64_t)(NQ * B) + p * B;
+    for (int p = warp; p < NQ; p += RNT / 32) {
+        const double* q = it.q + it.elem * (int64_t)(NQ * B) + p * B;
         double acc = 0.0;
-        for (int l = 0; l < B; ++l) acc = fma(qe[l], it.vec[l], acc);
-        it.out[(int64_t)idx * NQ + p] = acc;
+        for (int l = lane; l < B; l += 32) acc = fma(q[l], it.vec[l], acc);
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+        if (lane == 0) it.out[(int64_t)idx * NQ + p] = acc;
     }
     __syncthreads();
-    if (p == 0) *it.counter = idx + 1;
-}
-
-__global__ void point_source_kernel(int QB, double* q, int64_t elem, const double* coef, double amp) {
-    for (int i = threadIdx.x; i < QB; i += blockDim.x) q[elem * QB + i] += amp * coef[i];
-}
-
-// out[r * stride_out + p] = sum_l Q[e_r][p][l] phi_r[l]
-__global__ void receiver_kernel(int B, const double* q, int32_t nrec, const int64_t* elems, const double* phi,
-                                double* out, int64_t stride_out) {
-    const int r = blockIdx.x, p = threadIdx.x;
-    if (r >= nrec || p >= NQ) return;
-    const double* qe = q + elems[r] * (int64_t)(NQ * B) + p * B;
-    double acc = 0.0;
-    for (int l = 0; l < B; ++l) acc = fma(qe[l], phi[r * B + l], acc);
-    out[r * stride_out + p] = acc;
+    if (threadIdx.x == 0) *it.counter = idx + 1;
 }
 
 template <int N, class P>
@@ -425,28 +402,21 @@ int launch_lts_buffers(int N, int C, const int32_t* elems, int64_t count, const 
     return (int)cudaGetLastError();
 }
 
-int launch_point_source_tick(int N, double* q, int64_t elem, const double* coef, double f0, double tc, double dt,
-                             int64_t len, int64_t k_rel, const int64_t* tick, void* stream) {
-    point_source_tick_kernel<<<1, 256, 0, (cudaStream_t)stream>>>(NQ * n_modes(N), q, elem, coef, f0, tc, dt, len,
-                                                                  k_rel, tick);
-    return (int)cudaGetLastError();
-}
-
-int launch_receiver_count(int N, const double* q, int64_t elem, const double* phi, double* out, int32_t* counter,
-                          void* stream) {
-    receiver_count_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(n_modes(N), q, elem, phi, out, counter);
-    return (int)cudaGetLastError();
-}
-
 int launch_tick_sources(int N, const TickItem* items, int64_t count, void* stream) {
     if (count <= 0) return 0;
     source_items_kernel<<<(unsigned)count, 256, 0, (cudaStream_t)stream>>>(NQ * n_modes(N), items);
     return (int)cudaGetLastError();
 }
 
+int launch_source_list(int N, const TickItem* items, int count, int64_t k_add, void* stream) {
+    if (count <= 0) return 0;
+    source_list_kernel<<<1, 256, 0, (cudaStream_t)stream>>>(NQ * n_modes(N), items, count, k_add);
+    return (int)cudaGetLastError();
+}
+
 int launch_tick_receivers(int N, const TickItem* items, int64_t count, void* stream) {
     if (count <= 0) return 0;
-    receiver_items_kernel<<<(unsigned)count, 32, 0, (cudaStream_t)stream>>>(n_modes(N), items);
+    receiver_items_kernel<<<(unsigned)count, RNT, 0, (cudaStream_t)stream>>>(n_modes(N), items);
     return (int)cudaGetLastError();
 }
 
@@ -458,18 +428,6 @@ int launch_ticks_advance(int64_t* const* ticks, int count, int64_t n, void* stre
 
 int launch_tick_advance(int64_t* tick, int64_t n, void* stream) {
     tick_advance_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(tick, n);
-    return (int)cudaGetLastError();
-}
-
-int launch_point_source(int N, double* q, int64_t elem, const double* coef, double amp, void* stream) {
-    point_source_kernel<<<1, 256, 0, (cudaStream_t)stream>>>(NQ * n_modes(N), q, elem, coef, amp);
-    return (int)cudaGetLastError();
-}
-
-int launch_receivers(int N, const double* q, int32_t nrec, const int64_t* elems, const double* phi, double* out,
-                     int64_t stride_out, void* stream) {
-    if (nrec <= 0) return 0;
-    receiver_kernel<<<nrec, 32, 0, (cudaStream_t)stream>>>(n_modes(N), q, nrec, elems, phi, out, stride_out);
     return (int)cudaGetLastError();
 }
 

@@ -355,12 +355,10 @@ int launch_lts_buffers(int N, int C, const int32_t* elems, int64_t count, const 
 // precision and degree)
 int launch_corrector(const CorrectorData& d, bool volume, const int32_t* elems, int64_t count, void* stream,
                      const CorrectorData* runs = nullptr, const int32_t* item_run = nullptr);
-int launch_point_source(int N, double* q, int64_t elem, const double* coef, double amp, void* stream);
-// One point source or receiver of one run, for the launches of a batched
-// group that serve all its runs' sources (then receivers) of a tick.
-// Source: q[elem] += (S(t1) - S(t0)) coef over the step [(k+1-len) dt,
-// (k+1) dt], k = *tick + k_rel.  Receiver: out[*counter] = Q[elem] phi, then
-// ++*counter.
+// One point source or receiver of one run.  Source: q[elem] += (S(t1) - S(t0)) vec
+// over the step [(k+1-len) dt, (k+1) dt], k = *tick + k_rel (+ the launch's tick);
+// receiver: out[*counter] = Q[elem] vec, then ++*counter.  One launch takes the
+// sources (then one the receivers) of a cluster, or of all runs of a batched group.
 struct TickItem {
     double* q = nullptr;
     const double* vec = nullptr;     // coef (source) or phi (receiver)
@@ -371,16 +369,12 @@ struct TickItem {
     double f0 = 0.0, tc = 0.0, dt = 0.0;
 };
 int launch_tick_sources(int N, const TickItem* items, int64_t count, void* stream);
+// one run's list, in order, at tick k_add of the cycle
+int launch_source_list(int N, const TickItem* items, int count, int64_t k_add, void* stream);
 int launch_tick_receivers(int N, const TickItem* items, int64_t count, void* stream);
 // *ticks[i] += n for i < count (the tick counters of a group's runs)
 int launch_ticks_advance(int64_t* const* ticks, int count, int64_t n, void* stream);
-int launch_point_source_tick(int N, double* q, int64_t elem, const double* coef, double f0, double tc, double dt,
-                             int64_t len, int64_t k_rel, const int64_t* tick, void* stream);
-int launch_receiver_count(int N, const double* q, int64_t elem, const double* phi, double* out, int32_t* counter,
-                          void* stream);
 int launch_tick_advance(int64_t* tick, int64_t n, void* stream);
-int launch_receivers(int N, const double* q, int32_t nrec, const int64_t* elems, const double* phi, double* out,
-                     int64_t stride_out, void* stream);
 
 // Batched advance of several simulations (the server): runs of one degree,
 // precision, refinement, CTA variant and cluster count, each at the end of a
