@@ -175,17 +175,30 @@ struct SweepScratch {
     __device__ int* scale() const { return w + S::I_SCALE; }
     __device__ int* row() const { return w + S::I_ROW; }
 };
-// clears the maxima and fills the row starts and smax; the caller's barrier follows
+// star[3][NNZ] into the directions of the integer Khat rows, and smax; entries
+// are a thread's own, so no barrier is needed inside
+template <int NT, int NNZ>
+__device__ void adapt_star(double* star, double* smax) {
+    for (int i = threadIdx.x; i < NNZ; i += NT) {
+        double s0 = star[i], s1 = star[NNZ + i];
+        const double s2 = star[2 * NNZ + i];
+        adapted_directions(s0, s1, s2);
+        star[i] = s0;
+        star[NNZ + i] = s1;
+        smax[i] = fmax(fabs(s0), fmax(fabs(s1), fabs(s2)));
+    }
+}
+// clears the maxima, fills the row starts and adapts the star (loaded before the
+// caller's last barrier); the caller's barrier follows
 template <int NT, class S, class Sys>
-__device__ void sweep_setup(const SweepScratch<S>& W, double* smax, const double* star) {
+__device__ void sweep_setup(const SweepScratch<S>& W, double* smax, double* star) {
     for (int i = threadIdx.x; i < 2 * S::PT; i += NT) W.w[i] = 0;
     for (int i = threadIdx.x; i <= Sys::NQ; i += NT) {
         int n = 0;
         while (n < Sys::NNZ && Sys::row(n) < i) ++n;
         W.row()[i] = n;
     }
-    for (int i = threadIdx.x; i < Sys::NNZ; i += NT)
-        smax[i] = fmax(fabs(star[i]), fmax(fabs(star[Sys::NNZ + i]), fabs(star[2 * Sys::NNZ + i])));
+    adapt_star<NT, Sys::NNZ>(star, smax);
 }
 
 // dst[p, l, u] += SIGN sum_j sum_m Khat^j[l, o_g + m] X^j[p, m, u] for l < o_g with

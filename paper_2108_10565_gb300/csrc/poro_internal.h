@@ -391,6 +391,12 @@ void group_destroy(RunGroup* g);
 
 // x = num / den with den <= 10^6 if x is such a rational to 1e-14 relative
 bool rational_of(double x, int64_t& num, int64_t& den);
+// Coefficients of the derivatives along xi, eta, zeta -> along xi, eta - xi / 2,
+// zeta - eta, the directions of the integer Khat rows: sum_j n_j d_j is the same
+PORO_HD inline void adapted_directions(double& n0, double& n1, double n2) {
+    n1 += n2;
+    n0 += 0.5 * n1;
+}
 // Integer Khat rows in passes of at most `columns` columns (direction, mode) of
 // X: entries (column * stride, numerator) pass by pass, 1 / d_l per row, and
 // (appended to list) per pass the rows dealt to `warps` warps, [warps + 1]

@@ -418,8 +418,11 @@ bool element_constants(const ReferenceData& ref, const double* v12, const poro_m
     const double(*A)[NQ] = abc[0];
     const double mu = -A[SXY][QV];
     const double md = mu * dt, md_low = std::fma(mu, dt, -md);  // one rounding each, like the stars' entries
-    for (int j = 0; j < 3; ++j)
-        for (int d = 0; d < 3; ++d) iso[3 * j + d] = -std::fma(md, jinv[j][d], md_low * jinv[j][d]);
+    for (int d = 0; d < 3; ++d) {
+        double n[3] = {jinv[0][d], jinv[1][d], jinv[2][d]};
+        adapted_directions(n[0], n[1], n[2]);
+        for (int j = 0; j < 3; ++j) iso[3 * j + d] = -std::fma(md, n[j], md_low * n[j]);
+    }
     iso[9] = -A[SYY][QU] / mu;
     iso[10] = A[QP][QU] / mu;
     iso[11] = A[QP][QUF] / mu;

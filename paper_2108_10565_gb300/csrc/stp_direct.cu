@@ -55,7 +55,7 @@ namespace {
 // l << 21 | entries << 13 | first entry.
 constexpr int X_COLUMNS = 63;  // columns (direction, mode) of X a pass can hold
 constexpr int khat_entries(int N) {
-    return N == 1 ? 6 : N == 2 ? 46 : N == 3 ? 202 : N == 4 ? 647 : N == 5 ? 1708 : 3920;
+    return N == 1 ? 4 : N == 2 ? 29 : N == 3 ? 119 : N == 4 ? 364 : N == 5 ? 924 : 2058;
 }
 constexpr int entry_base(int N) { return N <= 1 ? 0 : entry_base(N - 1) + khat_entries(N - 1); }
 PORO_HD constexpr int n_passes(int N) { return N == 0 ? 0 : pass_count(N, X_COLUMNS) + n_passes(N - 1); }
@@ -424,6 +424,16 @@ int launch_n(const DirectParams& A, bool dw, int variant, void* stream) {
 bool khat_tables(const ReferenceData& R, int columns, int stride, int warps, std::vector<int32_t>& ent,
                  std::vector<int32_t>& list, std::vector<double>& inv_d, std::string& err) {
     const int N = R.N, B = R.B;
+    // The derivatives along xi, eta - xi / 2 and zeta - eta: the Dubiner basis is
+    // even or odd in the direction that collapses first, so these three matrices
+    // have 2,058 entries at N = 6 where those along xi, eta, zeta have 3,920
+    // (adapted_directions maps the coefficients).
+    std::vector<double> kh((size_t)3 * B * B);
+    for (size_t i = 0; i < (size_t)B * B; ++i) {
+        const double x = R.khat[i], y = R.khat[(size_t)B * B + i], z = R.khat[(size_t)2 * B * B + i];
+        const double v[3] = {x, y - 0.5 * x, z - y};
+        for (int j = 0; j < 3; ++j) kh[(size_t)j * B * B + i] = std::fabs(v[j]) < 1e-10 ? 0.0 : v[j];
+    }
     // integer rows over one denominator per row
     std::vector<int32_t> c((size_t)3 * B * B, 0);
     inv_d.assign(B, 1.0);
@@ -432,7 +442,7 @@ bool khat_tables(const ReferenceData& R, int columns, int stride, int warps, std
         for (int j = 0; j < 3; ++j)
             for (int m = 0; m < B; ++m) {
                 int64_t num = 0, den = 1;
-                const double v = R.khat[((size_t)j * B + l) * B + m];
+                const double v = kh[((size_t)j * B + l) * B + m];
                 if (v == 0.0) continue;
                 if (!rational_of(v, num, den) || (d = std::lcm(d, den)) > (1 << 30)) {
                     err = "Khat row has no small common denominator";
@@ -441,7 +451,7 @@ bool khat_tables(const ReferenceData& R, int columns, int stride, int warps, std
             }
         for (int j = 0; j < 3; ++j)
             for (int m = 0; m < B; ++m) {
-                const double v = R.khat[((size_t)j * B + l) * B + m] * (double)d;
+                const double v = kh[((size_t)j * B + l) * B + m] * (double)d;
                 const int64_t ci = std::llround(v);
                 sum += std::llabs(ci);
                 // the kernels' 64-bit sums need sum |c| < 2^23, their binary32 numerators |c| <= 2^22

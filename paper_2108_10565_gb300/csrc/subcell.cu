@@ -153,10 +153,8 @@ __global__ void __launch_bounds__(NT_) stp_subcell_kernel(const SubParams P) {
         init_rhs<NT, Sweep>(U, q0);
         __syncthreads();
         sweep_setup<NT, Sweep, BiotSystem>(X, smax, star);
-        for (int i = tid; i < NVAR * STAR_NNZ; i += NT) {
-            const double* s = var + (i / STAR_NNZ) * 3 * STAR_NNZ + i % STAR_NNZ;
-            smax[STAR_NNZ + i] = fmax(fabs(s[0]), fmax(fabs(s[STAR_NNZ]), fabs(s[2 * STAR_NNZ])));
-        }
+        for (int r = 0; r < NVAR; ++r)
+            adapt_star<NT, STAR_NNZ>(var + r * 3 * STAR_NNZ, smax + (1 + r) * STAR_NNZ);
         __syncthreads();
         alg3_sweep<N, NT, BiotSystem, Sweep>(U, star, zuf, sc[1], P.khat, X);  // Q_0 = Y_0^{-1} b0
         int it = 0;
