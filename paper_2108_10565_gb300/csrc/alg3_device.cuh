@@ -1,6 +1,6 @@
 // Device building blocks of the degree-block back-substitution (Section
-// "Block-wise back-substitution", Algorithm 3): the binary64 sweep of the
-// systems other than Biot's and of the sub-cell iteration, and the layout that
+// "Block-wise back-substitution", Algorithm 3): the binary64 sweep of
+// the Maxwell system and of the sub-cell iteration, and the layout that
 // the binary32 sweep of stp_mixed.cu shares.
 //
 // Shared-memory layout of one element's b / Q tensor: quantity p at offset
@@ -57,12 +57,10 @@ __device__ __forceinline__ void solve_row(double* row, const double* Zi, uint32_
 // (Z - e I)^{-1} and no coupling, and NPAIR pairs: src solved with
 // (Z - e I)^{-1}, then b_dst += g Q_src, then dst with Z^{-1}.
 // Per-element constants (in this order): star[3][NNZ], NSHM shifted time
-// matrices (Z - e I)^{-1}, NSC scalars with dt at DT_SC; TWO_PHASE systems
-// solve their blocks with solve_block (below) instead of the kinds above.
+// matrices (Z - e I)^{-1}, NSC scalars with dt at DT_SC.
 struct BiotSystem {  // Biot's equations: G couples u_f -> u, v_f -> v, w_f -> w
     static constexpr int NQ = poro::NQ, NNZ = STAR_NNZ, NPLAIN = 7, NSHIFT = 0, NPAIR = 3;
     static constexpr int NSHM = 1, NSC = 4, DT_SC = 2;
-    static constexpr bool TWO_PHASE = false;
     PORO_HD static constexpr int row(int n) { return star_row(n); }
     PORO_HD static constexpr int col(int n) { return star_col(n); }
     PORO_HD static constexpr int plain(int k) { return k < 6 ? k : QP; }
@@ -73,7 +71,6 @@ struct BiotSystem {  // Biot's equations: G couples u_f -> u, v_f -> v, w_f -> w
 struct MaxwellSystem {  // damped Maxwell: E diagonal, -sigma/eps on the electric rows
     static constexpr int NQ = maxwell::NQ, NNZ = maxwell::STAR_NNZ, NPLAIN = 3, NSHIFT = 3, NPAIR = 0;
     static constexpr int NSHM = 1, NSC = 4, DT_SC = 2;
-    static constexpr bool TWO_PHASE = false;
     PORO_HD static constexpr int row(int n) { return maxwell::star_row(n); }
     PORO_HD static constexpr int col(int n) { return maxwell::star_col(n); }
     PORO_HD static constexpr int plain(int k) { return 3 + k; }
@@ -81,58 +78,6 @@ struct MaxwellSystem {  // damped Maxwell: E diagonal, -sigma/eps on the electri
     PORO_HD static constexpr int pair_src(int) { return 0; }
     PORO_HD static constexpr int pair_dst(int) { return 0; }
 };
-// Viscoelastic attenuation: per mode, phase 1 solves the velocities with
-// Z^{-1} and mechanism l's six anelastic functions with (Z - e_l I)^{-1};
-// after a barrier, phase 2 adds to each stress its couplings to the solved
-// functions (E* strictly upper part) and solves it with Z^{-1}.
-struct ViscoSystem {
-    static constexpr int NQ = visco::NQ, NNZ = visco::STAR_NNZ, NPLAIN = 0, NSHIFT = 0, NPAIR = 0;
-    static constexpr int NSHM = visco::NMECH, NSC = visco::NSC, DT_SC = visco::sc_dt();
-    static constexpr bool TWO_PHASE = true;
-    PORO_HD static constexpr int row(int n) { return visco::star_row(n); }
-    PORO_HD static constexpr int col(int n) { return visco::star_col(n); }
-    PORO_HD static constexpr int plain(int) { return 0; }
-    PORO_HD static constexpr int shifted(int) { return 0; }
-    PORO_HD static constexpr int pair_src(int) { return 0; }
-    PORO_HD static constexpr int pair_dst(int) { return 0; }
-    // modes [o, o + d) of one degree block; zsh: NMECH matrices (Z - e_l I)^{-1};
-    // cp: per mechanism the couplings (normal diagonal, normal off-diagonal,
-    // shear) of E*.  The caller's barrier follows.
-    template <int T, int NT, int QS>
-    __device__ static void solve_block(double* bq, int o, int d, const double* zsh, const double* cp, uint32_t* qmax) {
-        const int tid = threadIdx.x;
-        constexpr int NM = visco::NMECH;
-        for (int it = tid; it < (3 + 6 * NM) * d; it += NT) {
-            const int kind = it / d, m = o + it % d, q = 6 + kind;
-            if (kind < 3) solve_plain<T>(bq + q * QS + m * T, qmax + q * T);
-            else solve_row<T>(bq + q * QS + m * T, zsh + ((kind - 3) / 6) * T * T, qmax + q * T);
-        }
-        __syncthreads();
-        for (int it = tid; it < 6 * d; it += NT) {
-            const int c = it / d, m = o + it % d;
-            double* row = bq + c * QS + m * T;
-#pragma unroll
-            for (int l = 0; l < NM; ++l) {
-                const double* th = bq + (9 + 6 * l) * QS + m * T;
-                if (c < 3) {
-                    // normal stress c: (Ylam + 2 Ymu) on th_cc, Ylam on the other two
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        const double g = k == c ? cp[3 * l] : cp[3 * l + 1];
-#pragma unroll
-                        for (int u = 0; u < T; ++u) row[u] = fma(g, th[k * QS + u], row[u]);
-                    }
-                } else {
-                    const double g = cp[3 * l + 2];
-#pragma unroll
-                    for (int u = 0; u < T; ++u) row[u] = fma(g, th[c * QS + u], row[u]);
-                }
-            }
-            solve_plain<T>(row, qmax + c * T);
-        }
-    }
-};
-
 template <int N, int NQ_ = NQ>
 struct Alg3Shape {
     static constexpr int B = n_modes(N);
@@ -292,12 +237,11 @@ __device__ __forceinline__ void init_rhs(double* bq, const double* q0) {
 
 // In-place sweep: on entry bq holds b, on exit the solution Q.  star[3][NNZ]:
 // the element's reference Jacobians on the union pattern; zsh: its NSHM shifted
-// matrices (Z - e I)^{-1}; gcoup = the coupling entry g of E* (Biot: E*_{u,uf});
-// cpl: the couplings of two-phase systems.  Begins after and ends with a
-// barrier; both maxima are clear at its ends.
+// matrices (Z - e I)^{-1}; gcoup = the coupling entry g of E* (Biot: E*_{u,uf}).
+// Begins after and ends with a barrier; both maxima are clear at its ends.
 template <int N, int NT, class Sys, class S>
 __device__ void alg3_sweep(double* bq, const double* star, const double* zsh, const double gcoup, const KhatRows& K,
-                           const SweepScratch<S>& W, const double* cpl = nullptr) {
+                           const SweepScratch<S>& W) {
     constexpr int T = S::T, QS = S::QS;
     const int tid = threadIdx.x;
     const int32_t* list = K.list;
@@ -310,26 +254,22 @@ __device__ void alg3_sweep(double* bq, const double* star, const double* zsh, co
         // and the coupled pairs (Biot: 6 stresses and p; u_f then u, v_f
         // then v, w_f then w)
         constexpr int NKIND = Sys::NPLAIN + Sys::NSHIFT + Sys::NPAIR;
-        if constexpr (Sys::TWO_PHASE) {
-            Sys::template solve_block<T, NT, QS>(bq, o, d, zsh, cpl, qm);
-        } else {
-            for (int it = tid; it < NKIND * d; it += NT) {
-                const int kind = it / d, m = o + it % d;
-                if (kind < Sys::NPLAIN) {
-                    const int q = Sys::plain(kind);
-                    solve_plain<T>(bq + q * QS + m * T, qm + q * T);
-                } else if (kind < Sys::NPLAIN + Sys::NSHIFT) {
-                    const int q = Sys::shifted(kind - Sys::NPLAIN);
-                    solve_row<T>(bq + q * QS + m * T, zsh, qm + q * T);
-                } else {
-                    const int i = kind - Sys::NPLAIN - Sys::NSHIFT, qf = Sys::pair_src(i), qv = Sys::pair_dst(i);
-                    double* rf = bq + qf * QS + m * T;
-                    double* rv = bq + qv * QS + m * T;
-                    solve_row<T>(rf, zsh, qm + qf * T);
+        for (int it = tid; it < NKIND * d; it += NT) {
+            const int kind = it / d, m = o + it % d;
+            if (kind < Sys::NPLAIN) {
+                const int q = Sys::plain(kind);
+                solve_plain<T>(bq + q * QS + m * T, qm + q * T);
+            } else if (kind < Sys::NPLAIN + Sys::NSHIFT) {
+                const int q = Sys::shifted(kind - Sys::NPLAIN);
+                solve_row<T>(bq + q * QS + m * T, zsh, qm + q * T);
+            } else {
+                const int i = kind - Sys::NPLAIN - Sys::NSHIFT, qf = Sys::pair_src(i), qv = Sys::pair_dst(i);
+                double* rf = bq + qf * QS + m * T;
+                double* rv = bq + qv * QS + m * T;
+                solve_row<T>(rf, zsh, qm + qf * T);
 #pragma unroll
-                    for (int u = 0; u < T; ++u) rv[u] = fma(gcoup, rf[u], rv[u]);
-                    solve_plain<T>(rv, qm + qv * T);
-                }
+                for (int u = 0; u < T; ++u) rv[u] = fma(gcoup, rf[u], rv[u]);
+                solve_plain<T>(rv, qm + qv * T);
             }
         }
         __syncthreads();

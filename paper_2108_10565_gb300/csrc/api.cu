@@ -276,7 +276,7 @@ poro_status poro_create_system(int device, int degree_N, poro_precision precisio
                                                                        : poro::subcell_columns(degree_N);
         const int warps = (mx ? poro::maxwell::threads(degree_N) : ve ? poro::visco::threads(degree_N)
                                                                       : poro::subcell_threads(degree_N)) / 32;
-        if (!poro::khat_tables(c->ref, columns, c->nq * c->T, warps, sent, slist, inv, err) ||
+        if (!poro::khat_tables(c->ref, columns, (ve ? poro::visco::ROWS : c->nq) * c->T, warps, sent, slist, inv, err) ||
             (system == PORO_SYSTEM_BIOT && !poro::direct_tables(c->ref, ent, list, inv, err))) {
             free_reference(c);
             cudaStreamDestroy(c->stream);

@@ -115,13 +115,15 @@ PORO_HD constexpr int star_col(int n) {
 // (NMECH), dt, pad
 constexpr int NSC = 3 * NMECH + NMECH + 2;
 PORO_HD constexpr int sc_dt() { return 4 * NMECH; }
-PORO_HD constexpr int elem_const_stride(int N) {
-    return (3 * STAR_NNZ + NMECH * (N + 1) * (N + 1) + NSC + 1) & ~1;
-}
-// CTA size of the predictor and the columns of X it holds (N = 5: block 5 in
-// three passes, so that two CTAs fit an SM; N = 6: blocks 6 and 5 in two)
+// ..., then (from an even offset) iso[16], the factors of the star products:
+// n^j = -dt grad xi_j [3][3], lam_u, 2 mu_u, mu_u, 1 / rho, omega[3]
+PORO_HD constexpr int ec_iso(int N) { return (3 * STAR_NNZ + NMECH * (N + 1) * (N + 1) + NSC + 1) & ~1; }
+PORO_HD constexpr int elem_const_stride(int N) { return ec_iso(N) + 16; }
+// CTA size of the predictor and the columns of X it holds (N = 6: block 6 in
+// two passes, so that three CTAs fit an SM)
 constexpr int threads(int N) { return N >= 4 ? 256 : N == 3 ? 128 : 64; }
-constexpr int columns(int N) { return N == 6 ? 42 : N == 5 ? 21 : 3 * block_size(N); }
+constexpr int columns(int N) { return N == 6 ? 63 : 3 * block_size(N); }
+constexpr int ROWS = 9;  // primitive rows the predictor's integer sums run over
 }  // namespace visco
 
 // Per-element constants, in doubles, in this order:

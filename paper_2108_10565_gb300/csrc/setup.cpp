@@ -550,6 +550,17 @@ bool visco_element_constants(const ReferenceData& ref, const double* v12, const 
         sc[3 * visco::NMECH + l] = e;
     }
     sc[visco::sc_dt()] = dt;
+    double* iso = out + visco::ec_iso(ref.N);
+    for (int d = 0; d < 3; ++d) {
+        double n[3] = {jinv[0][d], jinv[1][d], jinv[2][d]};
+        adapted_directions(n[0], n[1], n[2]);
+        for (int j = 0; j < 3; ++j) iso[3 * j + d] = -dt * n[j];
+    }
+    iso[9] = mat[1];
+    iso[10] = 2.0 * mat[2];
+    iso[11] = mat[2];
+    iso[12] = 1.0 / mat[0];
+    for (int l = 0; l < visco::NMECH; ++l) iso[13 + l] = mat[3 + l];
     return true;
 }
 

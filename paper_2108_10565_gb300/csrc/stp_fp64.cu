@@ -1,7 +1,7 @@
 // The space-time predictor of one element per CTA, in IEEE binary64, by the
 // degree-block back-substitution of the paper (Section "Block-wise
-// back-substitution", Algorithm 3), for the systems other than Biot's (whose
-// kernel is in stp_direct.cu): damped Maxwell and viscoelastic.
+// back-substitution", Algorithm 3), for the damped Maxwell system (Biot's
+// kernel is in stp_direct.cu, the viscoelastic one in stp_visco.cu).
 //
 // Per element the CTA keeps b (quantities x B x T) in shared memory and overwrites
 // it in place with the predictor Qt: once the modes of degree block g are solved,
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(NT) stp_fp64_kernel(const SweepParams P) {
     __syncthreads();
     sweep_setup<NT, S, Sys>(W, smax, star);
     __syncthreads();
-    alg3_sweep<N, NT, Sys, S>(bq, star, sm + S::OFF_ZSH, sc[1], P.khat, W, sc);
+    alg3_sweep<N, NT, Sys, S>(bq, star, sm + S::OFF_ZSH, sc[1], P.khat, W);
     // time integration and outputs (global layout [p][l][u], dense)
     const double dt = sc[Sys::DT_SC];
     if (P.iout) {
@@ -98,12 +98,6 @@ int launch_maxwell(const DeviceReference& ref, int64_t count, const double* q0, 
     return launch_nt<N, maxwell::threads(N), MaxwellSystem, maxwell::columns(N)>(ref, maxwell::elem_const_stride(N), count,
                                                                                  q0, econst, qt, iout, stream);
 }
-template <int N>
-int launch_visco(const DeviceReference& ref, int64_t count, const double* q0, const double* econst, double* qt,
-                 double* iout, void* stream) {
-    return launch_nt<N, visco::threads(N), ViscoSystem, visco::columns(N)>(ref, visco::elem_const_stride(N), count, q0,
-                                                                           econst, qt, iout, stream);
-}
 
 }  // namespace
 
@@ -116,19 +110,6 @@ int launch_stp_fp64_maxwell(const DeviceReference& ref, int64_t count, const dou
         case 4: return launch_maxwell<4>(ref, count, q0, econst, qt, iout, stream);
         case 5: return launch_maxwell<5>(ref, count, q0, econst, qt, iout, stream);
         case 6: return launch_maxwell<6>(ref, count, q0, econst, qt, iout, stream);
-        default: return (int)cudaErrorInvalidValue;
-    }
-}
-
-int launch_stp_fp64_visco(const DeviceReference& ref, int64_t count, const double* q0, const double* econst,
-                            double* qt, double* iout, void* stream) {
-    switch (ref.N) {
-        case 1: return launch_visco<1>(ref, count, q0, econst, qt, iout, stream);
-        case 2: return launch_visco<2>(ref, count, q0, econst, qt, iout, stream);
-        case 3: return launch_visco<3>(ref, count, q0, econst, qt, iout, stream);
-        case 4: return launch_visco<4>(ref, count, q0, econst, qt, iout, stream);
-        case 5: return launch_visco<5>(ref, count, q0, econst, qt, iout, stream);
-        case 6: return launch_visco<6>(ref, count, q0, econst, qt, iout, stream);
         default: return (int)cudaErrorInvalidValue;
     }
 }
