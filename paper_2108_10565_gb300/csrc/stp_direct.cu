@@ -116,9 +116,11 @@ struct Bin32x2 : Bin32x2Base {
 };
 
 // ------------------------------------------------------------ shape
-// CTA sizes the autotuner chooses from (index 0 is the default)
+// CTA sizes the autotuner chooses from (index 0 is the default), and the
+// largest one that a small launch gains from
 template <int N>
 struct DirectSizes {
+    static constexpr int WIDEST = N <= 2 ? 128 : N == 3 ? 256 : 512;
     static constexpr int NT0 = N == 6 ? 512 : N == 5 ? 256 : N == 4 ? 128 : 64;
     static constexpr int NT1 = N == 6 ? 256 : N == 5 ? 512 : N == 4 ? 256 : 128;
     static constexpr int MIN_BLOCKS = N == 6 ? 2 : N == 5 ? 3 : N == 4 ? 5 : 8;
@@ -412,11 +414,37 @@ int launch_nt(const DirectParams& A, void* stream) {
     return (int)cudaGetLastError();
 }
 
+// The default size is for launches that fill the chip several times over.  One
+// that leaves every CTA resident at once takes as long as one element, and the
+// phases of an element go faster on more warps: so the widest CTA is taken that
+// leaves at most 512 threads an SM.  Binary64 (double-binary32), microseconds a
+// launch, default size -> this rule, 152 SMs:
+//   100 elements   N = 2 13.8 -> 10.7 (13.3 -> 10.2)   N = 3 25.6 -> 15.5 (21.1 -> 13.3)
+//                  N = 4 31.0 -> 23.8 (25.8 -> 19.5)   N = 5 41.9 -> 37.0 (31.7 -> 27.5)
+//   304            N = 2 14.1 -> 12.5 (13.4 -> 10.8)   N = 3 26.4 -> 19.7 (21.3 -> 14.9)
+//   608            N = 2 17.9 -> 17.3 (14.9 -> 12.3)   N = 3 34.3 -> 31.3 (24.2 -> 18.6)
+// and one CTA more an SM turns it round (N = 3, 912 elements on 128 threads: 45.1
+// -> 62.5; 384 on 256: 28.8 -> 37.1).
+template <int N, class P>
+int launch_p(const DirectParams& A, int variant, void* stream) {
+    using D = DirectSizes<N>;
+    if (variant == 1) return launch_nt<N, D::NT1, P>(A, stream);
+    int dev = 0, sms = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (err != cudaSuccess) return (int)err;
+    if constexpr (D::WIDEST >= 512 && D::NT0 < 512)
+        if (A.count <= sms) return launch_nt<N, 512, P>(A, stream);
+    if constexpr (D::WIDEST >= 256 && D::NT0 < 256)
+        if (A.count <= 2 * (int64_t)sms) return launch_nt<N, 256, P>(A, stream);
+    if constexpr (D::NT0 < 128)
+        if (A.count <= 4 * (int64_t)sms) return launch_nt<N, 128, P>(A, stream);
+    return launch_nt<N, D::NT0, P>(A, stream);
+}
+
 template <int N>
 int launch_n(const DirectParams& A, bool dw, int variant, void* stream) {
-    constexpr int NT0 = DirectSizes<N>::NT0, NT1 = DirectSizes<N>::NT1;
-    if (dw) return variant == 1 ? launch_nt<N, NT1, Bin32x2>(A, stream) : launch_nt<N, NT0, Bin32x2>(A, stream);
-    return variant == 1 ? launch_nt<N, NT1, Bin64>(A, stream) : launch_nt<N, NT0, Bin64>(A, stream);
+    return dw ? launch_p<N, Bin32x2>(A, variant, stream) : launch_p<N, Bin64>(A, variant, stream);
 }
 
 }  // namespace

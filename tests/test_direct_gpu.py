@@ -113,3 +113,24 @@ def test_step_equals_predict_and_correct(L, N, precision, sweeps, tol):
 
     a, b = run(precision, True), run(precision if sweeps else 0, False)
     assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b), np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_launch_sizes_agree(L, N, precision):
+    """The CTA size that a launch takes by its number of elements (one, two or four CTAs an SM, or more) does not change
+    a bit of the predictor."""
+    d = population(613, N, seed=700 + N)
+    ctx = L.poro_create(0, N, precision)
+    try:
+        L.poro_set_isolated(ctx, d["vertices"], d["materials"], d["dt"])
+        L.poro_set_dofs(ctx, d["Q0"])
+        L.poro_set_variant(ctx, 1)
+        L.poro_predict(ctx)
+        ref = L.poro_get_predictor(ctx, 0, 613)
+    finally:
+        L.poro_destroy(ctx)
+    for n in (1, 152, 153, 304, 305, 608, 609):
+        part = {k: d[k][:n] for k in ("vertices", "materials")}
+        got = _predict(L, dict(part, N=N, dt=d["dt"]), precision, d["Q0"][:n])
+        np.testing.assert_array_equal(got, ref[:n], err_msg=f"{n} elements")
