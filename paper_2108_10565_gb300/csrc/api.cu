@@ -1146,8 +1146,10 @@ poro_status poro_set_clusters(poro_ctx* c, double cfl_c, int32_t max_clusters, d
             for (int i = 0; i < 2 * HALF; ++i) {
                 const double x = i < HALF ? itc->second[i] : cf * itc->second[i];
                 if (dw) {
-                    const float h = (float)x, hl[2] = {h, (float)(x - (double)h)};
-                    std::memcpy(dst + i, hl, sizeof hl);
+                    // entries 2n and 2n + 1: their high words, then their low ones
+                    float* to = reinterpret_cast<float*>(dst + i / 2 * 2) + i % 2;
+                    to[0] = (float)x;
+                    to[2] = (float)(x - (double)to[0]);
                 } else {
                     dst[i] = x;
                 }

@@ -23,7 +23,13 @@
 //
 // One CTA per element; neighbours are read only through I (or, for another
 // cluster, the buffered sub-step sums or the predictor), so Q is updated in
-// place.  What bounds it: binary64, the FP64 pipe; double-binary32, issue slots.
+// place.  What bounds it: binary64, the FP64 pipe; double-binary32, load and
+// barrier latency (issue slots 61 % busy).  Double-binary32 sums therefore run on
+// the packed binary32 operations, a lane per two of the 4 columns: half the
+// instructions, and a table entry is read by 2 lanes instead of 4.  A run of 5,184
+// elements at N = 6: 6.49 -> 6.33 ms a pass, 12 thousand in two clusters at N = 3:
+// 15.33 -> 15.06.  In binary64 that only leaves fewer lanes for the FP64 pipe
+// (N = 5, 6,000 elements: 3.54 -> 3.68 ms), so there a lane has one column.
 #include <cuda_runtime.h>
 
 #include "pair_device.cuh"
@@ -32,54 +38,60 @@
 namespace poro {
 namespace {
 
-// a table entry: value (binary64, or (hi, lo) binary32) and column
-template <class P>
-__device__ __forceinline__ void load_entry(const int4* at, typename P::R& v, int& col);
-template <>
-__device__ __forceinline__ void load_entry<Bin64Base>(const int4* at, double& v, int& col) {
-    const int4 e = __ldg(at);
-    v = __hiloint2double(e.y, e.x);
-    col = e.z;
+// 4 steps of a row's table entries: values (binary64, or (hi, lo) binary32)
+// and columns, a byte each
+template <class R>
+struct Entries {
+    R v[4];
+    uint32_t col;
+};
+__device__ __forceinline__ void load_values(const int4& a, const int4& b, double* v) {
+    v[0] = __hiloint2double(a.y, a.x);
+    v[1] = __hiloint2double(a.w, a.z);
+    v[2] = __hiloint2double(b.y, b.x);
+    v[3] = __hiloint2double(b.w, b.z);
 }
-template <>
-__device__ __forceinline__ void load_entry<Bin32x2Base>(const int4* at, float2& v, int& col) {
-    const int4 e = __ldg(at);
-    v = make_float2(__int_as_float(e.x), __int_as_float(e.y));
-    col = e.z;
+__device__ __forceinline__ void load_values(const int4& a, const int4& b, float2* v) {
+    v[0] = make_float2(__int_as_float(a.x), __int_as_float(a.y));
+    v[1] = make_float2(__int_as_float(a.z), __int_as_float(a.w));
+    v[2] = make_float2(__int_as_float(b.x), __int_as_float(b.y));
+    v[3] = make_float2(__int_as_float(b.z), __int_as_float(b.w));
+}
+template <int WIDTH, class R>
+__device__ __forceinline__ Entries<R> load_entries(const int4* at, int row) {
+    Entries<R> e;
+    load_values(__ldg(at + row), __ldg(at + WIDTH + row), e.v);
+    e.col = __ldg(reinterpret_cast<const uint32_t*>(at + 2 * WIDTH) + row);
+    return e;
 }
 
-// sum over one row's entries of value times x[4 column], `width` rows a step;
-// the next 4 entries load while 4 are used
-template <class P>
-__device__ __forceinline__ typename P::R row_sum(const int4* ent, int steps, int width, const typename P::R* x) {
-    typename P::R a = P::zero(), b = P::zero(), v[4];
-    int k[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) load_entry<P>(ent + i * width, v[i], k[i]);
+// sum over one row's entries of value times PACK columns of x [][4]; the rows of
+// a group of WIDTH lie side by side, and the next 4 steps load while 4 are used
+template <class P, int WIDTH>
+__device__ __forceinline__ typename P::V row_sum(const int4* ent, int steps, int row, const typename P::V* x) {
+    using R = typename P::R;
+    constexpr int C = 4 / P::PACK;
+    typename P::V a = P::zeros(), b = P::zeros();
+    if (steps == 0) return a;
+    Entries<R> e = load_entries<WIDTH, R>(ent, row);
     for (int n = 4; n <= steps; n += 4) {
-        typename P::R w[4];
-        int m[4];
-        const int4* next = ent + (n < steps ? n : 0) * width;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) load_entry<P>(next + i * width, w[i], m[i]);
+        if (n < steps) ent += face_block_words(WIDTH);
+        const Entries<R> next = load_entries<WIDTH, R>(ent, row);
 #pragma unroll
         for (int i = 0; i < 4; i += 2) {
-            a = P::fma(v[i], x[k[i] * 4], a);
-            b = P::fma(v[i + 1], x[k[i + 1] * 4], b);
+            a = P::vfma(P::all(e.v[i]), x[(e.col >> 8 * i & 255) * C], a);
+            b = P::vfma(P::all(e.v[i + 1]), x[(e.col >> (8 * i + 8) & 255) * C], b);
         }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            v[i] = w[i];
-            k[i] = m[i];
-        }
+        e = next;
     }
-    return P::add(a, b);
+    return P::vadd(a, b);
 }
 
 template <int N>
 struct FaceShape {
-    // a thread takes whole columns of the first step (8 B of them)
-    static constexpr int NT = N == 1 ? 32 : N == 2 ? 96 : N <= 4 ? 160 : 224, NW = NT / 32;
+    static constexpr int NT = N == 1 ? 32 : N == 2 ? 96 : N <= 4 ? 128 : 256;
+    static constexpr int MIN_BLOCKS = 1152 / NT;  // 1024 resident threads: 15.30 instead of 15.06 ms at N = 3
+    static constexpr int PG = NT / n_modes(N) < NQ ? NT / n_modes(N) : NQ;  // threads that share a mode in the last step
     static constexpr int B = n_modes(N), DF = face_modes(N), T = N + 1, TG = (DF + 7) / 8, BG = (B + 7) / 8;
     // shared layout in 8-byte words: the factors V [13][4], W [13][4] of the
     // four faces; Y [2 sides][4 faces][B][4]; traces [2][4][DF][4]
@@ -138,25 +150,27 @@ __device__ void face_side(const CorrectorData& D, int64_t e, int f, FaceSide& S)
 }
 
 template <int N, class P, bool BATCH>
-__global__ void __launch_bounds__(FaceShape<N>::NT)
+__global__ void __launch_bounds__(FaceShape<N>::NT, FaceShape<N>::MIN_BLOCKS)
     face_kernel(const CorrectorData D1, const int32_t* elems, const CorrectorData* runs, const int32_t* item_run) {
     using S = FaceShape<N>;
     using R = typename P::R;
-    constexpr int B = S::B, DF = S::DF, T = S::T, NT = S::NT, NW = S::NW;
+    using V = typename P::V;
+    constexpr int B = S::B, DF = S::DF, T = S::T, NT = S::NT;
+    constexpr int C = 4 / P::PACK, FACE = C * 2 * NQ;  // V's to 4 columns, and in one face's factors
     extern __shared__ __align__(16) double smf[];
-    R* VW = reinterpret_cast<R*>(smf);
-    R* Y = reinterpret_cast<R*>(smf) + S::OFF_Y;
-    R* tr = reinterpret_cast<R*>(smf) + S::OFF_T;
+    V* VW = reinterpret_cast<V*>(smf);
+    V* Y = reinterpret_cast<V*>(smf + S::OFF_Y);
+    V* tr = reinterpret_cast<V*>(smf + S::OFF_T);
     __shared__ FaceSide side[4];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x;
     // one run's data (D1), or the item's run of a batched launch over several
     // runs (their tables in global memory)
     const CorrectorData& D = BATCH ? runs[item_run[blockIdx.x]] : D1;
     const int64_t e = elems ? elems[blockIdx.x] : (int64_t)blockIdx.x;
     if (tid < 4) face_side<N>(D, e, tid, side[tid]);
     {
-        const R* g = reinterpret_cast<const R*>(D.fvw) + e * (int64_t)(4 * FACE_FACTORS);
-        for (int i = tid; i < 4 * FACE_FACTORS; i += NT) VW[i] = g[i];
+        const V* g = reinterpret_cast<const V*>(D.fvw) + e * (int64_t)(FACE * 4);
+        for (int i = tid; i < FACE * 4; i += NT) VW[i] = g[i];
     }
     __syncthreads();
     // Y[k][c] = sum_p V[p][c] I[p][k] of both sides of every face
@@ -178,62 +192,64 @@ __global__ void __launch_bounds__(FaceShape<N>::NT)
                 v[p] = P::of(a);
             }
         }
-        const R* V = VW + f * FACE_FACTORS;
-        R a[4];
+        const V* Vf = VW + f * FACE;
+        V a[C];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) a[c] = P::mul(V[c], v[0]);
+        for (int c = 0; c < C; ++c) a[c] = P::vmul(Vf[c], P::all(v[0]));
 #pragma unroll
         for (int p = 1; p < NQ; ++p)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) a[c] = P::fma(V[4 * p + c], v[p], a[c]);
-        R* y = Y + (sf * B + k) * 4;
+            for (int c = 0; c < C; ++c) a[c] = P::vfma(Vf[C * p + c], P::all(v[p]), a[c]);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) y[c] = a[c];
+        for (int c = 0; c < C; ++c) Y[(sf * B + k) * C + c] = a[c];
     }
     __syncthreads();
-    // traces of the 4 rows: a warp takes 8 rows of a face (ordered by length),
-    // lanes (row, c)
-    const int rs = lane >> 2, c = lane & 3;
-    for (int t = warp; t < 8 * S::TG; t += NW) {
-        const int sf = t / S::TG, f = sf & 3;  // sides 0: own, 1: the neighbour's
+    // traces of the 4 rows: 8 C lanes take 8 rows of a face (ordered by length),
+    // one per row and PACK columns
+    const int grp = tid / (8 * C), rs = tid / C % 8, c = tid % C;
+    constexpr int GROUPS = NT / (8 * C);
+    for (int t = grp; t < 8 * S::TG; t += GROUPS) {
+        const int sf = t & 7, f = t & 3;  // faces of side 0: own, 1: the neighbour's; long groups first
         if (sf >= 4 && side[f].mode == 0) continue;
         const int ft = sf < 4 ? f : side[f].face;
-        const int4 row = __ldg(D.ftab + face_trace_slots(N) + (ft * S::TG + t % S::TG) * 8 + rs);
-        const R a = row_sum<P>(D.ftab + row.x + rs, row.y, 8, Y + sf * B * 4 + c);
-        if (row.z >= 0) tr[(sf * DF + row.z) * 4 + c] = a;
+        const int4 row = __ldg(D.ftab + face_trace_slots(N) + (ft * S::TG + (t >> 3)) * 8 + rs);
+        const V a = row_sum<P, 8>(D.ftab + row.x, row.y, rs, Y + sf * B * C + c);
+        if (row.z >= 0) tr[(sf * DF + row.z) * C + c] = a;
     }
     __syncthreads();
     // difference of the sides, the neighbour's turned by its permutation
-    for (int it = tid; it < 16 * DF; it += NT) {
-        const int f = it / (4 * DF), ac = it - f * (4 * DF);
+    for (int it = tid; it < 4 * C * DF; it += NT) {
+        const int f = it / (C * DF), ac = it - f * (C * DF);
         if (side[f].mode == 0) continue;
-        const int4 row = __ldg(D.ftab + face_turn_slots(N) + side[f].perm * DF + (ac >> 2));
-        R* o = tr + f * DF * 4 + ac;
-        *o = P::sub(*o, row_sum<P>(D.ftab + row.x, row.y, 1, tr + (4 + f) * DF * 4 + (ac & 3)));
+        const int4 row = __ldg(D.ftab + face_turn_slots(N) + side[f].perm * DF + ac / C);
+        V* o = tr + f * DF * C + ac;
+        *o = P::vsub(*o, row_sum<P, 1>(D.ftab + row.x, row.y, 0, tr + (4 + f) * DF * C + ac % C));
     }
     __syncthreads();
     // M^{-1} Pf^T of the 4 rows, into the own side of Y
-    for (int t = warp; t < 4 * S::BG; t += NW) {
-        const int f = t / S::BG;
-        const int4 row = __ldg(D.ftab + face_back_slots(N) + t * 8 + rs);
-        const R a = row_sum<P>(D.ftab + row.x + rs, row.y, 8, tr + f * DF * 4 + c);
-        if (row.z >= 0) Y[(f * B + row.z) * 4 + c] = a;
+    for (int t = grp; t < 4 * S::BG; t += GROUPS) {
+        const int f = t & 3;
+        const int4 row = __ldg(D.ftab + face_back_slots(N) + (f * S::BG + (t >> 2)) * 8 + rs);
+        const V a = row_sum<P, 8>(D.ftab + row.x, row.y, rs, tr + f * DF * C + c);
+        if (row.z >= 0) Y[(f * B + row.z) * C + c] = a;
     }
     __syncthreads();
-    // Q[p][k] += sum_f sum_c (c_f W_f)[p][c] Y[f][k][c]
-    double* q = D.q + e * (int64_t)(NQ * B);
-    for (int it = tid; it < NQ * B; it += NT) {
-        const int p = it / B, k = it - p * B;
-        const double q0 = q[it];
-        R a[2] = {P::zero(), P::zero()};
+    // Q[p][k] += sum_f sum_c (c_f W_f)[p][c] Y[f][k][c]: a thread keeps its mode's
+    // Y for every PG-th quantity
+    if (tid < S::PG * B) {
+        const int p0 = tid / B, k = tid - p0 * B;
+        double* q = D.q + e * (int64_t)(NQ * B) + k;
+        V y[4 * C];
 #pragma unroll
-        for (int f = 0; f < 4; ++f) {
-            const R* W = VW + f * FACE_FACTORS + 4 * NQ + 4 * p;
-            const R* y = Y + (f * B + k) * 4;
+        for (int i = 0; i < 4 * C; ++i) y[i] = Y[(i / C * B + k) * C + i % C];
+        for (int p = p0; p < NQ; p += S::PG) {
+            const double q0 = q[p * B];
+            V a[2] = {P::zeros(), P::zeros()};
 #pragma unroll
-            for (int cc = 0; cc < 4; ++cc) a[cc & 1] = P::fma(W[cc], y[cc], a[cc & 1]);
+            for (int i = 0; i < 4 * C; ++i)
+                a[i & (2 / P::PACK - 1)] = P::vfma(VW[i / C * FACE + C * (NQ + p) + i % C], y[i], a[i & (2 / P::PACK - 1)]);
+            q[p * B] = q0 + P::value(P::normal(P::sum(P::PACK == 1 ? P::vadd(a[0], a[1]) : a[0])));
         }
-        q[it] = q0 + P::value(P::normal(P::add(a[0], a[1])));
     }
 }
 

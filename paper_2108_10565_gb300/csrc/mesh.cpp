@@ -454,22 +454,9 @@ void face_tables(int N, const std::vector<double>& mass, bool dw, std::vector<in
     face_traces(N, Pf, turn);
     const int32_t entries = face_turn_slots(N) + 6 * df;
     words.assign((size_t)4 * entries, 0);
-    int32_t at = entries;
-    auto put_entry = [&](double v, int c) {
-        int32_t w[4] = {0, 0, c, 0};
-        if (dw) {
-            const float h = (float)v, l = (float)(v - (double)h);
-            std::memcpy(&w[0], &h, 4);
-            std::memcpy(&w[1], &l, 4);
-        } else {
-            std::memcpy(w, &v, 8);
-        }
-        words.insert(words.end(), w, w + 4);
-        ++at;
-    };
     // rows in groups of `width` slots, longest first (so that a group's rows are
-    // of like length): a group's entries are step by step the next non-zero of
-    // each of its rows, zeros after a row's end, a multiple of 4 steps
+    // of like length): a group's steps are the next non-zero of each of its rows,
+    // zeros after a row's end
     auto put_rows = [&](int slot0, int slots, int width, bool sorted, const std::vector<std::vector<double>>& rows) {
         std::vector<std::vector<int>> cols(rows.size());
         std::vector<int> order(rows.size());
@@ -487,15 +474,29 @@ void face_tables(int N, const std::vector<double>& mass, bool dw, std::vector<in
             steps = (steps + 3) / 4 * 4;
             for (int r = 0; r < width; ++r) {
                 const int i = g * width + r;
-                const int32_t s[4] = {at, (int32_t)steps, i < (int)order.size() ? order[i] : -1, 0};
+                const int32_t s[4] = {(int32_t)(words.size() / 4), (int32_t)steps,
+                                      i < (int)order.size() ? order[i] : -1, 0};
                 std::memcpy(&words[(size_t)4 * (slot0 + i)], s, sizeof s);
             }
-            for (size_t n = 0; n < steps; ++n)
-                for (int r = 0; r < width; ++r) {
-                    const int i = g * width + r;
-                    const bool in = i < (int)order.size() && n < cols[order[i]].size();
-                    put_entry(in ? rows[order[i]][cols[order[i]][n]] : 0.0, in ? cols[order[i]][n] : 0);
-                }
+            for (size_t n0 = 0; n0 < steps; n0 += 4) {
+                const size_t at = words.size();
+                words.resize(at + 4 * (size_t)face_block_words(width), 0);
+                for (int r = 0; r < width; ++r)
+                    for (size_t n = 0; n < 4; ++n) {
+                        const int i = g * width + r;
+                        if (i >= (int)order.size() || n0 + n >= cols[order[i]].size()) continue;
+                        const int c = cols[order[i]][n0 + n];
+                        const double v = rows[order[i]][c];
+                        int32_t* to = &words[at + 4 * ((n / 2) * width + r) + 2 * (n % 2)];
+                        if (dw) {
+                            const float hl[2] = {(float)v, (float)(v - (double)(float)v)};
+                            std::memcpy(to, hl, sizeof hl);
+                        } else {
+                            std::memcpy(to, &v, sizeof v);
+                        }
+                        words[at + 8 * (size_t)width + r] |= c << 8 * n;
+                    }
+            }
         }
     };
     for (int f = 0; f < 4; ++f) {

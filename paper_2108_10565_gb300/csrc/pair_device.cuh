@@ -41,7 +41,50 @@ struct Bin64Base {
     __device__ static R select(bool c, R a, R b) { return c ? a : b; }
     __device__ static R normal(R a) { return a; }
     __device__ static uint32_t abs_bits(R a) { return (uint32_t)__double2hiint(a) & 0x7FFFFFFFu; }
+
+    // PACK values side by side
+    static constexpr int PACK = 1;
+    using V = double;
+    __device__ static V zeros() { return 0.0; }
+    __device__ static V all(R a) { return a; }
+    __device__ static V vmul(V a, V b) { return a * b; }
+    __device__ static V vfma(V a, V b, V c) { return ::fma(a, b, c); }
+    __device__ static V vadd(V a, V b) { return a + b; }
+    __device__ static V vsub(V a, V b) { return a - b; }
+    __device__ static R sum(V a) { return a; }
 };
+
+// the packed binary32 operations: one issue slot for two results
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ f32x2 pk_fma(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 pk_mul(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 pk_add(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// times -1, which is exact, stands for the sign modifier that the packed forms lack
+constexpr f32x2 MINUS_ONES = 0xBF800000BF800000ull;
+__device__ __forceinline__ f32x2 pk_neg(f32x2 a) { return pk_mul(a, MINUS_ONES); }
+__device__ __forceinline__ f32x2 pk_sub(f32x2 a, f32x2 b) { return pk_fma(b, MINUS_ONES, a); }
 
 // unevaluated sums (x, y) of two binary32 words, about 48 bits
 struct Bin32x2Base {
@@ -80,6 +123,36 @@ struct Bin32x2Base {
         return make_float2(s, e);
     }
     __device__ static uint32_t abs_bits(R a) { return __float_as_uint(a.x) & 0x7FFFFFFFu; }
+
+    // two values side by side, both high words, then both low ones; the same
+    // operations in the same order as above, bit for bit
+    static constexpr int PACK = 2;
+    struct __align__(16) V {
+        f32x2 h, l;
+    };
+    __device__ static V zeros() { return {0ull, 0ull}; }
+    __device__ static V all(R a) { return {pack2(a.x, a.x), pack2(a.y, a.y)}; }
+    __device__ static V vmul(V a, V b) {
+        const f32x2 p = pk_mul(a.h, b.h);
+        return {p, pk_fma(a.l, b.h, pk_fma(a.h, b.l, pk_fma(a.h, b.h, pk_neg(p))))};
+    }
+    __device__ static V vfma(V a, V b, V c) {
+        const f32x2 p = pk_mul(a.h, b.h);
+        const f32x2 e = pk_fma(a.l, b.h, pk_fma(a.h, b.l, pk_fma(a.h, b.h, pk_neg(p))));
+        const f32x2 s = pk_add(c.h, p), bb = pk_sub(s, c.h);
+        const f32x2 er = pk_add(pk_sub(c.h, pk_sub(s, bb)), pk_sub(p, bb));
+        return {s, pk_add(c.l, pk_add(er, e))};
+    }
+    __device__ static V vadd(V a, V b) {
+        const f32x2 s = pk_add(a.h, b.h), bb = pk_sub(s, a.h);
+        const f32x2 er = pk_add(pk_sub(a.h, pk_sub(s, bb)), pk_sub(b.h, bb));
+        return {s, pk_add(er, pk_add(a.l, b.l))};
+    }
+    __device__ static V vsub(V a, V b) { return vadd(a, {pk_neg(b.h), pk_neg(b.l)}); }
+    __device__ static R sum(V a) {
+        const float2 h = unpack2(a.h), l = unpack2(a.l);
+        return add(make_float2(h.x, l.x), make_float2(h.y, l.y));
+    }
 };
 
 }  // namespace poro

@@ -223,15 +223,17 @@ bool flux_factors(const poro_material& mL, const poro_material* mR, const double
 // normalised Dubiner basis of the reference triangle on each face (its vertices
 // in increasing local order); turn[6][df][df] with Fnb[f,h,s] = Pf[f]^T turn[s] Pf[h]
 void face_traces(int N, std::vector<double>& Pf, std::vector<double>& turn);
-// The corrector's table of 16-byte words: first the slots (first entry, steps, row;
+// The corrector's table of 16-byte words: first the slots (first word, steps, row;
 // row -1: none) of the traces, rows of Pf[f] in groups of 8, longest first; of
-// M^{-1} Pf^T, likewise; of the turns, one row each; then their entries (value as
-// binary64 or as (hi, lo) binary32, column), step by step for the rows of a group,
-// padded with zeros to a multiple of 4 steps.
+// M^{-1} Pf^T, likewise; of the turns, one row each; then their entries in blocks
+// of 4 steps of a group's rows, padded with zeros: the values of steps 0 and 1 (as
+// binary64 or (hi, lo) binary32), row by row, those of steps 2 and 3, and 4 columns
+// a row, a byte each.
 PORO_HD constexpr int face_modes(int N) { return (N + 1) * (N + 2) / 2; }
 PORO_HD constexpr int face_trace_slots(int) { return 0; }
 PORO_HD constexpr int face_back_slots(int N) { return 4 * ((face_modes(N) + 7) / 8) * 8; }
 PORO_HD constexpr int face_turn_slots(int N) { return face_back_slots(N) + 4 * ((n_modes(N) + 7) / 8) * 8; }
+PORO_HD constexpr int face_block_words(int width) { return 2 * width + (width + 3) / 4; }
 constexpr int FACE_FACTORS = 2 * 4 * NQ;  // V and W of one face
 void face_tables(int N, const std::vector<double>& mass, bool dw, std::vector<int32_t>& words);
 int face_permutation_index(const int p[3]);
