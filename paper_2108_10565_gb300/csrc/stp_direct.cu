@@ -253,21 +253,43 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 const R lo = P::shfl(b, lane - 1), hi = P::shfl(b, lane + 1);
                 return P::fma(z_hi, P::select(u == T - 1, b, hi), P::mul(z_lo, P::select(u == 0, b, lo)));
             };
-            // x: row q of Q; end: in lane u = 0 its value at the end of the step,
-            // Q~(1) = b_0 + (E* Q)_0 (the columns of Z^{-1} but the first sum to
-            // zero).  q0 may be the array written: its entries read by this task
-            // are the ones it writes.
-            auto put = [&](int q, R x, R end) {
+            // x: row q of Q; returns it in binary64
+            auto put = [&](int q, R x) {
                 x = P::normal(x);
+                const double v64 = P::value(x);
                 if (act) {
                     atomicMax(qmax + buf * PT + q * T + u, P::abs_bits(x));
                     c[q * T] = x;
-                    // outputs (global layout [p][l][u], dense) and the time integration
-                    const double v64 = P::value(x);
+                    // outputs (global layout [p][l][u], dense)
                     if (qo) qo[(q * B + m) * T + u] = v64;
-                    if (io && u == 0) io[q * B + m] = dt * v64;
                 }
-                if (qe && act && u == 0) qe[q * B + m] = P::value(P::normal(end));
+                return v64;
+            };
+            // the time integrals and Q~(1) of the task's rows, entry i in lane i of
+            // the group, from lane 0's value of the row and b_0 + (E* Q)_0 (the
+            // columns of Z^{-1} but the first sum to zero).  q0 may be the array
+            // written: its entries read by this task are the ones it writes.
+            auto finish = [&](auto row, const auto& v, const auto& end) {
+                constexpr int M = sizeof(v) / sizeof(double);
+#pragma unroll
+                for (int i = 0; i < M; i += T) {
+                    const bool mine = act && i + u < M;
+                    if (io) {
+                        double w = __shfl_sync(0xffffffffu, v[i], base);
+#pragma unroll
+                        for (int k = 1; k < T && i + k < M; ++k) {
+                            const double wk = __shfl_sync(0xffffffffu, v[i + k], base);
+                            w = u == k ? wk : w;
+                        }
+                        if (mine) io[row(i + u) * B + m] = dt * w;
+                    }
+                    if (qe) {
+                        R w = P::shfl(end[i], base);
+#pragma unroll
+                        for (int k = 1; k < T && i + k < M; ++k) w = P::select(u == k, P::shfl(end[i + k], base), w);
+                        if (mine) qe[row(i + u) * B + m] = P::value(P::normal(w));
+                    }
+                }
             };
             if (kind == 0) {
                 // normal stresses and pressure from D, Df, n_x u, n_y v
@@ -280,8 +302,9 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 const R b[4] = {rhs(q[0], 0, P::fma1(-2.f, gx, Lm)), rhs(q[1 / T], 1 % T, P::fma1(-2.f, gy, Lm)),
                                 rhs(q[2 / T], 2 % T, P::fma1(-2.f, gz, Lm)),
                                 rhs(q[3 / T], 3 % T, P::fma(iso[11], Df, P::mul(iso[10], D)))};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) put(i < 3 ? SXX + i : QP, plain(b[i]), b[i]);
+                const double v[4] = {put(SXX, plain(b[0])), put(SXX + 1, plain(b[1])), put(SXX + 2, plain(b[2])),
+                                     put(QP, plain(b[3]))};
+                finish([](int r) { return r < 3 ? SXX + r : QP; }, v, b);
             } else {
                 // one pair (u, u_f) of velocities and one shear stress
                 const int i = kind - 1;
@@ -296,9 +319,9 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 for (int s = 1; s < T; ++s) xf = P::fma(zuf[u * T + s], P::shfl(bf, base + s), xf);
                 xf = P::normal(xf);
                 const R by = P::fma(K[T * T + 1], xf, bu);  // + g Q_uf
-                put(SXY + i, plain(bs), bs);
-                put(QUF + i, xf, qe ? P::fma(K[T * T], xf, bf) : bf);
-                put(QU + i, plain(by), by);
+                const double v[3] = {put(QU + i, plain(by)), put(QUF + i, xf), put(SXY + i, plain(bs))};
+                const R end[3] = {by, P::fma(K[T * T], xf, bf), bs};
+                finish([i](int r) { return (r == 0 ? QU : r == 1 ? QUF : SXY) + i; }, v, end);
             }
         }
         __syncthreads();
