@@ -32,6 +32,7 @@
 // (N = 5, 6,000 elements: 3.54 -> 3.68 ms), so there a lane has one column.
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "pair_device.cuh"
 #include "poro_internal.h"
 
@@ -172,6 +173,8 @@ __global__ void __launch_bounds__(FaceShape<N>::NT, FaceShape<N>::MIN_BLOCKS)
         const V* g = reinterpret_cast<const V*>(D.fvw) + e * (int64_t)(FACE * 4);
         for (int i = tid; i < FACE * 4; i += NT) VW[i] = g[i];
     }
+    chain_wait();
+    if (chain_early(N)) chain_go();
     __syncthreads();
     // Y[k][c] = sum_p V[p][c] I[p][k] of both sides of every face
     for (int it = tid; it < 8 * B; it += NT) {
@@ -182,13 +185,13 @@ __global__ void __launch_bounds__(FaceShape<N>::NT, FaceShape<N>::MIN_BLOCKS)
         R v[NQ];
         if (sf < 4 || F.mode == 1) {
 #pragma unroll
-            for (int p = 0; p < NQ; ++p) v[p] = P::of(__ldg(I + p * B + k));
+            for (int p = 0; p < NQ; ++p) v[p] = P::of(I[p * B + k]);
         } else {
 #pragma unroll
             for (int p = 0; p < NQ; ++p) {
                 double a = 0.0;
 #pragma unroll
-                for (int s = 0; s < T; ++s) a = ::fma(__ldg(I + (p * B + k) * T + s), F.w[s], a);
+                for (int s = 0; s < T; ++s) a = ::fma(I[(p * B + k) * T + s], F.w[s], a);
                 v[p] = P::of(a);
             }
         }
@@ -260,6 +263,8 @@ template <bool BATCH>
 __global__ void __launch_bounds__(VNT) volume_kernel(int N, const CorrectorData D1, const int32_t* elems,
                                                      const CorrectorData* runs, const int32_t* item_run) {
     extern __shared__ double smv[];
+    chain_wait();
+    chain_go();
     const int B = n_modes(N), QB = NQ * B;
     double* I = smv;      // [13][B]
     double* X = I + QB;   // [13][B]
@@ -303,6 +308,8 @@ __global__ void __launch_bounds__(VNT) volume_kernel(int N, const CorrectorData 
 // at ticks that are multiples of 2^L
 __global__ void lts_buffer_kernel(int QB, int C, const int32_t* elems, int64_t count, const int32_t* slot,
                                   const double* iout, double* buf, int64_t tick) {
+    chain_wait();
+    chain_go();
     for (int64_t it = blockIdx.x; it < count; it += gridDim.x) {
         const int64_t e = elems[it];
         for (int L = 0; L < C; ++L) {
@@ -333,17 +340,29 @@ __device__ void add_source(int QB, const TickItem& it, int64_t k_add) {
     for (int i = threadIdx.x; i < QB; i += blockDim.x) q[i] += amp * it.vec[i];
 }
 
-__global__ void tick_advance_kernel(int64_t* tick, int64_t n) { *tick += n; }
+__global__ void tick_advance_kernel(int64_t* tick, int64_t n) {
+    chain_wait();
+    chain_go();
+    *tick += n;
+}
 
 __global__ void ticks_advance_kernel(int64_t* const* ticks, int count, int64_t n) {
+    chain_wait();
+    chain_go();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < count) *ticks[i] += n;
 }
 
 // one CTA per source item (of several runs), or one CTA for a run's list (its
 // sources may share an element)
-__global__ void source_items_kernel(int QB, const TickItem* items) { add_source(QB, items[blockIdx.x], 0); }
+__global__ void source_items_kernel(int QB, const TickItem* items) {
+    chain_wait();
+    chain_go();
+    add_source(QB, items[blockIdx.x], 0);
+}
 __global__ void source_list_kernel(int QB, const TickItem* items, int count, int64_t k_add) {
+    chain_wait();
+    chain_go();
     for (int i = 0; i < count; ++i) {
         add_source(QB, items[i], k_add);
         __syncthreads();
@@ -358,6 +377,8 @@ constexpr int RNT = 32 * NQ;
 __global__ void __launch_bounds__(RNT) receiver_items_kernel(int B, const TickItem* items) {
     const TickItem& it = items[blockIdx.x];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    chain_wait();
+    chain_go();
     const int32_t idx = *it.counter;
     const double* q = it.q + it.elem * (int64_t)(NQ * B) + warp * B;
     double acc = 0.0;
@@ -376,8 +397,7 @@ int launch_faces_p(const CorrectorData& d, const int32_t* elems, int64_t count, 
     auto* kern = runs ? face_kernel<N, P, true> : face_kernel<N, P, false>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BYTES);
     if (err != cudaSuccess) return (int)err;
-    kern<<<(unsigned)count, S::NT, S::SMEM_BYTES, (cudaStream_t)stream>>>(d, elems, runs, item_run);
-    return (int)cudaGetLastError();
+    return (int)launch_chained(kern, (unsigned)count, S::NT, S::SMEM_BYTES, stream, d, elems, runs, item_run);
 }
 
 template <int N>
@@ -395,8 +415,8 @@ int launch_corrector(const CorrectorData& d, bool volume, const int32_t* elems, 
     if (volume) {
         const size_t smem = sizeof(double) * 2 * NQ * n_modes(d.N);
         auto* kern = runs ? volume_kernel<true> : volume_kernel<false>;
-        kern<<<(unsigned)count, VNT, smem, (cudaStream_t)stream>>>(d.N, d, elems, runs, item_run);
-        if (const cudaError_t err = cudaGetLastError()) return (int)err;
+        if (const cudaError_t err = launch_chained(kern, (unsigned)count, VNT, smem, stream, d.N, d, elems, runs, item_run))
+            return (int)err;
     }
     switch (d.N) {
         case 1: return launch_faces_n<1>(d, elems, count, stream, runs, item_run);
@@ -413,38 +433,32 @@ int launch_lts_buffers(int N, int C, const int32_t* elems, int64_t count, const 
                        double* buf, int64_t tick, void* stream) {
     if (count <= 0) return 0;
     const int64_t grid = count < 65536 ? count : 65536;
-    lts_buffer_kernel<<<(unsigned)grid, 128, 0, (cudaStream_t)stream>>>(NQ * n_modes(N), C, elems, count, slot, iout,
-                                                                       buf, tick);
-    return (int)cudaGetLastError();
+    return (int)launch_chained(lts_buffer_kernel, (unsigned)grid, 128, 0, stream, NQ * n_modes(N), C, elems, count, slot,
+                               iout, buf, tick);
 }
 
 int launch_tick_sources(int N, const TickItem* items, int64_t count, void* stream) {
     if (count <= 0) return 0;
-    source_items_kernel<<<(unsigned)count, 256, 0, (cudaStream_t)stream>>>(NQ * n_modes(N), items);
-    return (int)cudaGetLastError();
+    return (int)launch_chained(source_items_kernel, (unsigned)count, 256, 0, stream, NQ * n_modes(N), items);
 }
 
 int launch_source_list(int N, const TickItem* items, int count, int64_t k_add, void* stream) {
     if (count <= 0) return 0;
-    source_list_kernel<<<1, 256, 0, (cudaStream_t)stream>>>(NQ * n_modes(N), items, count, k_add);
-    return (int)cudaGetLastError();
+    return (int)launch_chained(source_list_kernel, 1u, 256, 0, stream, NQ * n_modes(N), items, count, k_add);
 }
 
 int launch_tick_receivers(int N, const TickItem* items, int64_t count, void* stream) {
     if (count <= 0) return 0;
-    receiver_items_kernel<<<(unsigned)count, RNT, 0, (cudaStream_t)stream>>>(n_modes(N), items);
-    return (int)cudaGetLastError();
+    return (int)launch_chained(receiver_items_kernel, (unsigned)count, RNT, 0, stream, n_modes(N), items);
 }
 
 int launch_ticks_advance(int64_t* const* ticks, int count, int64_t n, void* stream) {
     if (count <= 0) return 0;
-    ticks_advance_kernel<<<(unsigned)((count + 127) / 128), 128, 0, (cudaStream_t)stream>>>(ticks, count, n);
-    return (int)cudaGetLastError();
+    return (int)launch_chained(ticks_advance_kernel, (unsigned)((count + 127) / 128), 128, 0, stream, ticks, count, n);
 }
 
 int launch_tick_advance(int64_t* tick, int64_t n, void* stream) {
-    tick_advance_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(tick, n);
-    return (int)cudaGetLastError();
+    return (int)launch_chained(tick_advance_kernel, 1u, 1, 0, stream, tick, n);
 }
 
 }  // namespace poro

@@ -40,6 +40,7 @@
 #include <set>
 #include <utility>
 
+#include "chain.cuh"
 #include "fixed_device.cuh"
 #include "pair_device.cuh"
 #include "poro_internal.h"
@@ -167,6 +168,8 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
     int* flag = si + S::I_FLAG;  // [0] non-finite value met, [1] the bounded wait gave up
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+    chain_wait();
+    if (chain_early(N)) chain_go();
     const int64_t it0 = blockIdx.x;
     const int64_t e = A.elems ? (int64_t)A.elems[it0] : it0;
     RunPtrs run{A.q0, A.econst, A.qt, A.iout, A.qend};
@@ -433,8 +436,7 @@ int launch_nt(const DirectParams& A, void* stream) {
     cudaError_t err = cudaFuncSetAttribute(stp_direct_kernel<N, NT_, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            S::SMEM_BYTES);
     if (err != cudaSuccess) return (int)err;
-    stp_direct_kernel<N, NT_, P><<<(unsigned)A.count, NT_, S::SMEM_BYTES, (cudaStream_t)stream>>>(A);
-    return (int)cudaGetLastError();
+    return (int)launch_chained(stp_direct_kernel<N, NT_, P>, (unsigned)A.count, NT_, S::SMEM_BYTES, stream, A);
 }
 
 // The default size is for launches that fill the chip several times over.  One
