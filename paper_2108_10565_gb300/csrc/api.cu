@@ -79,7 +79,8 @@ struct poro_ctx {
     std::vector<int32_t*> d_cl_elems;
     int32_t *d_cl = nullptr, *d_slot = nullptr;
     double* d_buf = nullptr;
-    std::vector<char> cl_has_slot;             // a cluster with elements that buffer for a larger neighbour
+    std::vector<int4*> d_cl_bufs;              // per cluster (element, slot, level) of its buffers
+    std::vector<int64_t> cl_bufs;              // their numbers
     bool use_graphs = true;
     int64_t* d_tick = nullptr;                 // device copy of the tick counter (graph replays)
     // persistent receiver buffers (no allocation in steady-state advances)
@@ -136,6 +137,8 @@ void free_mesh_device(poro_ctx* c) {
     c->sources.clear();
     for (auto& p : c->d_cl_elems) dfree(p);
     c->d_cl_elems.clear();
+    for (auto& p : c->d_cl_bufs) dfree(p);
+    c->d_cl_bufs.clear();
     dfree(c->d_cl);
     dfree(c->d_slot);
     dfree(c->d_buf);
@@ -1215,23 +1218,29 @@ poro_status poro_set_clusters(poro_ctx* c, double cfl_c, int32_t max_clusters, d
     for (int64_t e = 0; e < ne; ++e) c->cl_elems[c->h_cl[e]].push_back((int32_t)e);
     std::vector<int32_t> slot((size_t)ne * C, -1);
     int32_t nslot = 0;
-    c->cl_has_slot.assign(C, 0);
+    std::vector<std::vector<int4>> bufs(C);
     for (int64_t e = 0; e < ne; ++e)
         for (int f = 0; f < 4; ++f) {
             const int64_t r = c->h_nb[4 * e + f];
             if (r >= 0 && c->h_cl[r] > c->h_cl[e] && slot[e * C + c->h_cl[r]] < 0) {
+                bufs[c->h_cl[e]].push_back(make_int4((int)e, nslot, c->h_cl[r], 0));
                 slot[e * C + c->h_cl[r]] = nslot++;
-                c->cl_has_slot[c->h_cl[e]] = 1;
             }
         }
+    c->cl_bufs.clear();
     for (int k = 0; k < C; ++k) {
         int32_t* d = nullptr;
-        if (!c->cl_elems[k].empty() &&
-            (er = upload((void**)&d, c->cl_elems[k].data(), c->cl_elems[k].size() * sizeof(int32_t))) != cudaSuccess) {
+        int4* b = nullptr;
+        if (!c->cl_elems[k].empty())
+            er = upload((void**)&d, c->cl_elems[k].data(), c->cl_elems[k].size() * sizeof(int32_t));
+        c->d_cl_elems.push_back(d);
+        if (er == cudaSuccess && !bufs[k].empty()) er = upload((void**)&b, bufs[k].data(), bufs[k].size() * sizeof(int4));
+        c->d_cl_bufs.push_back(b);
+        c->cl_bufs.push_back((int64_t)bufs[k].size());
+        if (er != cudaSuccess) {
             free_population(c);
             return cuda_fail(c, er, "poro_set_clusters");
         }
-        c->d_cl_elems.push_back(d);
     }
     if (C > 1) {
         if ((er = upload((void**)&c->d_cl, c->h_cl.data(), ne * sizeof(int32_t))) != cudaSuccess ||
@@ -1359,8 +1368,8 @@ static int enqueue_tick(poro_ctx* c, int64_t k, unsigned what, cudaStream_t st,
                                         want_qt ? c->d_qt : nullptr, c->d_iout, in_place ? c->d_q0 : nullptr, st,
                                         c->variant);
         // (a cluster whose elements buffer for no larger neighbour has nothing to add)
-        if (rc == 0 && C > 1 && (what & TICK_BUFFERS) && c->cl_has_slot[cl])
-            rc = poro::launch_lts_buffers(c->N, C, el, cnt, c->d_slot, c->d_iout, c->d_buf, k, st);
+        if (rc == 0 && C > 1 && (what & TICK_BUFFERS))
+            rc = poro::launch_lts_buffers(c->N, c->d_cl_bufs[cl], c->cl_bufs[cl], c->d_iout, c->d_buf, k, st);
         if (rc == 0) rc = mark(prof, cl, false, st);
     }
     {

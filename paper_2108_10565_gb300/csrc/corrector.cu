@@ -304,23 +304,17 @@ __global__ void __launch_bounds__(VNT) volume_kernel(int N, const CorrectorData 
     }
 }
 
-// buffers of the sub-step integrals for larger neighbours: level L restarts
-// at ticks that are multiples of 2^L
-__global__ void lts_buffer_kernel(int QB, int C, const int32_t* elems, int64_t count, const int32_t* slot,
-                                  const double* iout, double* buf, int64_t tick) {
+// buffers of the sub-step integrals for larger neighbours, one CTA per buffer:
+// one of level L restarts at ticks that are multiples of 2^L.  (A CTA per element
+// of the cluster, most of them without a buffer, took 9 microseconds for 4,676.)
+__global__ void lts_buffer_kernel(int QB, const int4* items, const double* iout, double* buf, int64_t tick) {
+    const int4 it = items[blockIdx.x];
     chain_wait();
     chain_go();
-    for (int64_t it = blockIdx.x; it < count; it += gridDim.x) {
-        const int64_t e = elems[it];
-        for (int L = 0; L < C; ++L) {
-            const int sl = slot[e * C + L];
-            if (sl < 0) continue;
-            const bool reset = (tick & (((int64_t)1 << L) - 1)) == 0;
-            double* b = buf + (int64_t)sl * QB;
-            const double* I = iout + e * QB;
-            for (int i = threadIdx.x; i < QB; i += blockDim.x) b[i] = reset ? I[i] : b[i] + I[i];
-        }
-    }
+    const bool reset = (tick & (((int64_t)1 << it.z) - 1)) == 0;
+    const double* I = iout + (int64_t)it.x * QB;
+    double* b = buf + (int64_t)it.y * QB;
+    for (int i = threadIdx.x; i < QB; i += blockDim.x) b[i] = reset ? I[i] : b[i] + I[i];
 }
 
 // q[elem] += (S(t1) - S(t0)) vec over the step [(k+1-len) dt, (k+1) dt] with S the
@@ -429,12 +423,10 @@ int launch_corrector(const CorrectorData& d, bool volume, const int32_t* elems, 
     }
 }
 
-int launch_lts_buffers(int N, int C, const int32_t* elems, int64_t count, const int32_t* slot, const double* iout,
-                       double* buf, int64_t tick, void* stream) {
+int launch_lts_buffers(int N, const int4* items, int64_t count, const double* iout, double* buf, int64_t tick,
+                       void* stream) {
     if (count <= 0) return 0;
-    const int64_t grid = count < 65536 ? count : 65536;
-    return (int)launch_chained(lts_buffer_kernel, (unsigned)grid, 128, 0, stream, NQ * n_modes(N), C, elems, count, slot,
-                               iout, buf, tick);
+    return (int)launch_chained(lts_buffer_kernel, (unsigned)count, 128, 0, stream, NQ * n_modes(N), items, iout, buf, tick);
 }
 
 int launch_tick_sources(int N, const TickItem* items, int64_t count, void* stream) {

@@ -350,8 +350,9 @@ struct CorrectorData {
     const double* qt = nullptr;       // [ne][13][B][T] full predictors (larger neighbours)
     int64_t tick = 0;                 // tick k of the correction (interval ends at k + 1)
 };
-int launch_lts_buffers(int N, int C, const int32_t* elems, int64_t count, const int32_t* slot, const double* iout,
-                       double* buf, int64_t tick, void* stream);
+// one cluster's sub-step buffers, items (element, slot, level, -)
+int launch_lts_buffers(int N, const int4* items, int64_t count, const double* iout, double* buf, int64_t tick,
+                       void* stream);
 // The faces' part of the corrector; with `volume` first the volume and source
 // part (for a predictor that did not write Q~(1)).  `runs` (device array,
 // nullable) / `item_run`: a launch over several runs; item i is element
