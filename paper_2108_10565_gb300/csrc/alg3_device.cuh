@@ -116,9 +116,9 @@ struct SweepScratch {
     int2* X;
     int* w;              // I_WORDS
     const double* smax;  // [NNZ] max_j |star_j|
+    int* row;            // [NQ + 1] row starts of the star pattern
     __device__ uint32_t* qmax(int buf) const { return reinterpret_cast<uint32_t*>(w) + buf * S::PT; }
     __device__ int* scale() const { return w + S::I_SCALE; }
-    __device__ int* row() const { return w + S::I_ROW; }
 };
 // star[3][NNZ] into the directions of the integer Khat rows, and smax; entries
 // are a thread's own, so no barrier is needed inside
@@ -133,17 +133,22 @@ __device__ void adapt_star(double* star, double* smax) {
         smax[i] = fmax(fabs(s0), fmax(fabs(s1), fabs(s2)));
     }
 }
-// clears the maxima, fills the row starts and adapts the star (loaded before the
-// caller's last barrier); the caller's barrier follows
-template <int NT, class S, class Sys>
-__device__ void sweep_setup(const SweepScratch<S>& W, double* smax, double* star) {
-    for (int i = threadIdx.x; i < 2 * S::PT; i += NT) W.w[i] = 0;
+// fills the row starts and adapts the star (loaded before the caller's last
+// barrier); the caller's barrier follows
+template <int NT, class Sys>
+__device__ void star_setup(int* row, double* smax, double* star) {
     for (int i = threadIdx.x; i <= Sys::NQ; i += NT) {
         int n = 0;
         while (n < Sys::NNZ && Sys::row(n) < i) ++n;
-        W.row()[i] = n;
+        row[i] = n;
     }
     adapt_star<NT, Sys::NNZ>(star, smax);
+}
+// the same, and clears the maxima
+template <int NT, class S, class Sys>
+__device__ void sweep_setup(const SweepScratch<S>& W, double* smax, double* star) {
+    for (int i = threadIdx.x; i < 2 * S::PT; i += NT) W.w[i] = 0;
+    star_setup<NT, Sys>(W.row, smax, star);
 }
 
 // dst[p, l, u] += SIGN sum_j sum_m Khat^j[l, o_g + m] X^j[p, m, u] for l < o_g with
@@ -160,7 +165,7 @@ __device__ void khat_block(double* dst, const double* src, int g, const double* 
     for (int r = tid; r < PT; r += NT) {
         const int p = r / T, u = r - p * T;
         double b = 0.0;
-        for (int n = W.row()[p]; n < W.row()[p + 1]; ++n) b += W.smax[n] * bound_of(qmax[Sys::col(n) * T + u], 0.0);
+        for (int n = W.row[p]; n < W.row[p + 1]; ++n) b += W.smax[n] * bound_of(qmax[Sys::col(n) * T + u], 0.0);
         W.scale()[r] = row_scale(b);
         qmax_next[r] = 0u;
     }

@@ -181,11 +181,30 @@ bool visco_element_constants(const ReferenceData& ref, const double* v12, const 
 
 // ----- sub-cell material (setup.cpp, subcell.cu) -----
 // Per element, besides the mean-material constants (elem_const_stride
-// layout, from the mode-0 Jacobians): star_r[3][54] for the variation modes
-// r = 1..3 of the linearly interpolated Jacobians, then (e_r, g_r) of E*_r.
-constexpr int subcell_threads(int N) { return N >= 4 ? 256 : 128; }
+// layout, from the mode-0 Jacobians): dt grad xi_j on the pattern of the 13
+// primitive rows, [3][26], then for the variation modes r = 1..3 of the
+// linearly interpolated Jacobians their 9 entries k0..k8 in x-direction
+// (subcell.cu, combine_row) and (e_r, g_r) of E*_r.
+// (N = 3, 500 elements: 1.60 ms on 256 threads, 1.79 on 128; N = 4, where two CTAs
+// fit an SM, 3.73 on 256, 4.69 on 512; N = 6, 100 elements: 5.97 on 512, 6.95 on 256)
+constexpr int subcell_threads(int N) { return N >= 5 ? 512 : N >= 3 ? 256 : 128; }
 constexpr int subcell_columns(int N) { return N == 6 ? 30 : 3 * block_size(N); }
-PORO_HD constexpr int subcell_var_stride() { return (3 * 3 * STAR_NNZ + 6 + 1) & ~1; }
+constexpr int PRIM_NNZ = 26, SUBCELL_MODE = 11;
+PORO_HD constexpr int subcell_var_stride() { return (3 * PRIM_NNZ + 3 * SUBCELL_MODE + 1) & ~1; }
+// entry n of the primitive rows: row, quantity, component of n
+PORO_HD constexpr int prim_row(int n) {
+    constexpr int t[PRIM_NNZ] = {0, 0, 0, 1, 1, 1, 2, 3, 3, 4, 4, 5, 5, 6, 6, 6, 7, 7, 7, 8, 8, 8, 9, 10, 11, 12};
+    return t[n];
+}
+PORO_HD constexpr int prim_col(int n) {
+    constexpr int t[PRIM_NNZ] = {QU,  QV,  QW,  QUF, QVF, QWF, QU,  QU,  QV,  QV,  QW, QU, QW,
+                                 SXX, SXY, SXZ, SXY, SYY, SYZ, SXZ, SYZ, SZZ, QV,  QP, QP, QP};
+    return t[n];
+}
+PORO_HD constexpr int prim_dir(int n) {
+    constexpr int t[PRIM_NNZ] = {0, 1, 2, 0, 1, 2, 0, 1, 0, 2, 1, 2, 0, 0, 1, 2, 0, 1, 2, 0, 1, 2, 1, 0, 1, 2};
+    return t[n];
+}
 // Mh3_r = M^{-1} int phi_k phi_r phi_l, r = 1..3, as CSR over all rows k:
 // row pointers [3][B + 1] absolute into col / val (device)
 struct SubcellReference {

@@ -643,28 +643,26 @@ bool subcell_element_constants(const ReferenceData& ref, const double P[4][4], c
     const int T = ref.T;
     std::memset(mean_out, 0, sizeof(double) * elem_const_stride(ref.N));
     std::memset(var_out, 0, sizeof(double) * subcell_var_stride());
+    for (int j = 0; j < 3; ++j)
+        for (int n = 0; n < PRIM_NNZ; ++n) var_out[j * PRIM_NNZ + n] = dt * jinv[j][prim_dir(n)];
+    // modal coefficient r of an entry that is linear inside the element
+    auto modal = [&](int r, auto entry) {
+        double a = 0.0;
+        for (int v = 0; v < 4; ++v) a += P[r][v] * entry(v);
+        return a;
+    };
     double e[4], g[4];
     for (int r = 0; r < 4; ++r) {
-        double* star = r == 0 ? mean_out : var_out + (r - 1) * 3 * STAR_NNZ;
-        for (int j = 0; j < 3; ++j)
-            for (int n = 0; n < STAR_NNZ; ++n) {
-                const int p = star_row(n), q = star_col(n);
-                double s = 0.0;
-                for (int d = 0; d < 3; ++d) {
-                    double a = 0.0;
-                    for (int v = 0; v < 4; ++v) a += P[r][v] * abc[v][d][p][q];
-                    s += jinv[j][d] * a;
-                }
-                star[j * STAR_NNZ + n] = dt * s;
-            }
-        e[r] = g[r] = 0.0;
-        for (int v = 0; v < 4; ++v) {
-            e[r] += P[r][v] * E[v][QUF][QUF];
-            g[r] += P[r][v] * E[v][QU][QUF];
-        }
-        e[r] *= dt;
-        g[r] *= dt;
+        e[r] = dt * modal(r, [&](int v) { return E[v][QUF][QUF]; });
+        g[r] = dt * modal(r, [&](int v) { return E[v][QU][QUF]; });
     }
+    for (int j = 0; j < 3; ++j)
+        for (int n = 0; n < STAR_NNZ; ++n) {
+            double s = 0.0;
+            for (int d = 0; d < 3; ++d)
+                s += jinv[j][d] * modal(0, [&](int v) { return abc[v][d][star_row(n)][star_col(n)]; });
+            mean_out[j * STAR_NNZ + n] = dt * s;
+        }
     std::vector<double> zm(ref.z);
     for (int u = 0; u < T; ++u) zm[u * T + u] -= e[0];
     if (!invert_small(T, zm.data(), mean_out + ec_zinv(ref.N))) { err = "element: singular time block"; return false; }
@@ -672,9 +670,13 @@ bool subcell_element_constants(const ReferenceData& ref, const double P[4][4], c
     sc[0] = e[0];
     sc[1] = g[0];
     sc[2] = dt;
+    constexpr int entry[9][2] = {{SXY, QV}, {SYY, QU},   {SXX, QUF},  {QP, QU}, {QP, QUF},
+                                 {QU, SXX}, {QU, QP},    {QUF, SXX},  {QUF, QP}};
     for (int r = 1; r < 4; ++r) {
-        var_out[3 * 3 * STAR_NNZ + 2 * (r - 1)] = e[r];
-        var_out[3 * 3 * STAR_NNZ + 2 * (r - 1) + 1] = g[r];
+        double* k = var_out + 3 * PRIM_NNZ + (r - 1) * SUBCELL_MODE;
+        for (int i = 0; i < 9; ++i) k[i] = modal(r, [&](int v) { return abc[v][0][entry[i][0]][entry[i][1]]; });
+        k[9] = e[r];
+        k[10] = g[r];
     }
     return true;
 }

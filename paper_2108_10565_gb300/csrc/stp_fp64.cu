@@ -55,7 +55,8 @@ __global__ void __launch_bounds__(NT) stp_fp64_kernel(const SweepParams P) {
     double* star = sm + S::OFF_STAR;
     double* sc = sm + S::OFF_SC;
     double* smax = sm + S::OFF_MAX;
-    const SweepScratch<S> W{reinterpret_cast<int2*>(sm + S::OFF_X), reinterpret_cast<int*>(sm + S::OFF_I), smax};
+    int* ints = reinterpret_cast<int*>(sm + S::OFF_I);
+    const SweepScratch<S> W{reinterpret_cast<int2*>(sm + S::OFF_X), ints, smax, ints + S::I_ROW};
     const int tid = threadIdx.x;
     const int64_t e = blockIdx.x;
     // element constants: stars, shifted time matrices and scalars are contiguous

@@ -17,10 +17,20 @@
 // The contraction factor is about the relative variation of the material
 // inside the element.
 //
+// The three variation terms share their derivatives: isotropic Jacobians act
+// through 13 primitive rows of the geometry alone (those of stp_direct.cu, here with
+// n^j = dt grad xi_j), so W = sum_j Khat^j prim^j(Q_k) is formed once an iteration
+// and every mode's term is W combined with 9 of its Jacobians' entries.  That is 2
+// passes of Khat products (integer sums) an iteration, one over W and one in the
+// sweep, instead of 4, and 26 instead of 162 multiply-adds a mode, time mode and
+// direction for the variations.  N = 4, 500 elements: 3.90 -> 2.69 ms a pass.  What bounds
+// it: latency, of the sweep's small blocks and of the barriers between them (2
+// elements an SM at N = 4, 1 from N = 5 on).
+//
 // Shared memory: U (iterate), V (right-hand side, then the next iterate) and W
-// (one variation term) in the b / Q layout of the sweep, its fixed-point X (the
-// Khat products are integer sums, in the sweep and in the variation terms), the
-// mean element constants, the variation stars and the reduction words.
+// in the b / Q layout of the sweep, its fixed-point X (whose place takes a mode's
+// combined term in between), the mean element constants, those of the variation and
+// the reduction words.
 #include <cuda_runtime.h>
 
 #include "alg3_device.cuh"
@@ -31,7 +41,7 @@ namespace {
 struct SubParams {
     const double* q0;
     const double* econst;  // mean-material constants (the layout of the FP64 predictor)
-    const double* evar;    // per element: star_r[3][3][54] for r = 1..3, then (e_r, g_r) for r = 1..3
+    const double* evar;    // per element: dt grad xi_j on the primitive rows, 11 words per variation mode
     double* qt;
     double* iout;
     int32_t* iters;        // per element: iterations, negative if not converged
@@ -47,6 +57,13 @@ struct SubParams {
 
 constexpr int NVAR = 3;  // variation modes r = 1..3
 
+// the 13 primitive rows, in the form that khat_block takes
+struct Primitives {
+    static constexpr int NQ = poro::NQ, NNZ = PRIM_NNZ;
+    PORO_HD static constexpr int row(int n) { return prim_row(n); }
+    PORO_HD static constexpr int col(int n) { return prim_col(n); }
+};
+
 template <int N, int NT_>
 struct SubShape : SweepShape<N, BiotSystem, subcell_columns(N)> {
     using S = SweepShape<N, BiotSystem, subcell_columns(N)>;
@@ -56,33 +73,42 @@ struct SubShape : SweepShape<N, BiotSystem, subcell_columns(N)> {
     static constexpr int OFF_X = 3 * S::SQ;
     static constexpr int OFF_STAR = OFF_X + S::X_WORDS;            // mean constants: star, zuf, sc (EC words)
     static constexpr int EC = 3 * STAR_NNZ + S::T * S::T + 4;
-    static constexpr int OFF_VAR = OFF_STAR + EC;                   // variation stars and (e_r, g_r)
-    static constexpr int VAR = NVAR * 3 * STAR_NNZ + 2 * NVAR;
-    static constexpr int OFF_MAX = OFF_VAR + VAR;                   // max_j |star| of the mean, of the variations
-    static constexpr int OFF_RED = OFF_MAX + (1 + NVAR) * STAR_NNZ; // 2 NW reduction words
+    static constexpr int OFF_VAR = OFF_STAR + EC;                   // constants of the variation
+    static constexpr int VAR = 3 * PRIM_NNZ + NVAR * SUBCELL_MODE;
+    static constexpr int OFF_MAX = OFF_VAR + VAR;                   // max_j of the mean's star, of the primitives'
+    static constexpr int OFF_RED = OFF_MAX + STAR_NNZ + PRIM_NNZ;   // 2 NW reduction words
     static constexpr int OFF_I = OFF_RED + 2 * NW;
-    static constexpr int SMEM_BYTES = 8 * OFF_I + 4 * S::I_WORDS;
+    static constexpr int SMEM_BYTES = 8 * OFF_I + 4 * (S::I_WORDS + NQ + 1);
+    // rows of a combined term that X's place holds: all of them up to N = 5
+    static constexpr int CHUNK = S::X_WORDS / S::QS < NQ ? S::X_WORDS / S::QS : NQ;
+    static_assert(CHUNK >= 1, "room for a row of a combined term");
 };
 
-// W <- -E*_r U (source variation): u_f rows e_r U_uf, u rows g_r U_uf
-template <int NT, class S>
-__device__ void source_term(double* W, const double* U, double e, double g) {
-    constexpr int QS = S::QS, BT = S::B * S::T;
-    for (int i = threadIdx.x; i < NQ * BT; i += NT) {
-        const int p = i / BT, m = i - p * BT;
-        double v = 0.0;
-        if (p >= QUF) v = -e * U[p * QS + m];
-        else if (p >= QU && p <= QW) v = -g * U[(p + QUF - QU) * QS + m];
-        W[p * QS + m] = v;
+// row p of sum_j Khat^j A^{j*}_r U - E*_r U at one (mode, time mode), from the
+// primitive sums w and the iterate u (both [13], stride QS), with the
+// x-direction entries k of the Jacobians and k[9] = e, k[10] = g of E*
+template <int QS>
+__device__ __forceinline__ double combine_row(int p, const double* w, const double* u, const double* k) {
+    const double D = w[0], Df = w[QS];
+    if (p <= SZZ) {  // normal stresses: k1 D + k2 Df + 2 k0 n_p u_p
+        const double gx = w[2 * QS], gy = w[9 * QS];
+        const double gp = p == SXX ? gx : p == SYY ? gy : D - gx - gy;
+        return fma(2.0 * k[0], gp, fma(k[2], Df, k[1] * D));
     }
+    if (p < QU) return k[0] * w[p * QS];
+    if (p == QP) return fma(k[4], Df, k[3] * D);
+    const int i = p < QP ? p - QU : p - QUF;
+    const double Sg = w[(QU + i) * QS], G = w[(QUF + i) * QS], f = u[(QUF + i) * QS];
+    return p < QP ? fma(-k[10], f, fma(k[6], G, k[5] * Sg)) : fma(-k[9], f, fma(k[8], G, k[7] * Sg));
 }
 
-// W += sum_j Khat^j (A^{j*}_r U) over all degree blocks (strictly upper in
-// degree: rows l < o_g take column block g); begins after and ends with a barrier
+// W = sum_j Khat^j prim^j(U) over all degree blocks (strictly upper in degree:
+// rows l < o_g take column block g); begins after and ends with a barrier
 template <int N, int NT, class S>
-__device__ void flux_term(double* W, const double* U, const double* starr, const KhatRows& K, const SweepScratch<S>& X) {
+__device__ void flux_term(double* W, const double* U, const double* prim, const KhatRows& K, const SweepScratch<S>& X) {
     constexpr int T = S::T;
     const int32_t* list = K.list;
+    for (int i = threadIdx.x; i < S::SQ; i += NT) W[i] = 0.0;
 #pragma unroll 1
     for (int g = N; g >= 1; --g) {
         const int o = block_offset(g), d = block_size(g);
@@ -91,16 +117,18 @@ __device__ void flux_term(double* W, const double* U, const double* starr, const
             atomicMax(X.qmax(0) + q * T + mu % T, (uint32_t)__double2hiint(U[q * S::QS + o * T + mu]) & 0x7FFFFFFFu);
         }
         __syncthreads();
-        khat_block<N, NT, BiotSystem, S, 1>(W, U, g, starr, K, list, X, X.qmax(0), X.qmax(1));
+        khat_block<N, NT, Primitives, S, 1>(W, U, g, prim, K, list, X, X.qmax(0), X.qmax(1));
         for (int i = threadIdx.x; i < S::PT; i += NT) X.qmax(0)[i] = 0u;
         __syncthreads();
     }
 }
 
-// V -= Mh3_r W (all rows k); ends with a barrier
-template <int NT, class S>
-__device__ void mass_term(double* V, const double* W, const int32_t* row, const int32_t* col, const double* val) {
-    constexpr int B = S::B, T = S::T, QS = S::QS, PT = S::PT, PUL = S::PUL, NW = NT / 32;
+// V -= Mh3_r W for the rows [p0, p0 + np) of quantities, W their place; ends with
+// a barrier
+template <int NT, class S, int CHUNK>
+__device__ void mass_term(double* V, const double* W, int p0, int np, const int32_t* row, const int32_t* col,
+                          const double* val) {
+    constexpr int B = S::B, T = S::T, QS = S::QS, PUL = (CHUNK * T + 31) / 32, NW = NT / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int k = warp; k < B; k += NW) {
         const int n0 = __ldg(row + k), n1 = __ldg(row + k + 1);
@@ -113,13 +141,13 @@ __device__ void mass_term(double* V, const double* W, const int32_t* row, const 
 #pragma unroll
             for (int q = 0; q < PUL; ++q) {
                 const int pu = lane + 32 * q;
-                if (pu < PT) acc[q] = fma(v, W[(pu / T) * QS + l + pu % T], acc[q]);
+                if (pu < np * T) acc[q] = fma(v, W[(pu / T) * QS + l + pu % T], acc[q]);
             }
         }
 #pragma unroll
         for (int q = 0; q < PUL; ++q) {
             const int pu = lane + 32 * q;
-            if (pu < PT) V[(pu / T) * QS + k * T + pu % T] -= acc[q];
+            if (pu < np * T) V[(p0 + pu / T) * QS + k * T + pu % T] -= acc[q];
         }
     }
     __syncthreads();
@@ -139,7 +167,10 @@ __global__ void __launch_bounds__(NT_) stp_subcell_kernel(const SubParams P) {
     double* smax = sm + S::OFF_MAX;
     double* red = sm + S::OFF_RED;
     using Sweep = typename S::S;
-    const SweepScratch<Sweep> X{reinterpret_cast<int2*>(sm + S::OFF_X), reinterpret_cast<int*>(sm + S::OFF_I), smax};
+    int* ints = reinterpret_cast<int*>(sm + S::OFF_I);
+    const SweepScratch<Sweep> X{reinterpret_cast<int2*>(sm + S::OFF_X), ints, smax, ints + S::I_ROW};
+    const SweepScratch<Sweep> Xp{X.X, ints, smax + STAR_NNZ, ints + S::I_WORDS};
+    double* term = sm + S::OFF_X;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     for (int64_t e = blockIdx.x; e < P.count; e += gridDim.x) {
@@ -153,8 +184,7 @@ __global__ void __launch_bounds__(NT_) stp_subcell_kernel(const SubParams P) {
         init_rhs<NT, Sweep>(U, q0);
         __syncthreads();
         sweep_setup<NT, Sweep, BiotSystem>(X, smax, star);
-        for (int r = 0; r < NVAR; ++r)
-            adapt_star<NT, STAR_NNZ>(var + r * 3 * STAR_NNZ, smax + (1 + r) * STAR_NNZ);
+        star_setup<NT, Primitives>(Xp.row, smax + STAR_NNZ, var);
         __syncthreads();
         alg3_sweep<N, NT, BiotSystem, Sweep>(U, star, zuf, sc[1], P.khat, X);  // Q_0 = Y_0^{-1} b0
         int it = 0;
@@ -162,14 +192,18 @@ __global__ void __launch_bounds__(NT_) stp_subcell_kernel(const SubParams P) {
         while (it < P.max_iter && !stop) {
             ++it;
             init_rhs<NT, Sweep>(V, q0);
-            for (int r = 0; r < NVAR; ++r) {
-                source_term<NT, Sweep>(W, U, var[NVAR * 3 * STAR_NNZ + 2 * r], var[NVAR * 3 * STAR_NNZ + 2 * r + 1]);
-                __syncthreads();
-                SweepScratch<Sweep> Xr = X;
-                Xr.smax = smax + (1 + r) * STAR_NNZ;
-                flux_term<N, NT, Sweep>(W, U, var + r * 3 * STAR_NNZ, P.khat, Xr);
-                mass_term<NT, Sweep>(V, W, P.m3_row + r * (B + 1), P.m3_col, P.m3_val);
-            }
+            flux_term<N, NT, Sweep>(W, U, var, P.khat, Xp);
+            for (int r = 0; r < NVAR; ++r)
+                for (int p0 = 0; p0 < NQ; p0 += S::CHUNK) {
+                    const int np = min(S::CHUNK, NQ - p0);
+                    const double* kr = var + 3 * PRIM_NNZ + r * SUBCELL_MODE;
+                    for (int i = tid; i < np * BT; i += NT) {
+                        const int p = i / BT, m = i - p * BT;
+                        term[p * QS + m] = combine_row<QS>(p0 + p, W + m, U + m, kr);
+                    }
+                    __syncthreads();
+                    mass_term<NT, Sweep, S::CHUNK>(V, term, p0, np, P.m3_row + r * (B + 1), P.m3_col, P.m3_val);
+                }
             alg3_sweep<N, NT, BiotSystem, Sweep>(V, star, zuf, sc[1], P.khat, X);  // Q_{k+1}
             // max |Q_{k+1} - Q_k| and max |Q_{k+1}| over the element
             double dmax = 0.0, vmax = 0.0;
