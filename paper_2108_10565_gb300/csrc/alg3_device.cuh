@@ -85,8 +85,6 @@ struct Alg3Shape {
     static constexpr int QBT = NQ_ * B * T;                // dense size (global layout)
     static constexpr int QS = bank_stride(B * T, T);       // shared quantity stride
     static constexpr int SQ = NQ_ * QS;                    // shared size of b / Q
-    static constexpr int DMAX = block_size(N);
-    static constexpr int XSMAX = bank_stride(DMAX * T, T);
     static constexpr int PT = NQ_ * T;                     // (p, u) pairs of one mode
     static constexpr int PUL = (PT + 31) / 32;             // pairs per lane
 };

@@ -27,18 +27,6 @@ __device__ __forceinline__ void dw_mac(float& h, float& l, float ah, float al, f
     l = __fadd_rn(l, __fadd_rn(er, e));
 }
 
-// acc += a * b with b a single binary32 word
-__device__ __forceinline__ void dw_mac1(float& h, float& l, float ah, float al, float b) {
-    const float p = __fmul_rn(ah, b);
-    float e = __fmaf_rn(ah, b, -p);
-    e = __fmaf_rn(al, b, e);
-    const float s = __fadd_rn(h, p);
-    const float bb = __fsub_rn(s, h);
-    const float er = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    h = s;
-    l = __fadd_rn(l, __fadd_rn(er, e));
-}
-
 // acc += a * (bh + bl) with a exact
 __device__ __forceinline__ void dw_mac_x2(float& h, float& l, float a, float bh, float bl) {
     const float p = __fmul_rn(a, bh);
@@ -97,15 +85,6 @@ __device__ __forceinline__ float2 dw_split(double x) {
     return make_float2(h, (float)(x - (double)h));
 }
 
-// a + b for two double-word values
-__device__ __forceinline__ float2 dw_add(float2 a, float2 b) {
-    float s, e;
-    two_sum(a.x, b.x, s, e);
-    e = __fadd_rn(e, __fadd_rn(a.y, b.y));
-    const float h = __fadd_rn(s, e);
-    return make_float2(h, __fsub_rn(e, __fsub_rn(h, s)));
-}
-
 // ------------------------------------------------------- fixed-point words
 // 2^k as binary32, k in [-126, 127]
 __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) << 23); }
@@ -116,29 +95,6 @@ __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) 
 // constant is subtracted (exact by Sterbenz's lemma)
 __device__ __forceinline__ float small_int_to_float(int v) {
     return __fsub_rn(__int_as_float(0x4B400000 + v), 12582912.0f);
-}
-
-// nearest integer to x * f for |x * f| < 2^22 and f a power of two: the
-// exact product is rounded to the unit last place of 1.5 * 2^23 (a sum that
-// rounds up to 2^24 gives the pattern of 2^24, i.e. v = 2^22)
-__device__ __forceinline__ int round_to_int(float x, float f) {
-    return __float_as_int(__fmaf_rn(x, f, 12582912.0f)) - 0x4B400000;
-}
-
-// exact double-word (h, l) of an integer |v| <= 2^44: v = a 2^22 + b with
-// |a| <= 2^22 and b in [0, 2^22), both exact in binary32, joined by Fast2Sum
-// (|a 2^22| > b unless a = 0)
-__device__ __forceinline__ void int_to_dw(long long v, float& h, float& l) {
-    const float fa = __fmul_rn(small_int_to_float((int)(v >> 22)), 4194304.0f);
-    const float fb = small_int_to_float((int)(v & 0x3FFFFF));
-    h = __fadd_rn(fa, fb);
-    l = __fsub_rn(fb, __fsub_rn(h, fa));
-}
-__device__ __forceinline__ void int_to_dw(int v, float& h, float& l) {
-    const float fa = __fmul_rn(small_int_to_float(v >> 22), 4194304.0f);
-    const float fb = small_int_to_float(v & 0x3FFFFF);
-    h = __fadd_rn(fa, fb);
-    l = __fsub_rn(fb, __fsub_rn(h, fa));
 }
 
 }  // namespace poro

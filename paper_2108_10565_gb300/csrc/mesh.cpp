@@ -519,39 +519,6 @@ void face_tables(int N, const std::vector<double>& mass, bool dw, std::vector<in
     }
 }
 
-void face_matrices(int N, std::vector<double>& Floc, std::vector<double>& Fnb) {
-    const int B = n_modes(N);
-    std::vector<double> qa, qb, qw;
-    triangle_rule(N, qa, qb, qw);
-    const int nq = (int)qw.size();
-    Floc.assign((size_t)4 * B * B, 0.0);
-    Fnb.assign((size_t)4 * 4 * 6 * B * B, 0.0);
-    std::vector<double> phL(B), phR(B);
-    for (int q = 0; q < nq; ++q) {
-        const double lam[3] = {1 - qa[q] - qb[q], qa[q], qb[q]};
-        for (int f = 0; f < 4; ++f) {
-            double xi[3];
-            face_point(f, lam, xi);
-            basis_at(N, xi, phL.data());
-            double* Fl = Floc.data() + (size_t)f * B * B;
-            for (int k = 0; k < B; ++k)
-                for (int l = 0; l < B; ++l) Fl[k * B + l] += qw[q] * phL[k] * phL[l];
-            for (int h = 0; h < 4; ++h)
-                for (int s = 0; s < 6; ++s) {
-                    // local face vertex i sits on neighbour face vertex PERM[s][i]
-                    double mu[3];
-                    for (int i = 0; i < 3; ++i) mu[PERM[s][i]] = lam[i];
-                    double xr[3];
-                    face_point(h, mu, xr);
-                    basis_at(N, xr, phR.data());
-                    double* Fn = Fnb.data() + (((size_t)f * 4 + h) * 6 + s) * B * B;
-                    for (int k = 0; k < B; ++k)
-                        for (int l = 0; l < B; ++l) Fn[k * B + l] += qw[q] * phL[k] * phR[l];
-                }
-        }
-    }
-}
-
 int face_permutation_index(const int p[3]) {
     for (int s = 0; s < 6; ++s)
         if (PERM[s][0] == p[0] && PERM[s][1] == p[1] && PERM[s][2] == p[2]) return s;

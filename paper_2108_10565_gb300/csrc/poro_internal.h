@@ -231,16 +231,14 @@ bool flux_solver(const poro_material& mL, const poro_material* mR, const double 
                  double* Fp, std::string& err);
 // phi_l(xi) for all l (singularity-free homogenised recurrences)
 void basis_at(int N, const double xi[3], double* phi);
-// Floc[4][B][B] = int_face phi_k phi_l, Fnb[4][4][6][B][B] = int_face phi_k(L) phi_l(R)
-// for local face f, neighbour face h, vertex permutation s
-void face_matrices(int N, std::vector<double>& Floc, std::vector<double>& Fnb);
-// the same face in factors: A_n^L - F^- = W V (every kind) and, on interior
+// one face in factors: A_n^L - F^- = W V (every kind) and, on interior
 // faces, F^+ = W V; V and W as [13][4]
 bool flux_factors(const poro_material& mL, const poro_material* mR, const double n[3], int kind, double* V, double* W,
                   std::string& err);
-// Pf[4][df][B] with Floc[f] = Pf^T Pf, df = (N+1)(N+2)/2: traces in the
-// normalised Dubiner basis of the reference triangle on each face (its vertices
-// in increasing local order); turn[6][df][df] with Fnb[f,h,s] = Pf[f]^T turn[s] Pf[h]
+// Pf[4][df][B], df = (N+1)(N+2)/2: traces in the normalised Dubiner basis of the
+// reference triangle on each face (its vertices in increasing local order), so
+// that int_face f phi_k phi_l is Pf^T Pf; turn[6][df][df]: with the neighbour's
+// trace on its face h under vertex permutation s, Pf[f]^T turn[s] Pf[h]
 void face_traces(int N, std::vector<double>& Pf, std::vector<double>& turn);
 // The corrector's table of 16-byte words: first the slots (first word, steps, row;
 // row -1: none) of the traces, rows of Pf[f] in groups of 8, longest first; of
