@@ -311,17 +311,17 @@ def run_reference(args):
 
 
 # ------------------------------------------------------------------ our arm
-# Issue cost of the refinement residual, in instruction slots of the 128-lane
-# binary32 rate: its Khat and time-matrix products are exact integer
-# multiply-adds (IMAD at half the binary32 rate: 2 slots); its star, E* and
-# coupling products are double-word multiply-adds of 12 binary32 instructions.
-INT_MAC_SLOTS = 2.0
+# Issue cost of the double-binary32 kernel, in instruction slots of the 128-lane
+# binary32 rate: a 32 x 32 + 64 bit integer multiply-add (measured at 13 to 19
+# lanes a clock and SM, here 16) and a double-word multiply-add of 12 binary32
+# instructions.
+WIDE_MAC_SLOTS = 8.0
 DW_OPS_PER_MAC = 12.0
 # DRAM bytes (read + write) per element of the headline kernels at N = 6, from
 # one ncu capture each of the 20,000-element case (dram__bytes_read.sum +
 # dram__bytes_write.sum divided by the elements); the traffic grows in
 # proportion to the elements, so a launch of n elements moves n times this
-TRAFFIC_BYTES_PER_ELEMENT = {("mixed", 6, 1): 77336.0, ("mixed_bf16", 6, 1): 77169.0, ("fp64", 6, None): 77491.0}
+TRAFFIC_BYTES_PER_ELEMENT = {("mixed", 6, 1): 76347.0, ("fp64", 6, None): 76394.0}
 # nominal tf32 : bf16 dense tensor ratio (1.1 : 2.25 PFLOP/s)
 TF32_PER_BF16 = 1.1 / 2.25
 
@@ -338,6 +338,18 @@ def tc_tile_flops(N, bf16=False):
         kpad = (d + 15) // 16 * 16 if bf16 else (d + 7) // 8 * 8
         tot += 3 * 3 * 2 * 128 * npad * kpad
     return tot
+
+
+def direct_work(N):
+    """Work of one element in the predictor kernel (Biot), in lane operations:
+    `arith` multiplies and multiply-adds in the kernel's arithmetic (25 a
+    direction, mode of degree >= 1 and time mode for the star products, 57 + 3 T
+    a mode and time mode for the time solves, one per row that a degree block's
+    Khat sums reach), and `int_macs` entries of the integer Khat rows."""
+    B, T = (N + 1) * (N + 2) * (N + 3) // 6, N + 1
+    nnz = {1: 4, 2: 29, 3: 119, 4: 364, 5: 924, 6: 2058}[N]
+    rows = sum(-(-((g + 1) * (g + 2) // 2) // 21) * (g * (g + 1) * (g + 2) // 6) for g in range(1, N + 1))
+    return {"arith": 75 * (B - 1) * T + (57 + 3 * T) * B * T + 13 * T * rows, "int_macs": 13 * T * nnz}
 
 
 def fp32_alu_peak_tflops(sm_mhz):
@@ -929,74 +941,69 @@ def run_ours(args):
 
     def roofline(name):
         """Roofline of one form's kernel against the measured peaks
-        (MEASURED_PEAKS.json): HBM copy bandwidth and dense bf16 tensor
-        throughput (tf32 = bf16 x the nominal tf32 : bf16 ratio).  `frac` is
-        the largest fraction over those roofs and `bound` names it; the
-        binary64 kernel, which neither roof bounds, reports its FP64 pipe
-        against the nominal unit count x the sampled clock.  `model` keeps the
-        kernel's own issue-slot model apart from these."""
+        (MEASURED_PEAKS.json): HBM copy bandwidth and, for the unrefined
+        form, dense bf16 tensor throughput (tf32 = bf16 x the nominal
+        tf32 : bf16 ratio).  `frac` is the largest fraction over those roofs
+        and `bound` names it; the binary64 kernel, which neither roof bounds,
+        reports its FP64 pipe against the nominal unit count x the sampled
+        clock.  `model` keeps the double-binary32 kernel's own issue-slot model
+        apart from these."""
         r = res[name]
         mhz = (r["clocks"] or {}).get("sm_mhz") or 2070.0
         t = statistics.mean(r["per"]) * 1e-3
         Bm, Tm = (N + 1) * (N + 2) * (N + 3) // 6, N + 1
-        stride = (3 * 54 + Tm * Tm + 4 + 1) & ~1
-        alg_bytes = 8.0 * (13 * Bm + stride + 13 * Bm * Tm + 13 * Bm)  # Q0, constants in; Qt, I out
+        # Q0 and the element's (Z - e I)^{-1}, 3 scalars and 15 star factors in; Qt, I out
+        alg_bytes = 8.0 * (13 * Bm + Tm * Tm + 18 + 13 * Bm * Tm + 13 * Bm)
         hbm_ach = alg_bytes * n / t / 1e9
         terms = {"hbm": {"achieved": hbm_ach, "peak": hbm_gbs, "unit": "GB/s", "frac": hbm_ach / hbm_gbs,
                          "algorithmic_bytes_per_element": alg_bytes}}
-        if r["prec"] == L.PORO_FP64:
-            ach = r["flops"][0] * n / t / 1e12
+        work = direct_work(N)
+        if r["prec"] == L.PORO_FP64 or r["sweeps"] == 2:  # binary64 arithmetic, Khat sums in integers
+            ach = 2.0 * work["arith"] * n / t / 1e12
             peak = fp64_alu_peak_tflops(mhz)
             tb = TRAFFIC_BYTES_PER_ELEMENT.get(("fp64", N, None))
             terms["fp64_pipe"] = {"achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak}
             return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                    "traffic": tb * n if tb else None, "kernel": f"stp_fp64_kernel<{N}>",
-                    "flops_per_element": r["flops"][0], "terms": terms,
+                    "traffic": tb * n if tb else None, "kernel": f"stp_direct_kernel<{N},Bin64>",
+                    "binary64_operations_per_element": work["arith"],
+                    "integer_multiply_adds_per_element": 2 * work["int_macs"],
+                    "algorithmic_flops_per_element": r["flops"][0], "terms": terms,
                     "peak_source": "binary64 FMA pipe, nominal (152 SM x 2 FMA/clk x 2 flop x 2.07 GHz = 1.25 "
-                                   "TFLOP/s) scaled to the sampled clock; no measured FP64 peak exists"}
-        # the Khat products of the sweeps on the tensor cores: dense degree
-        # blocks (o_g rows x d_g columns, 13 T right-hand columns, 3
-        # directions), 3 split products, per sweep (algorithmic); the tiles as
-        # issued pad rows to 128 and columns to the MMA shape
+                                   "TFLOP/s) scaled to the sampled clock; no measured FP64 peak exists; the Khat "
+                                   "products are integer sums and not counted"}
+        if r["sweeps"] == 1:  # double-binary32 on the binary32 and integer pipes
+            b = terms["hbm"]
+            slots = {"double_word": DW_OPS_PER_MAC * work["arith"], "integer": (WIDE_MAC_SLOTS + 1) * work["int_macs"]}
+            t_alu = sum(slots.values()) * n / (152 * 128 * mhz * 1e6)
+            tb = TRAFFIC_BYTES_PER_ELEMENT.get(("mixed", N, 1))
+            return {"bound": "hbm", "achieved": b["achieved"], "peak": b["peak"], "unit": b["unit"], "frac": b["frac"],
+                    "traffic": tb * n if tb else None, "kernel": f"stp_direct_kernel<{N},Bin32x2>",
+                    "peak_source": peaks_src + " (hbm_gbs)", "terms": terms,
+                    "model": {"frac": t_alu / t, "bound_times_ms": {"binary32_issue": 1e3 * t_alu},
+                              "slots_per_element": slots,
+                              "derivation": f"issue at 152 SM x 128 lanes x {mhz:.0f} MHz: {DW_OPS_PER_MAC:g} slots per "
+                                            f"double-word operation, {WIDE_MAC_SLOTS:g} + 1 per entry of the integer "
+                                            "Khat rows; the kernel's own instruction mix, not a hardware roof"}}
+        # the unrefined form: one binary32 sweep with its Khat products on the
+        # tensor cores, dense degree blocks (o_g rows x d_g columns, 13 T
+        # right-hand columns, 3 directions), 3 split products (algorithmic); the
+        # tiles as issued pad rows to 128 and columns to the MMA shape
         bf = r["prec"] == L.PORO_BF16X3_REFINE
-        sw = 1 + r["sweeps"]
         tc_alg = sum(3 * (g * (g + 1) * (g + 2) // 6) * ((g + 1) * (g + 2) // 2) * 13 * Tm * 2 * 3
-                     for g in range(1, N + 1)) * sw
+                     for g in range(1, N + 1))
         tc_peak = tensor_bf16_burst * (1.0 if bf else TF32_PER_BF16)
         tc_ach = tc_alg * n / t / 1e12
         terms["tensor"] = {"achieved": tc_ach, "peak": tc_peak, "unit": "TFLOP/s", "frac": tc_ach / tc_peak,
                            "dtype": "bf16" if bf else "tf32",
                            "peak_source": "measured bf16 burst" + ("" if bf else f" x {TF32_PER_BF16:.3f}"),
                            "algorithmic_flops_per_element": tc_alg,
-                           "issued_flops_per_element": tc_tile_flops(N, bf) * sw}
+                           "issued_flops_per_element": tc_tile_flops(N, bf)}
         bound = max(("hbm", "tensor"), key=lambda k: terms[k]["frac"])
         b = terms[bound]
-        # the kernel's own issue model (not a hardware roof): binary32 pipe
-        # at 152 x 128 lanes per clock, 1 slot per FMA, INT_MAC_SLOTS per
-        # integer MAC, DW_OPS_PER_MAC per double-word MAC, overlapped with the
-        # issued tensor tiles
-        s3 = 2.0 * 13 * Bm * Tm * Tm + 2.0 * 3 * Bm * Tm
-        s4a = 2.0 * 3 * 54 * (Bm - 1) * Tm
-        s15 = 13 * Bm * Tm + 13 * Bm
-        s4b = r["flops"][0] - (s3 + s4a + s15)
-        f_alu = (s3 + s4a + s15) * sw
-        int_macs = (s4b / 2 + 13 * Bm * Tm * Tm) * r["sweeps"]
-        dw_macs = (6 * Bm * Tm + 3 * 54 * Bm * Tm) * r["sweeps"]
-        t_alu = (f_alu / 2 + INT_MAC_SLOTS * int_macs + DW_OPS_PER_MAC * dw_macs) * n / (152 * 128 * mhz * 1e6)
-        t_tc = tc_tile_flops(N, bf) * sw * n / (tc_peak * 1e12)
-        tb = TRAFFIC_BYTES_PER_ELEMENT.get(("mixed_bf16" if bf else "mixed", N, r["sweeps"]))
         return {"bound": bound, "achieved": b["achieved"], "peak": b["peak"], "unit": b["unit"], "frac": b["frac"],
-                "traffic": tb * n if tb else None,
-                "kernel": f"stp_mixed_kernel<{N},{r['sweeps']}" + (",bf16>" if bf else ">"),
+                "traffic": None, "kernel": f"stp_mixed_kernel<{N}" + (",bf16>" if bf else ">"),
                 "peak_source": peaks_src + " (" + ("hbm_gbs" if bound == "hbm" else "bf16_tflops burst") + ")",
-                "terms": terms,
-                "model": {"frac": max(t_alu, t_tc) / t, "bound_times_ms": {"binary32_issue": 1e3 * t_alu,
-                                                                           "tensor_tiles": 1e3 * t_tc},
-                          "residual_macs_per_element": {"integer": int_macs, "double_word": dw_macs},
-                          "derivation": f"binary32 pipe issue at 152 SM x 128 lanes x {mhz:.0f} MHz: 1 slot per "
-                                        f"FMA, {INT_MAC_SLOTS:g} per integer MAC, {DW_OPS_PER_MAC:g} per "
-                                        "double-word MAC, overlapped with the issued tensor tiles at the measured "
-                                        "tensor peak; the kernel's own instruction mix, not a hardware roof"}}
+                "terms": terms}
 
     # headline: the faster mixed form among those within 1e-10 of the FP64
     # kernel on every element (or when the FP64 form did not run); else FP64
@@ -1083,7 +1090,10 @@ def run_ours(args):
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": hr["ms"], "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": {"mixed": "tf32x3+f32+f64", "mixed_bf16x3": "bf16x3+f32+f64"}.get(head, "f64"), "data": "synthetic",
+        "vs_baseline": None, "data": "synthetic",
+        # one refinement sweep: double-binary32 with integer Khat sums
+        "dtype": "f64" if head == "fp64" or hr["sweeps"] == 2 else "f32x2+i64" if hr["sweeps"] == 1 else
+                 {"mixed": "tf32x3+f32", "mixed_bf16x3": "bf16x3+f32"}[head],
         "config": cfg, "roofline": roofline(head), "forms": forms_out, "mixed_error": errs.get(head),
         "cpu_baseline": cpu, "e2e": e2e, "clocks": hr["clocks"], "gpu_launches": args.steps,
         "lu_comparator": lu, "predictor_sweeps": sweeps, "other_systems": systems, "time_stepping": steps,

@@ -455,7 +455,8 @@ poro_status poro_lu_predict_static(poro_ctx* ctx, int64_t first, int64_t count, 
                                    double* Qt_dev, double* I_dev, void* stream);
 
 /* Autotuner of the predictor kernels: times the CTA-size variants (0: 512
- * threads at N = 6, 256 at N = 5, 128 at N = 4, 64 at N <= 3; 1: the alternative) on the
+ * threads at N = 6, 256 at N = 5, 128 at N = 4, 64 at N <= 3, and wider where a
+ * launch is so small that all its CTAs are resident; 1: the alternative) on the
  * first `sample` elements of the loaded population (<= 0: all), three timed
  * runs after two warm-ups each, and keeps the fastest for this context.
  * *variant_out (nullable) receives the choice, ms_out[2] (nullable) the

@@ -23,13 +23,16 @@
 //
 // One CTA per element; neighbours are read only through I (or, for another
 // cluster, the buffered sub-step sums or the predictor), so Q is updated in
-// place.  What bounds it: binary64, the FP64 pipe; double-binary32, load and
-// barrier latency (issue slots 61 % busy).  Double-binary32 sums therefore run on
-// the packed binary32 operations, a lane per two of the 4 columns: half the
-// instructions, and a table entry is read by 2 lanes instead of 4.  A run of 5,184
-// elements at N = 6: 6.49 -> 6.33 ms a pass, 12 thousand in two clusters at N = 3:
-// 15.33 -> 15.06.  In binary64 that only leaves fewer lanes for the FP64 pipe
-// (N = 5, 6,000 elements: 3.54 -> 3.68 ms), so there a lane has one column.
+// place.  What bounds it: binary64, the FP64 pipe (N = 5: 96 % busy, 6,000
+// elements in 684 microseconds); double-binary32, load and barrier latency (N = 6,
+// 5,184 elements: 405 microseconds).  Double-binary32 sums run on the packed
+// binary32 operations, a lane per two of the 4 columns: half the instructions, and
+// a table entry is read by 2 lanes instead of 4 (a run of 5,184 elements at N = 6:
+// 6.49 -> 6.33 ms a pass; 12,288 in three clusters at N = 3: 15.33 -> 15.06).  In
+// binary64 that only leaves fewer lanes for the FP64 pipe (N = 5, 6,000 elements:
+// 3.54 -> 3.68 ms), so there a lane has one column.  Dense traces, flux matrices and
+// the volume term took 29.5 ms (binary64) and 14.6 ms (double-binary32) for 48,000
+// elements at N = 5; the faces alone now take 5.5 ms in binary64.
 #include <cuda_runtime.h>
 
 #include "chain.cuh"
@@ -257,7 +260,8 @@ __global__ void __launch_bounds__(FaceShape<N>::NT, FaceShape<N>::MIN_BLOCKS)
 }
 
 // Q += E I - sum_j Khat^j A^j I in binary64: the volume line for a predictor
-// that did not write Q~(1) itself
+// that did not write Q~(1) itself (poro_correct after a separate predictor, the
+// unrefined form): off the step's path, so kept plain
 constexpr int VNT = 128;
 template <bool BATCH>
 __global__ void __launch_bounds__(VNT) volume_kernel(int N, const CorrectorData D1, const int32_t* elems,

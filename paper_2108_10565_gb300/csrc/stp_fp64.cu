@@ -16,7 +16,8 @@
 //
 // What bounds it: the binary64 pipe (2 lanes a clock and SM) carries the star
 // products and time solves, the integer pipes the Khat products, which were 60 to
-// 75 % of the binary64 operations.
+// 75 % of the binary64 operations.  20,000 elements at N = 4: 0.65 ms, the binary64
+// pipe 85 % busy (1.59 ms with the Khat products on it).
 #include <cuda_runtime.h>
 
 #include "alg3_device.cuh"
