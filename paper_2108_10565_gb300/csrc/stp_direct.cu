@@ -131,7 +131,13 @@ struct DirectSizes {
     static constexpr int WIDEST = N <= 2 ? 128 : N == 3 ? 256 : 512;
     static constexpr int NT0 = N == 6 ? 512 : N == 5 ? 256 : N == 4 ? 128 : 64;
     static constexpr int NT1 = N == 6 ? 256 : N == 5 ? 512 : N == 4 ? 256 : 128;
-    static constexpr int MIN_BLOCKS = N == 6 ? 2 : N == 5 ? 3 : N == 4 ? 5 : 8;
+    // CTAs an SM that the default size's registers leave room for: what shared memory
+    // allows from N = 3 on.  Against 8 CTAs, 40,000 elements, microseconds, binary64
+    // (double-binary32): N = 3 1,554 -> 1,555 (937 -> 897), N = 2 780 -> 758 (499 ->
+    // 468), N = 1 455 -> 438 (305 -> 272).  Narrower passes over X for still more CTAs
+    // cost more at their barriers (N = 4, 24 columns, 6 CTAs: 1,551 -> 1,603, 927 -> 968;
+    // N = 5, 30 columns, 4 CTAs: 2,456 -> 2,593, 1,505 -> 1,567 for 16,384).
+    static constexpr int MIN_BLOCKS = N == 6 ? 2 : N == 5 ? 3 : N == 4 ? 5 : N == 3 ? 10 : 14;
 };
 
 template <int N, int NT_>
