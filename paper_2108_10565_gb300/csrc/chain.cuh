@@ -19,7 +19,7 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 __device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // The predictor and the faces let the next kernel in early up to degree 4, where
 // elements are short: a cycle of 384 elements at N = 2 takes 41.3 instead of 43.4
-// microseconds, 12 thousand elements in two clusters at N = 3 14.02 instead of
+// microseconds, 12,288 elements in three clusters at N = 3 14.02 instead of
 // 14.10 ms.  At N = 6 (5,184 elements) the early CTAs crowd the SMs that run out
 // first: 6.02 ms a pass instead of 5.97.
 constexpr bool chain_early(int N) { return N <= 4; }
