@@ -63,7 +63,8 @@ typedef enum {
     PORO_FP64 = 0,          /* IEEE binary64; the Khat products as exact integer sums of
                                62-bit fixed-point rows, rounded once */
     PORO_FP32_REFINE = 1,   /* double-binary32 (~48 bits) with integer Khat products: within
-                               1e-10 of binary64 at the default refinement (about 1e-14) */
+                               1e-10 of binary64 at the default refinement (about 1e-14);
+                               time stepping adds each step's change to a binary64 field */
     PORO_BF16X3_REFINE = 2  /* the same; the two differ in the unrefined form only (tf32 or
                                bf16 split products, poro_set_refinement) */
 } poro_precision;

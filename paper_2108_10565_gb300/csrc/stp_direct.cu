@@ -92,7 +92,7 @@ struct DirectParams {
     const double* econst;
     double* qt;
     double* iout;
-    double* qend;           // Q~(1) [ne][13][B], may be q0
+    double* qend;           // Q~(1) [ne][13][B], may be q0 (in double-binary32: q0 and its change, added in binary64)
     int64_t count;
     int stride;
     const double* inv_d;    // [B] 1 / d_l
@@ -282,9 +282,12 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 return v64;
             };
             // the time integrals and Q~(1) of the task's rows, entry i in lane i of
-            // the group, from lane 0's value of the row and b_0 + (E* Q)_0 (the
-            // columns of Z^{-1} but the first sum to zero).  q0 may be the array
-            // written: its entries read by this task are the ones it writes.
+            // the group, from lane 0's value of the row and of b + E* Q (the columns
+            // of Z^{-1} but the first sum to zero).  In double-binary32 `end` leaves
+            // q0 out of b, and what remains, the step's change, is added to q0 in
+            // binary64, so that a field carried from step to step keeps its bits.
+            // q0 may be the array written: its entries read by this task are the
+            // ones it writes.
             auto finish = [&](auto row, const auto& v, const auto& end) {
                 constexpr int M = sizeof(v) / sizeof(double);
 #pragma unroll
@@ -303,7 +306,11 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                         R w = P::shfl(end[i], base);
 #pragma unroll
                         for (int k = 1; k < T && i + k < M; ++k) w = P::select(u == k, P::shfl(end[i + k], base), w);
-                        if (mine) qe[row(i + u) * B + m] = P::value(P::normal(w));
+                        if (mine) {
+                            const int at = row(i + u) * B + m;
+                            const double x = P::value(P::normal(w));
+                            qe[at] = P::DW ? q0[at] + x : x;
+                        }
                     }
                 }
             };
@@ -315,28 +322,33 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 const R D = c[0], Df = c[T], gx = c[2 * T], gy = c[9 * T];
                 const R gz = P::sub(P::sub(D, gx), gy);
                 const R Lm = P::neg(P::fma(iso[10], Df, P::mul(iso[9], D)));
-                const R b[4] = {rhs(q[0], 0, P::fma1(-2.f, gx, Lm)), rhs(q[1 / T], 1 % T, P::fma1(-2.f, gy, Lm)),
-                                rhs(q[2 / T], 2 % T, P::fma1(-2.f, gz, Lm)),
-                                rhs(q[3 / T], 3 % T, P::fma(iso[11], Df, P::mul(iso[10], D)))};
+                R a[4], b[4];
+                b[0] = rhs(q[0], 0, a[0] = P::fma1(-2.f, gx, Lm));
+                b[1] = rhs(q[1 / T], 1 % T, a[1] = P::fma1(-2.f, gy, Lm));
+                b[2] = rhs(q[2 / T], 2 % T, a[2] = P::fma1(-2.f, gz, Lm));
+                b[3] = rhs(q[3 / T], 3 % T, a[3] = P::fma(iso[11], Df, P::mul(iso[10], D)));
                 const double v[4] = {put(SXX, plain(b[0])), put(SXX + 1, plain(b[1])), put(SXX + 2, plain(b[2])),
                                      put(QP, plain(b[3]))};
-                finish([](int r) { return r < 3 ? SXX + r : QP; }, v, b);
+                finish([](int r) { return r < 3 ? SXX + r : QP; }, v, P::DW ? a : b);
             } else {
                 // one pair (u, u_f) of velocities and one shear stress
                 const int i = kind - 1;
                 const R q = load(u == 0 ? QU + i : u == 1 ? QUF + i : SXY + i);
                 const R qs = T > 2 ? q : load(SXY + i);
-                const R bs = rhs(qs, T > 2 ? 2 : 0, P::neg(c[(SXY + i) * T]));
+                const R as = P::neg(c[(SXY + i) * T]);
+                const R bs = rhs(qs, T > 2 ? 2 : 0, as);
                 const R Sg = c[(QU + i) * T], Gp = c[(QUF + i) * T];
-                const R bu = rhs(q, 0, P::neg(P::fma(iso[13], Gp, P::mul(iso[12], Sg))));
-                const R bf = rhs(q, 1, P::fma(iso[14], Gp, P::mul(iso[13], Sg)));
+                const R au = P::neg(P::fma(iso[13], Gp, P::mul(iso[12], Sg)));
+                const R af = P::fma(iso[14], Gp, P::mul(iso[13], Sg));
+                const R bu = rhs(q, 0, au), bf = rhs(q, 1, af);
                 R xf = P::mul(zuf[u * T], P::shfl(bf, base));
 #pragma unroll
                 for (int s = 1; s < T; ++s) xf = P::fma(zuf[u * T + s], P::shfl(bf, base + s), xf);
                 xf = P::normal(xf);
                 const R by = P::fma(K[T * T + 1], xf, bu);  // + g Q_uf
                 const double v[3] = {put(QU + i, plain(by)), put(QUF + i, xf), put(SXY + i, plain(bs))};
-                const R end[3] = {by, P::fma(K[T * T], xf, bf), bs};
+                const R end[3] = {P::DW ? P::fma(K[T * T + 1], xf, au) : by, P::fma(K[T * T], xf, P::DW ? af : bf),
+                                  P::DW ? as : bs};
                 finish([i](int r) { return (r == 0 ? QU : r == 1 ? QUF : SXY) + i; }, v, end);
             }
         }

@@ -134,3 +134,55 @@ def test_launch_sizes_agree(L, N, precision):
         part = {k: d[k][:n] for k in ("vertices", "materials")}
         got = _predict(L, dict(part, N=N, dt=d["dt"]), precision, d["Q0"][:n])
         np.testing.assert_array_equal(got, ref[:n], err_msg=f"{n} elements")
+
+
+def _advance(L, N, precision, mesh, q0, steps, sweeps=1):
+    from paper_2108_10565_gb300 import inputs
+
+    ctx = L.poro_create(0, N, precision)
+    try:
+        if precision:
+            L.poro_set_refinement(ctx, sweeps)
+        L.poro_set_mesh(ctx, mesh["vertices"], mesh["tets"], mesh["neighbors"], mesh["face_tag"])
+        L.poro_set_materials(ctx, np.tile(inputs.REFERENCE_MATERIAL, (mesh["tets"].shape[0], 1)))
+        dt, _ = L.poro_set_clusters(ctx, 0.5, 1)
+        L.poro_set_dofs(ctx, q0)
+        L.poro_advance(ctx, (steps + 0.5) * dt)
+        return L.poro_get_dofs(ctx)
+    finally:
+        L.poro_destroy(ctx)
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("precision", [1, 2])
+def test_mixed_steps_carry_the_field_in_binary64(L, N, precision):
+    """The double-binary32 predictor gives a step's change, and the field itself stays in binary64.  A uniform field
+    without relative fluid flow does not change (the two sides of every face are equal word by word, so the change is
+    zero), and entries below binary32's range (whose change is then zero) stay as they are."""
+    from paper_2108_10565_gb300 import inputs
+
+    mesh = inputs.kuhn_box_mesh(3)
+    ne, B = mesh["tets"].shape[0], (N + 1) * (N + 2) * (N + 3) // 6
+    rng = np.random.default_rng(N)
+    q0 = np.zeros((ne, 13, B))
+    q0[:, :10, 0] = rng.standard_normal(10) * np.r_[np.full(6, 1e7), np.ones(3), 1e7]
+    np.testing.assert_array_equal(_advance(L, N, precision, mesh, q0, 3), q0)
+    q0 = rng.standard_normal((ne, 13, B)) * 1e-60
+    np.testing.assert_array_equal(_advance(L, N, precision, mesh, q0, 3), q0)
+
+
+@pytest.mark.parametrize("N", [2, 3])
+def test_mixed_steps_do_not_drift(L, N):
+    """Thousands of mixed steps against as many in binary64, elements 1e-9 of the field's size among them: every step
+    rounds its change in about 2^-48, so that n steps are within n 2^-48 of the field's size."""
+    from paper_2108_10565_gb300 import inputs
+
+    steps = 4000
+    mesh = inputs.kuhn_box_mesh(3)
+    ne, B = mesh["tets"].shape[0], (N + 1) * (N + 2) * (N + 3) // 6
+    q0 = np.random.default_rng(N).standard_normal((ne, 13, B)) * np.r_[np.full(6, 1e7), np.ones(3), 1e7, np.zeros(3)][:, None]
+    q0[::2] *= 1e-9
+    a, b = _advance(L, N, 1, mesh, q0, steps), _advance(L, N, 0, mesh, q0, steps)
+    for p in range(13):
+        err = np.abs(a[:, p] - b[:, p]).max() / np.abs(b[:, p]).max()
+        assert err <= steps * 2.0 ** -48, (p, err)
