@@ -1736,20 +1736,24 @@ static int group_tick_items(RunGroup* g) {
             for (int cl = 0; cl < g->C; ++cl) {
                 const int64_t len = (int64_t)1 << cl;
                 if ((k + 1) % len || c->cl_elems[cl].empty()) continue;
-                for (auto& sr : c->sources)
-                    if (c->h_cl[sr.elem] == cl) {
-                        TickItem it;
-                        it.q = c->d_q0;
-                        it.vec = sr.d_coef;
-                        it.tick = c->d_tick;
-                        it.elem = sr.elem;
-                        it.len = len;
-                        it.k_rel = k;
-                        it.f0 = sr.f0;
-                        it.tc = sr.t0;
-                        it.dt = c->dt;
-                        src.push_back(it);
-                    }
+                // an element's sources side by side (one CTA adds them), in their order
+                std::vector<poro_ctx::Source> due;
+                for (const auto& sr : c->sources)
+                    if (c->h_cl[sr.elem] == cl) due.push_back(sr);
+                std::stable_sort(due.begin(), due.end(), [](const auto& a, const auto& b) { return a.elem < b.elem; });
+                for (const auto& sr : due) {
+                    TickItem it;
+                    it.q = c->d_q0;
+                    it.vec = sr.d_coef;
+                    it.tick = c->d_tick;
+                    it.elem = sr.elem;
+                    it.len = len;
+                    it.k_rel = k;
+                    it.f0 = sr.f0;
+                    it.tc = sr.t0;
+                    it.dt = c->dt;
+                    src.push_back(it);
+                }
                 for (int r = 0; r < (int)c->rec_elem.size(); ++r)
                     if (c->h_cl[c->rec_elem[r]] == cl) {
                         TickItem it;

@@ -351,12 +351,21 @@ __global__ void ticks_advance_kernel(int64_t* const* ticks, int count, int64_t n
     if (i < count) *ticks[i] += n;
 }
 
-// one CTA per source item (of several runs), or one CTA for a run's list (its
-// sources may share an element)
+// The source items of several runs, those of one element side by side: its first
+// item's CTA adds them all, in order.  Or one CTA for a run's list.
 __global__ void source_items_kernel(int QB, const TickItem* items) {
     chain_wait();
     chain_go();
-    add_source(QB, items[blockIdx.x], 0);
+    const TickItem* it = items + blockIdx.x;
+    const TickItem* end = items + gridDim.x;
+    const double* q = it->q;
+    const int64_t elem = it->elem;
+    auto same = [&](const TickItem& o) { return o.q == q && o.elem == elem; };
+    if (it > items && same(it[-1])) return;
+    for (; it < end && same(*it); ++it) {
+        add_source(QB, *it, 0);
+        __syncthreads();
+    }
 }
 __global__ void source_list_kernel(int QB, const TickItem* items, int count, int64_t k_add) {
     chain_wait();

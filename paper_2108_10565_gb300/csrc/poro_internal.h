@@ -390,6 +390,7 @@ struct TickItem {
     int64_t elem = 0, len = 1, k_rel = 0;
     double f0 = 0.0, tc = 0.0, dt = 0.0;
 };
+// (items of one element side by side)
 int launch_tick_sources(int N, const TickItem* items, int64_t count, void* stream);
 // one run's list, in order, at tick k_add of the cycle
 int launch_source_list(int N, const TickItem* items, int count, int64_t k_add, void* stream);

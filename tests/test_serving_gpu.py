@@ -112,6 +112,33 @@ def test_alone_equals_in_the_mix(L, batched):
         L.poro_server_destroy(srv)
 
 
+def test_sources_of_one_element_in_the_mix(L):
+    """Several sources in one element (A, B, A again, with one of another element between them): a batched group adds
+    them in the order in which the run alone does, none is lost, bit for bit."""
+    base = _scenarios()[0]
+    a, b = np.array([0.31, 0.62, 0.44]), np.array([0.305, 0.622, 0.441])
+    far = dict(base["src"][0], x=np.array([0.75, 0.2, 0.6]))
+    one = [dict(base["src"][0], x=a), far] + [dict(base["src"][0], x=x, t0=2e-4 + 1e-5 * i, amplitude=1e6 * (i + 1))
+                                              for i, x in enumerate((b, a, b, a, a))]
+    base = dict(base, rec=[a, *base["rec"]])
+    scs = [dict(base, src=one), dict(base, src=one[::-1], cycles=9), dict(base, src=one[2:], cycles=7)]
+    ends = [_t_end(L, sc) for sc in scs]
+    alone = [_alone(L, sc, te) for sc, te in zip(scs, ends)]
+    srv = L.poro_server_create(0, 64 << 30, 8)
+    try:
+        L.poro_server_set_batching(srv, True)
+        tickets = [_submit(L, srv, sc, te) for sc, te in zip(scs, ends)]
+        for t in tickets:
+            assert L.poro_wait(srv, t, 300_000) == L.PORO_REQ_DONE, L.poro_request_error(srv, t)
+        for sc, t, ref in zip(scs, tickets, alone):
+            for r in range(len(sc["rec"])):
+                q = L.poro_fetch(srv, t, r)[1]
+                assert np.array_equal(q, ref[r][1])
+            assert ref[0][1].any()  # the receiver in the sources' element (the others may lie too far)
+    finally:
+        L.poro_server_destroy(srv)
+
+
 def test_failure_isolation_and_cancel(L):
     scs = _scenarios()
     good = scs[0]
