@@ -205,12 +205,15 @@ __global__ void __launch_bounds__(NT_) stp_subcell_kernel(const SubParams P) {
                     mass_term<NT, Sweep, S::CHUNK>(V, term, p0, np, P.m3_row + r * (B + 1), P.m3_col, P.m3_val);
                 }
             alg3_sweep<N, NT, BiotSystem, Sweep>(V, star, zuf, sc[1], P.khat, X);  // Q_{k+1}
-            // max |Q_{k+1} - Q_k| and max |Q_{k+1}| over the element
+            // max |Q_{k+1} - Q_k| and max |Q_{k+1}| over the element (fmax drops a NaN,
+            // so non-finite differences are noted apart)
             double dmax = 0.0, vmax = 0.0;
+            bool bad = false;
             for (int i = tid; i < NQ * BT; i += NT) {
                 const int p = i / BT, m = i - p * BT;
-                const double v = V[p * QS + m];
-                dmax = fmax(dmax, fabs(v - U[p * QS + m]));
+                const double v = V[p * QS + m], dv = fabs(v - U[p * QS + m]);
+                bad |= !isfinite(dv);
+                dmax = fmax(dmax, dv);
                 vmax = fmax(vmax, fabs(v));
             }
 #pragma unroll
@@ -222,7 +225,7 @@ __global__ void __launch_bounds__(NT_) stp_subcell_kernel(const SubParams P) {
                 red[warp] = dmax;
                 red[NW + warp] = vmax;
             }
-            __syncthreads();
+            const bool finite = !__syncthreads_or(bad);
             dmax = 0.0;
             vmax = 0.0;
             for (int w = 0; w < NW; ++w) {
@@ -230,7 +233,6 @@ __global__ void __launch_bounds__(NT_) stp_subcell_kernel(const SubParams P) {
                 vmax = fmax(vmax, red[NW + w]);
             }
             // a non-finite iterate stops the loop unconverged (and is written out as it is)
-            const bool finite = isfinite(dmax) && isfinite(vmax);
             converged = finite && dmax <= P.tol * vmax;
             stop = converged || !finite;
             double* t = U;

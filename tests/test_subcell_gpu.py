@@ -130,3 +130,21 @@ def test_subcell_iteration_limit_and_errors(L):
         assert ex.value.status == L.PORO_EUNSUPPORTED
     finally:
         L.poro_destroy(ctx)
+
+
+@pytest.mark.parametrize("N", [1, 4, 6])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("where", [(7, 0), (2, -1), (slice(None), slice(None))])
+def test_non_finite_data_do_not_converge(L, N, bad, where):
+    """One element with a non-finite entry, or nothing but such entries: its iteration count is negative, its result is
+    not finite, and the other elements are what they are without it."""
+    d = _population(4, N, 0.2, seed=1500 + N)
+    ref, _, ref_iters = _gpu(L, d, N)
+    q0 = d["Q0"].copy()
+    q0[2][where] = bad
+    qt, _, iters = _gpu(L, dict(d, Q0=q0), N)
+    keep = np.arange(4) != 2
+    np.testing.assert_array_equal(qt[keep], ref[keep])
+    np.testing.assert_array_equal(iters[keep], ref_iters[keep])
+    assert (ref_iters > 0).all() and iters[2] < 0, iters
+    assert not np.isfinite(qt[2]).all()
