@@ -458,10 +458,13 @@ poro_status poro_lu_predict_static(poro_ctx* ctx, int64_t first, int64_t count, 
 /* Autotuner of the predictor kernels: times the CTA-size variants (0: 512
  * threads at N = 6, 256 at N = 5, 128 at N = 4, 64 at N <= 3, and wider where a
  * launch is so small that all its CTAs are resident; 1: the alternative) on the
- * first `sample` elements of the loaded population (<= 0: all), three timed
- * runs after two warm-ups each, and keeps the fastest for this context.
- * *variant_out (nullable) receives the choice, ms_out[2] (nullable) the
- * mean milliseconds per run of each variant.  The DOFs are not changed; the
+ * first `sample` elements of the loaded population (<= 0: all; at least so many
+ * that launches of all of it take the same CTA size, 4 per SM), three timed
+ * runs after two warm-ups each, and keeps the fastest for this context.  A kept
+ * alternative replaces the default size, small launches stay on their wider CTAs;
+ * where both variants are the same kernel for the population, it is timed once and
+ * variant 0 kept.  *variant_out (nullable) receives the choice, ms_out[2] (nullable)
+ * the mean milliseconds per run of each variant.  The DOFs are not changed; the
  * context's predictor buffers are overwritten.  The paper has no counterpart
  * (its kernels are generated per architecture). */
 poro_status poro_autotune(poro_ctx* ctx, int64_t sample, int32_t* variant_out, double* ms_out);
@@ -478,11 +481,11 @@ poro_status poro_set_variant(poro_ctx* ctx, int32_t variant);
  * one refinement sweep (the default) only. */
 #define PORO_TILE_CHOICES 12
 
-/* Autotuner over the available tile choices: times each on the first
- * `sample` elements of the loaded population (<= 0: all; two warm-ups,
- * three timed runs) and keeps the fastest for this context.  *choice_out
- * (nullable) receives it, ms_out[PORO_TILE_CHOICES] (nullable) the mean
- * milliseconds per run of each choice (-1 for choices not available).  The
+/* Autotuner over the available tile choices: times the kernel of each CTA size
+ * once, as poro_autotune does, and keeps the fastest for this context.
+ * *choice_out (nullable) receives it (0 or 6), ms_out[PORO_TILE_CHOICES] (nullable)
+ * the mean milliseconds per run of each choice, those of one CTA size alike (-1 for
+ * choices not available).  The
  * DOFs are kept; the predictor buffers are overwritten.  The paper has no
  * counterpart (its kernels are generated per architecture).
  * Errors: PORO_ESTATE (no population), PORO_EUNSUPPORTED (not Biot). */

@@ -35,7 +35,7 @@ struct poro_ctx {
     poro::LUScratch lu;
     int64_t lu_first = 0, lu_count = 0;
     int refine = 1;
-    int variant = 0;   // predictor CTA-size variant (poro_autotune)
+    int variant = 0;   // predictor CTA-size variant (launch_stp_fp64)
     int64_t n_elem = 0;
     int stride = 0;
     double* d_econst = nullptr;
@@ -1948,47 +1948,63 @@ poro_status poro_flux_matrices(const poro_material* mL, const poro_material* mR,
     return PORO_OK;
 }
 
+// The elements that a tuner times of `sample` asked for: at least as many as make
+// the launch rule take the CTA size that the whole population's launch gets.
+static int64_t tuner_sample(const poro_ctx* c, int64_t sample) {
+    const int64_t n = std::max<int64_t>(1, std::min(sample > 0 ? sample : c->n_elem, c->n_elem));
+    return std::max(n, std::min(c->n_elem, poro::direct_default_count()));
+}
+
+// Times the kernels that the variants 0 and 1 of a tuner stand for on the first n
+// elements, ms[2] per run; variant 1 as the alternative to the default size, so that
+// small launches (a small cluster's) keep their wider CTAs.  Where both are one
+// kernel it is timed once.
+static poro_status time_variants(poro_ctx* c, int64_t n, double ms[2], const char* who) {
+    const bool swept = c->prec != PORO_FP64 && c->refine == 0;  // the unrefined form: bf16 has one CTA size
+    const bool one = swept ? c->prec == PORO_BF16X3_REFINE
+                           : poro::direct_cta_size(c->N, 0, n) == poro::direct_cta_size(c->N, 2, n);
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+        if (e0) cudaEventDestroy(e0);
+        return cuda_fail(c, cudaErrorMemoryAllocation, who);
+    }
+    const int saved = c->variant;
+    poro_status st = PORO_OK;
+    for (int v = 0; v < (one ? 1 : 2) && st == PORO_OK; ++v) {
+        c->variant = 2 * v;
+        for (int w = 0; w < 2 && st == PORO_OK; ++w)
+            st = dispatch_predict(c, 0, n, c->d_q0, c->d_qt, c->d_iout, PORO_SOLVE_BLOCK, c->stream);
+        cudaEventRecord(e0, c->stream);
+        for (int r = 0; r < 3 && st == PORO_OK; ++r)
+            st = dispatch_predict(c, 0, n, c->d_q0, c->d_qt, c->d_iout, PORO_SOLVE_BLOCK, c->stream);
+        cudaEventRecord(e1, c->stream);
+        const cudaError_t er = cudaEventSynchronize(e1);
+        if (st == PORO_OK && er != cudaSuccess) st = cuda_fail(c, er, who);
+        if (st == PORO_OK) st = device_status(c, who);
+        float t = 0.f;
+        if (st == PORO_OK) cudaEventElapsedTime(&t, e0, e1);
+        ms[v] = t / 3.0;
+    }
+    if (one) ms[1] = ms[0];
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    c->variant = saved;
+    return st;
+}
+
 poro_status poro_autotune(poro_ctx* c, int64_t sample, int32_t* variant_out, double* ms_out) {
     if (!c) return fail(nullptr, PORO_EINVAL, "poro_autotune: ctx is NULL");
     if (c->system != PORO_SYSTEM_BIOT || c->subcell)
         return fail(c, PORO_EUNSUPPORTED, "poro_autotune: the autotuner is built for Biot's constant-material predictor");
     if (!c->d_econst || c->n_elem <= 0) return fail(c, PORO_ESTATE, "poro_autotune: no element population loaded");
     cudaSetDevice(c->device);
-    const int64_t n = std::max<int64_t>(1, std::min(sample > 0 ? sample : c->n_elem, c->n_elem));
-    double best = 1e300;
-    int bestv = 0;
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    const int saved = c->variant;
-    for (int v = 0; v < 2; ++v) {
-        c->variant = v;
-        poro_status s = PORO_OK;
-        for (int w = 0; w < 2 && s == PORO_OK; ++w)
-            s = dispatch_predict(c, 0, n, c->d_q0, c->d_qt, c->d_iout, PORO_SOLVE_BLOCK, c->stream);
-        cudaEventRecord(e0, c->stream);
-        for (int r = 0; r < 3 && s == PORO_OK; ++r)
-            s = dispatch_predict(c, 0, n, c->d_q0, c->d_qt, c->d_iout, PORO_SOLVE_BLOCK, c->stream);
-        cudaEventRecord(e1, c->stream);
-        cudaError_t er = cudaEventSynchronize(e1);
-        if (s != PORO_OK || er != cudaSuccess) {
-            c->variant = saved;
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            return s != PORO_OK ? s : cuda_fail(c, er, "poro_autotune");
-        }
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms_out) ms_out[v] = ms / 3.0;
-        if (ms < best) {
-            best = ms;
-            bestv = v;
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    c->variant = bestv;
-    if (variant_out) *variant_out = bestv;
+    double ms[2];
+    if (poro_status st = time_variants(c, tuner_sample(c, sample), ms, "poro_autotune")) return st;
+    const int best = ms[1] < ms[0] ? 1 : 0;
+    c->variant = 2 * best;
+    if (ms_out)
+        for (int v = 0; v < 2; ++v) ms_out[v] = ms[v];
+    if (variant_out) *variant_out = best;
     return PORO_OK;
 }
 
@@ -2022,43 +2038,15 @@ poro_status poro_autotune_tiles(poro_ctx* c, int64_t sample, int32_t* choice_out
         return fail(c, PORO_EUNSUPPORTED, "poro_autotune_tiles: Biot constant-material contexts only");
     if (!c->d_econst || c->n_elem <= 0) return fail(c, PORO_ESTATE, "poro_autotune_tiles: no element population loaded");
     cudaSetDevice(c->device);
-    const int64_t n = std::max<int64_t>(1, std::min(sample > 0 ? sample : c->n_elem, c->n_elem));
-    const int saved_v = c->variant;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
-        if (e0) cudaEventDestroy(e0);
-        return cuda_fail(c, cudaErrorMemoryAllocation, "poro_autotune_tiles: events");
-    }
-    double best = 1e300;
-    int bestc = 0;
-    poro_status st = PORO_OK;
-    for (int choice = 0; choice < PORO_TILE_CHOICES && st == PORO_OK; ++choice) {
-        if (ms_out) ms_out[choice] = -1.0;
-        if (!tile_choice_valid(c, choice)) continue;
-        apply_tile_choice(c, choice);
-        for (int w = 0; w < 2 && st == PORO_OK; ++w)
-            st = dispatch_predict(c, 0, n, c->d_q0, c->d_qt, c->d_iout, PORO_SOLVE_BLOCK, c->stream);
-        cudaEventRecord(e0, c->stream);
-        for (int r = 0; r < 3 && st == PORO_OK; ++r)
-            st = dispatch_predict(c, 0, n, c->d_q0, c->d_qt, c->d_iout, PORO_SOLVE_BLOCK, c->stream);
-        cudaEventRecord(e1, c->stream);
-        const cudaError_t er = cudaEventSynchronize(e1);
-        if (st == PORO_OK && er != cudaSuccess) st = cuda_fail(c, er, "poro_autotune_tiles");
-        if (st == PORO_OK) st = device_status(c, "poro_autotune_tiles");
-        float ms = 0.f;
-        if (st == PORO_OK) cudaEventElapsedTime(&ms, e0, e1);
-        if (st == PORO_OK && ms_out) ms_out[choice] = ms / 3.0;
-        if (st == PORO_OK && ms < best) {
-            best = ms;
-            bestc = choice;
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    c->variant = saved_v;
-    if (st != PORO_OK) return st;
-    apply_tile_choice(c, bestc);
-    if (choice_out) *choice_out = bestc;
+    // the layouts of one CTA size are one kernel: it is timed once for all of them
+    double ms[2];
+    if (poro_status st = time_variants(c, tuner_sample(c, sample), ms, "poro_autotune_tiles")) return st;
+    const int best = tile_choice_valid(c, 6) && ms[1] < ms[0] ? 6 : 0;
+    c->variant = best ? 2 : 0;
+    if (ms_out)
+        for (int choice = 0; choice < PORO_TILE_CHOICES; ++choice)
+            ms_out[choice] = tile_choice_valid(c, choice) ? ms[choice / 6] : -1.0;
+    if (choice_out) *choice_out = best;
     return PORO_OK;
 }
 

@@ -438,12 +438,17 @@ int launch_stp_direct(const DeviceReference& ref, bool dw, bool whole_nan, int32
                       const int32_t* elems, int64_t count, const double* q0, const double* econst, double* qt,
                       double* iout, double* qend, void* stream, int variant, const RunPtrs* runs,
                       const int32_t* item_run);
+// the CTA size it takes for `count` elements (variant 0, 1 or 2), and a count from
+// which on variant 0 takes the default size at every degree
+int direct_cta_size(int N, int variant, int64_t count);
+int64_t direct_default_count();
 
 // Launch the FP64 Algorithm-3 predictor for `count` elements.
 // q0[count][13][B], econst[count][stride], qt, iout, qend (Q~(1), may be q0) nullable.
 // `elems` (nullable): element index list; outputs are indexed by element.
-// `variant` selects the CTA size (0: default, 1: the alternative the
-// autotuner may pick).  `runs` / `item_run`: items of several runs, as for
+// `variant` selects the CTA size (0: default, wider for launches of few elements;
+// 1: the alternative; 2: the alternative in place of the default, for launches of
+// more elements, which the autotuners may pick).  `runs` / `item_run`: items of several runs, as for
 // launch_stp_mixed.
 int launch_stp_fp64(const DeviceReference& ref, const int32_t* elems, int64_t count, const double* q0,
                     const double* econst, double* qt, double* iout, double* qend, void* stream, int variant = 0,

@@ -475,21 +475,40 @@ int launch_nt(const DirectParams& A, void* stream) {
 //   608            N = 2 17.9 -> 17.3 (14.9 -> 12.3)   N = 3 34.3 -> 31.3 (24.2 -> 18.6)
 // and one CTA more an SM turns it round (N = 3, 912 elements on 128 threads: 45.1
 // -> 62.5; 384 on 256: 28.8 -> 37.1).
+// Variant 1 is the alternative size for every launch, variant 2 only for those that
+// the rule leaves to the default size.
+template <int N>
+int cta_size(int variant, int64_t count, int64_t sms) {
+    using D = DirectSizes<N>;
+    if (variant == 1) return D::NT1;
+    if (D::WIDEST >= 512 && D::NT0 < 512 && count <= sms) return 512;
+    if (D::WIDEST >= 256 && D::NT0 < 256 && count <= 2 * sms) return 256;
+    if (D::WIDEST >= 128 && D::NT0 < 128 && count <= 4 * sms) return 128;
+    return variant == 2 ? D::NT1 : D::NT0;
+}
+
+int sm_count(int& sms) {
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return (int)err;
+}
+
 template <int N, class P>
 int launch_p(const DirectParams& A, int variant, void* stream) {
     using D = DirectSizes<N>;
-    if (variant == 1) return launch_nt<N, D::NT1, P>(A, stream);
-    int dev = 0, sms = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (err != cudaSuccess) return (int)err;
-    if constexpr (D::WIDEST >= 512 && D::NT0 < 512)
-        if (A.count <= sms) return launch_nt<N, 512, P>(A, stream);
-    if constexpr (D::WIDEST >= 256 && D::NT0 < 256)
-        if (A.count <= 2 * (int64_t)sms) return launch_nt<N, 256, P>(A, stream);
-    if constexpr (D::NT0 < 128)
-        if (A.count <= 4 * (int64_t)sms) return launch_nt<N, 128, P>(A, stream);
-    return launch_nt<N, D::NT0, P>(A, stream);
+    int sms = 0;
+    if (const int err = sm_count(sms)) return err;
+    const int nt = cta_size<N>(variant, A.count, sms);
+    if constexpr (D::NT0 == 64)
+        if (nt == 64) return launch_nt<N, 64, P>(A, stream);
+    if constexpr (D::NT0 <= 128 && D::WIDEST >= 128)
+        if (nt == 128) return launch_nt<N, 128, P>(A, stream);
+    if constexpr (D::WIDEST >= 256)
+        if (nt == 256) return launch_nt<N, 256, P>(A, stream);
+    if constexpr (D::WIDEST >= 512)
+        if (nt == 512) return launch_nt<N, 512, P>(A, stream);
+    return (int)cudaErrorInvalidValue;
 }
 
 template <int N>
@@ -610,6 +629,26 @@ int upload_direct_tables(int N, const std::vector<int32_t>& ent, const std::vect
         e = cudaMemcpyToSymbol(c_list, list.data(), sizeof(int32_t) * list.size(), sizeof(int32_t) * list_base(N));
     if (e == cudaSuccess) done.insert({dev, N});
     return (int)e;
+}
+
+int direct_cta_size(int N, int variant, int64_t count) {
+    int sms = 0;
+    if (sm_count(sms)) return 0;
+    switch (N) {
+        case 1: return cta_size<1>(variant, count, sms);
+        case 2: return cta_size<2>(variant, count, sms);
+        case 3: return cta_size<3>(variant, count, sms);
+        case 4: return cta_size<4>(variant, count, sms);
+        case 5: return cta_size<5>(variant, count, sms);
+        case 6: return cta_size<6>(variant, count, sms);
+        default: return 0;
+    }
+}
+
+int64_t direct_default_count() {
+    int sms = 0;
+    sm_count(sms);
+    return 4 * (int64_t)sms + 1;
 }
 
 int launch_stp_direct(const DeviceReference& ref, bool dw, bool whole_nan, int32_t* status, long long wait_limit,

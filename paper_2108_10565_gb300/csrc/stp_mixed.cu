@@ -608,7 +608,7 @@ int launch_n(const MixedReference& ref, int variant, const int32_t* elems, int64
     // the bf16 form is built for the default CTA size only
     if (ref.bf16)
         return launch_nr<N, K2Sizes<N>::NT0, 1>(ref, elems, count, q0, econst, qt, iout, stream, runs, item_run);
-    if (variant == 1)
+    if (variant != 0)
         return launch_nr<N, K2Sizes<N>::NT1, 0>(ref, elems, count, q0, econst, qt, iout, stream, runs, item_run);
     return launch_nr<N, K2Sizes<N>::NT0, 0>(ref, elems, count, q0, econst, qt, iout, stream, runs, item_run);
 }

@@ -186,3 +186,38 @@ def test_mixed_steps_do_not_drift(L, N):
     for p in range(13):
         err = np.abs(a[:, p] - b[:, p]).max() / np.abs(b[:, p]).max()
         assert err <= steps * 2.0 ** -48, (p, err)
+
+
+def _autotune(L, N, n, sample, precision=0):
+    d = population(n, N, seed=600 + N)
+    ctx = L.poro_create(0, N, precision)
+    try:
+        L.poro_set_isolated(ctx, d["vertices"], d["materials"], d["dt"])
+        L.poro_set_dofs(ctx, d["Q0"])
+        L.poro_predict(ctx)
+        before = L.poro_get_predictor(ctx, 0, n)
+        best, ms = L.poro_autotune(ctx, sample)
+        tile, tile_ms = L.poro_autotune_tiles(ctx, sample)
+        L.poro_predict(ctx)
+        np.testing.assert_array_equal(L.poro_get_predictor(ctx, 0, n), before)
+        return best, list(ms), tile, list(tile_ms)
+    finally:
+        L.poro_destroy(ctx)
+
+
+@pytest.mark.parametrize("N", [1, 3])
+def test_autotuners_time_one_kernel_once(L, N):
+    """Up to 4 elements an SM both variants are the same kernel at N <= 3 (128 threads; at N = 3 up to two an SM 256): the
+    tuners time it once and keep variant 0."""
+    for n in (100, 400):
+        best, ms, tile, tile_ms = _autotune(L, N, n, 0)
+        assert best == 0 and ms[0] == ms[1] > 0
+        assert tile == 0 and tile_ms[0] == tile_ms[6] > 0
+
+
+def test_autotuners_time_the_kernel_that_runs(L):
+    """A sample of 100 elements out of 2,000 would be launched with a CTA size that 2,000 are not: the tuners time as many
+    as take the population's size (over 4 an SM, here at 3 CTAs an SM: two waves and more, against one)."""
+    _, small, _, small_tiles = _autotune(L, 5, 100, 0)
+    _, ms, _, tile_ms = _autotune(L, 5, 2000, 100)
+    assert ms[0] > 1.5 * small[0] and tile_ms[0] > 1.5 * small_tiles[0]
