@@ -104,15 +104,18 @@ poro_status sfail(poro_server* s, poro_status st, const std::string& m) {
     return st;
 }
 
-// device bytes one request needs (element data, faces, predictors, buffers,
-// reference and face matrices, receivers), with 25 % headroom
+// device bytes one request needs, with 25 % headroom: per element the constants, Q, I,
+// the predictor, the faces' factors, neighbours and lists (and, clustered, buffers for
+// half of the larger levels); the tables of the degree, at most dense; the receivers;
+// 32 MB for allocation granularity, launch graphs and a group's lists (a context of
+// 384 elements with 4 receivers took up to 4 MB more than its arrays, N = 1 to 6)
 size_t footprint_bytes(int N, int64_t ne, int C, int nrec) {
-    const size_t B = (size_t)poro::n_modes(N), T = (size_t)N + 1, QB = poro::NQ * B;
-    size_t per = (size_t)poro::elem_const_stride(N) * 8 + 2 * QB * 8 + QB * T * 8 + 4 * (4 + 4 + 8) +
-                 4 * 2 * poro::NQ * poro::NQ * 8;
-    if (C > 1) per += (size_t)(C - 1) * QB * 8 / 2 + 8 * C;
-    size_t fixed = 96 * B * B * 8 + 4 * B * B * 8 + (size_t)3 * B * B * 8 * 2 + (size_t)nrec * 1024 * poro::NQ * 8;
-    return (size_t)((double)(per * (size_t)ne + fixed) * 1.25) + (64u << 20);
+    const size_t B = (size_t)poro::n_modes(N), T = (size_t)N + 1, QB = poro::NQ * B, df = (size_t)poro::face_modes(N);
+    size_t per = (size_t)poro::elem_const_stride(N) * 8 + 2 * QB * 8 + QB * T * 8 + 4 * poro::FACE_FACTORS * 8 +
+                 4 * (4 + 4 + 1);
+    if (C > 1) per += (size_t)(C - 1) * QB * 8 / 2 + 12 * C;
+    size_t fixed = (8 * df * B + 6 * df * df) * 12 + (size_t)3 * B * B * 8 * 2 + (size_t)nrec * 1024 * poro::NQ * 8;
+    return (size_t)((double)(per * (size_t)ne + fixed) * 1.25) + (32u << 20);
 }
 
 // Context, mesh, materials, clusters, sources and receivers of a request;

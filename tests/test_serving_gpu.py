@@ -186,3 +186,26 @@ def test_admission_by_memory_budget(L):
         assert np.array_equal(L.poro_fetch(srv, t1, 0)[1], L.poro_fetch(srv, t2, 0)[1])
     finally:
         L.poro_server_destroy(srv)
+
+
+@pytest.mark.parametrize("N,n", [(1, 24), (2, 20), (4, 14), (6, 8)])
+def test_footprint_is_what_a_context_takes(L, N, n):
+    """The footprint that admission reserves covers the device memory of a set-up mesh with its predictor, and exceeds
+    it by no more than its quarter of headroom and the constant part."""
+    import torch
+
+    mesh = inputs.kuhn_box_mesh(n)
+    ne = mesh["tets"].shape[0]
+    L.poro_destroy(L.poro_create(0, N, 0))  # the library and its device context are up
+    free = torch.cuda.mem_get_info(0)[0]
+    ctx = L.poro_create(0, N, 0)
+    try:
+        L.poro_set_mesh(ctx, mesh["vertices"], mesh["tets"], mesh["neighbors"], mesh["face_tag"])
+        L.poro_set_materials(ctx, np.tile(inputs.REFERENCE_MATERIAL, (ne, 1)))
+        dt, _ = L.poro_set_clusters(ctx, 0.5, 1)
+        L.poro_advance(ctx, 2.5 * dt)
+        used = free - torch.cuda.mem_get_info(0)[0]
+    finally:
+        L.poro_destroy(ctx)
+    fp = L.poro_footprint_bytes(N, ne, 1, 0)
+    assert used <= fp <= 1.3 * used + (32 << 20), (used >> 20, fp >> 20)
