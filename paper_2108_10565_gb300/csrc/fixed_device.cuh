@@ -18,7 +18,8 @@ namespace poro {
 constexpr int POISON = INT32_MIN;  // row scale of a row with a non-finite bound
 
 // Binary64: x = v 2^s with |x| <= 2^30 as a 64-bit integer with 32 fraction
-// bits, as two signed words (high, low).  sh0 = 1053 - s.
+// bits, as two signed words (high, low).  sh0 = 1053 - s, one more than the biased
+// exponent of the row's bound.  (Magnitudes below 2^-1022 are not kept.)
 __device__ __forceinline__ int2 quantise(double v, int sh0) {
     const int hi = __double2hiint(v);
     const int E = (hi >> 20) & 0x7FF;
@@ -33,7 +34,7 @@ __device__ __forceinline__ int2 quantise(double v, int sh0) {
 // scale word of a row from the bound on its entries
 __device__ __forceinline__ int row_scale(double bound) {
     const int E = (__double2hiint(bound) >> 20) & 0x7FF;
-    return E == 0x7FF ? POISON : 1053 - min(30 - (E - 1022), 1000);
+    return E == 0x7FF ? POISON : E + 1;
 }
 __device__ __forceinline__ double bound_of(uint32_t bits, double) {
     return __hiloint2double((int)(bits >= 0x7FF00000u ? 0x7FF80000u : bits + 1u), 0);

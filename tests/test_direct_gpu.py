@@ -45,6 +45,18 @@ def test_power_of_two_scaling_is_exact(L, N, precision, sweeps, powers):
 
 
 @pytest.mark.parametrize("N", [1, 3, 6])
+def test_smallest_binary64_data(L, N):
+    """Velocities near the lower end of binary64's range: the stresses and pressure that follow from them (2^20 times as
+    large, so that nothing on the way leaves the normal range) are as accurate as those of data of ordinary size."""
+    d = population(5, N, seed=850 + N)
+    q0 = d["Q0"].copy()
+    q0[:, :6] = q0[:, 9] = 0.0
+    ref, got = _predict(L, d, 0, q0), _predict(L, d, 0, np.ldexp(q0, -1010))
+    for p in (0, 1, 2, 3, 4, 5, 9):
+        assert rel_l2(np.ldexp(got[:, p], 1010), ref[:, p]) <= 1e-14, p
+
+
+@pytest.mark.parametrize("N", [1, 3, 6])
 @pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 1e-10), (2, 1e-10)])
 def test_rows_of_unlike_size(L, N, precision, tol):
     """Quantities many orders of magnitude apart (stresses in Pa beside velocities in m/s), zero rows among them: every
