@@ -261,50 +261,57 @@ __global__ void __launch_bounds__(FaceShape<N>::NT, FaceShape<N>::MIN_BLOCKS)
 
 // Q += E I - sum_j Khat^j A^j I in binary64: the volume line for a predictor
 // that did not write Q~(1) itself (poro_correct after a separate predictor, the
-// unrefined form): off the step's path, so kept plain
-constexpr int VNT = 128;
+// unrefined form).  A thread takes a mode's star product in one direction, then one
+// row and mode of the sum.  What bounds it: the binary64 pipe, so the division by dt
+// comes once, at the end.  poro_correct, this kernel and the faces, milliseconds in
+// binary64 (double-binary32): 48,000 elements at N = 2 1.71 (1.22), N = 3 3.93 (3.02);
+// 16,464 at N = 5 5.10 (4.06), 10,368 at N = 6 5.44 (4.39).  One thread a mode for all
+// three directions, with divisions there: 4.83 (4.34), 6.83 (5.91), 6.02 (4.98), 6.23 (5.16).
+constexpr int volume_threads(int N) { return NQ * n_modes(N) < 256 ? (NQ * n_modes(N) + 31) / 32 * 32 : 256; }
 template <bool BATCH>
-__global__ void __launch_bounds__(VNT) volume_kernel(int N, const CorrectorData D1, const int32_t* elems,
+__global__ void __launch_bounds__(256) volume_kernel(int N, const CorrectorData D1, const int32_t* elems,
                                                      const CorrectorData* runs, const int32_t* item_run) {
     extern __shared__ double smv[];
     chain_wait();
     chain_go();
-    const int B = n_modes(N), QB = NQ * B;
-    double* I = smv;      // [13][B]
-    double* X = I + QB;   // [13][B]
+    const int B = n_modes(N), QB = NQ * B, NT = blockDim.x;
+    double* I = smv;           // [13][B]
+    double* X = I + QB;        // [3][13][B]: dt A^j I
+    double* star = X + 3 * QB;
     const int tid = threadIdx.x;
     const CorrectorData& D = BATCH ? runs[item_run[blockIdx.x]] : D1;
     const int64_t e = elems ? elems[blockIdx.x] : (int64_t)blockIdx.x;
     const double* ec = D.econst + e * elem_const_stride(N);
     const double* sc = ec + ec_scalars(N);
-    const double ev = sc[0] / sc[2], gv = sc[1] / sc[2];
+    for (int i = tid; i < QB; i += NT) I[i] = D.iout[e * QB + i];
+    for (int i = tid; i < 3 * STAR_NNZ; i += NT) star[i] = ec[i];
+    __syncthreads();
+    for (int i = tid; i < 3 * B; i += NT) {
+        const int j = i / B, l = i - j * B;
+        const double* sj = star + j * STAR_NNZ;
+        double acc[NQ];
+#pragma unroll
+        for (int p = 0; p < NQ; ++p) acc[p] = 0.0;
+#pragma unroll
+        for (int n = 0; n < STAR_NNZ; ++n) acc[star_row(n)] = fma(sj[n], I[star_col(n) * B + l], acc[star_row(n)]);
+#pragma unroll
+        for (int p = 0; p < NQ; ++p) X[j * QB + p * B + l] = acc[p];
+    }
+    __syncthreads();
+    const double ev = sc[0], gv = sc[1], dt = sc[2];
     double* q = D.q + e * QB;
-    for (int i = tid; i < QB; i += VNT) I[i] = D.iout[e * QB + i];
-    for (int j = 0; j < 3; ++j) {
-        __syncthreads();
-        const double* sj = ec + j * STAR_NNZ;
-        for (int l = tid; l < B; l += VNT) {
-            double acc[NQ];
-#pragma unroll
-            for (int p = 0; p < NQ; ++p) acc[p] = 0.0;
-#pragma unroll
-            for (int n = 0; n < STAR_NNZ; ++n) acc[star_row(n)] = fma(sj[n], I[star_col(n) * B + l], acc[star_row(n)]);
-#pragma unroll
-            for (int p = 0; p < NQ; ++p) X[p * B + l] = acc[p] / sc[2];
+    for (int i = tid; i < QB; i += NT) {
+        const int p = i / B, k = i - p * B;
+        double acc = 0.0;
+        for (int j = 0; j < 3; ++j) {
+            const int32_t* kr = D.krow + j * (B + 1) + k;
+            const double* x = X + j * QB + p * B;
+            for (int n = kr[0]; n < kr[1]; ++n) acc = fma(D.kval[n], x[D.kcol[n]], acc);
         }
-        __syncthreads();
-        const int32_t* kr = D.krow + j * (B + 1);
-        for (int i = tid; i < QB; i += VNT) {
-            const int p = i / B, k = i - p * B;
-            double acc = 0.0;
-            for (int n = kr[k]; n < kr[k + 1]; ++n) acc = fma(D.kval[n], X[p * B + D.kcol[n]], acc);
-            if (j == 0) {
-                // Darcy source term E I: u rows from u_f, u_f rows from u_f
-                if (p >= QU && p <= QW) acc = fma(-gv, I[(p + QUF - QU) * B + k], acc);
-                if (p >= QUF) acc = fma(-ev, I[i], acc);
-            }
-            q[i] -= acc;
-        }
+        // Darcy source term E I: u rows from u_f, u_f rows from u_f
+        if (p >= QU && p <= QW) acc = fma(-gv, I[(p + QUF - QU) * B + k], acc);
+        if (p >= QUF) acc = fma(-ev, I[i], acc);
+        q[i] -= acc / dt;
     }
 }
 
@@ -420,9 +427,10 @@ int launch_corrector(const CorrectorData& d, bool volume, const int32_t* elems, 
                      const CorrectorData* runs, const int32_t* item_run) {
     if (count <= 0) return 0;
     if (volume) {
-        const size_t smem = sizeof(double) * 2 * NQ * n_modes(d.N);
+        const size_t smem = sizeof(double) * (4 * NQ * n_modes(d.N) + 3 * STAR_NNZ);  // 36 KB at N = 6
         auto* kern = runs ? volume_kernel<true> : volume_kernel<false>;
-        if (const cudaError_t err = launch_chained(kern, (unsigned)count, VNT, smem, stream, d.N, d, elems, runs, item_run))
+        if (const cudaError_t err = launch_chained(kern, (unsigned)count, volume_threads(d.N), smem, stream, d.N, d, elems,
+                                                   runs, item_run))
             return (int)err;
     }
     switch (d.N) {
