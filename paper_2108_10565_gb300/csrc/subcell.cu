@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(NT_) stp_subcell_kernel(const SubParams P) {
     double* sc = zuf + T * T;
     double* var = sm + S::OFF_VAR;
     double* smax = sm + S::OFF_MAX;
-    double* red = sm + S::OFF_RED;
+    unsigned long long* red = reinterpret_cast<unsigned long long*>(sm + S::OFF_RED);
     using Sweep = typename S::S;
     int* ints = reinterpret_cast<int*>(sm + S::OFF_I);
     const SweepScratch<Sweep> X{reinterpret_cast<int2*>(sm + S::OFF_X), ints, smax, ints + S::I_ROW};
@@ -205,35 +205,35 @@ __global__ void __launch_bounds__(NT_) stp_subcell_kernel(const SubParams P) {
                     mass_term<NT, Sweep, S::CHUNK>(V, term, p0, np, P.m3_row + r * (B + 1), P.m3_col, P.m3_val);
                 }
             alg3_sweep<N, NT, BiotSystem, Sweep>(V, star, zuf, sc[1], P.khat, X);  // Q_{k+1}
-            // max |Q_{k+1} - Q_k| and max |Q_{k+1}| over the element (fmax drops a NaN,
-            // so non-finite differences are noted apart)
-            double dmax = 0.0, vmax = 0.0;
-            bool bad = false;
+            // max |Q_{k+1} - Q_k| and max |Q_{k+1}| over the element, as bit patterns:
+            // the integer maximum of magnitudes is theirs, with NaN above infinity
+            // (fmax would drop a NaN, and its comparisons run on the binary64 pipe)
+            using Bits = unsigned long long;
+            Bits dmax = 0, vmax = 0;
             for (int i = tid; i < NQ * BT; i += NT) {
                 const int p = i / BT, m = i - p * BT;
-                const double v = V[p * QS + m], dv = fabs(v - U[p * QS + m]);
-                bad |= !isfinite(dv);
-                dmax = fmax(dmax, dv);
-                vmax = fmax(vmax, fabs(v));
+                const double v = V[p * QS + m];
+                dmax = max(dmax, (Bits)__double_as_longlong(fabs(v - U[p * QS + m])));
+                vmax = max(vmax, (Bits)__double_as_longlong(fabs(v)));
             }
 #pragma unroll
             for (int s = 16; s > 0; s >>= 1) {
-                dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, s));
-                vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, s));
+                dmax = max(dmax, __shfl_xor_sync(0xffffffffu, dmax, s));
+                vmax = max(vmax, __shfl_xor_sync(0xffffffffu, vmax, s));
             }
             if (lane == 0) {
                 red[warp] = dmax;
                 red[NW + warp] = vmax;
             }
-            const bool finite = !__syncthreads_or(bad);
-            dmax = 0.0;
-            vmax = 0.0;
+            __syncthreads();
+            dmax = vmax = 0;
             for (int w = 0; w < NW; ++w) {
-                dmax = fmax(dmax, red[w]);
-                vmax = fmax(vmax, red[NW + w]);
+                dmax = max(dmax, red[w]);
+                vmax = max(vmax, red[NW + w]);
             }
             // a non-finite iterate stops the loop unconverged (and is written out as it is)
-            converged = finite && dmax <= P.tol * vmax;
+            const bool finite = max(dmax, vmax) < 0x7FF0000000000000ull;
+            converged = finite && __longlong_as_double(dmax) <= P.tol * __longlong_as_double(vmax);
             stop = converged || !finite;
             double* t = U;
             U = V;
