@@ -283,30 +283,34 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
             };
             // the time integrals and Q~(1) of the task's rows, entry i in lane i of
             // the group, from lane 0's value of the row and of b + E* Q (the columns
-            // of Z^{-1} but the first sum to zero).  In double-binary32 `end` leaves
+            // of Z^{-1} but the first sum to zero).  In double-binary32 `ends` leaves
             // q0 out of b, and what remains, the step's change, is added to q0 in
             // binary64, so that a field carried from step to step keeps its bits.
             // q0 may be the array written: its entries read by this task are the
             // ones it writes.
-            auto finish = [&](auto row, const auto& v, const auto& end) {
+            auto finish = [&](auto row, const auto& v, auto ends) {
                 constexpr int M = sizeof(v) / sizeof(double);
+                if (io) {
 #pragma unroll
-                for (int i = 0; i < M; i += T) {
-                    const bool mine = act && i + u < M;
-                    if (io) {
+                    for (int i = 0; i < M; i += T) {
                         double w = __shfl_sync(0xffffffffu, v[i], base);
 #pragma unroll
                         for (int k = 1; k < T && i + k < M; ++k) {
                             const double wk = __shfl_sync(0xffffffffu, v[i + k], base);
                             w = u == k ? wk : w;
                         }
-                        if (mine) io[row(i + u) * B + m] = dt * w;
+                        if (act && i + u < M) io[row(i + u) * B + m] = dt * w;
                     }
-                    if (qe) {
+                }
+                if (qe) {
+                    R end[M];
+                    ends(end);
+#pragma unroll
+                    for (int i = 0; i < M; i += T) {
                         R w = P::shfl(end[i], base);
 #pragma unroll
                         for (int k = 1; k < T && i + k < M; ++k) w = P::select(u == k, P::shfl(end[i + k], base), w);
-                        if (mine) {
+                        if (act && i + u < M) {
                             const int at = row(i + u) * B + m;
                             const double x = P::value(P::normal(w));
                             qe[at] = P::DW ? q0[at] + x : x;
@@ -329,7 +333,10 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 b[3] = rhs(q[3 / T], 3 % T, a[3] = P::fma(iso[11], Df, P::mul(iso[10], D)));
                 const double v[4] = {put(SXX, plain(b[0])), put(SXX + 1, plain(b[1])), put(SXX + 2, plain(b[2])),
                                      put(QP, plain(b[3]))};
-                finish([](int r) { return r < 3 ? SXX + r : QP; }, v, P::DW ? a : b);
+                finish([](int r) { return r < 3 ? SXX + r : QP; }, v, [&](R* end) {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) end[r] = P::DW ? a[r] : b[r];
+                });
             } else {
                 // one pair (u, u_f) of velocities and one shear stress
                 const int i = kind - 1;
@@ -347,9 +354,11 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 xf = P::normal(xf);
                 const R by = P::fma(K[T * T + 1], xf, bu);  // + g Q_uf
                 const double v[3] = {put(QU + i, plain(by)), put(QUF + i, xf), put(SXY + i, plain(bs))};
-                const R end[3] = {P::DW ? P::fma(K[T * T + 1], xf, au) : by, P::fma(K[T * T], xf, P::DW ? af : bf),
-                                  P::DW ? as : bs};
-                finish([i](int r) { return (r == 0 ? QU : r == 1 ? QUF : SXY) + i; }, v, end);
+                finish([i](int r) { return (r == 0 ? QU : r == 1 ? QUF : SXY) + i; }, v, [&](R* end) {
+                    end[0] = P::DW ? P::fma(K[T * T + 1], xf, au) : by;
+                    end[1] = P::fma(K[T * T], xf, P::DW ? af : bf);
+                    end[2] = P::DW ? as : bs;
+                });
             }
         }
         __syncthreads();
