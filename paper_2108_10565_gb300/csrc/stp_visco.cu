@@ -13,8 +13,12 @@
 // primitive sums until the mode is solved, its stresses and velocities
 // afterwards; the anelastic functions go from registers to the output.
 //
-// A warp solves T lanes (u) of 32 / T modes: normal stresses with their 9 anelastic
-// functions, or one shear stress with its 3 and one velocity.  b = S^{-1}w q0 -
+// A warp solves T lanes (u) of 32 / T modes' normal stresses with their 9 anelastic
+// functions, or of 32 / T pairs of a mode and a shear stress with its 3 and one
+// velocity; at N <= 2, where blocks have few modes, a mode's normal stresses are three
+// groups of lanes (8,000 elements at N = 1: 142 microseconds undivided, 89 so; with
+// each shear stress a task of its own besides 196, and 357 instead of 284, now 215,
+// at N = 2).  b = S^{-1}w q0 -
 // combinations; th with (Z - e_l I)^{-1} (dense), then the couplings of E*'s strictly
 // upper part into the stresses, which like the velocities take the tridiagonal
 // Z^{-1}.
@@ -22,8 +26,8 @@
 // What bounds it: the binary64 pipe, 94 thousand operations an element at N = 5, over
 // half of them the dense solves of the anelastic functions; with star products and
 // Khat on all 27 rows they were 128 thousand, and the integer sums three times as
-// many.  4,001 elements at N = 5: 1.13 ms, the pipe 81 % busy (2.22 ms on 27 rows, 4.01
-// with the Khat products in binary64).
+// many.  4,001 elements at N = 5: 1.03 ms (1.13 with a task per shear stress, the pipe then
+// 81 % busy; 2.22 on 27 rows, 4.01 with the Khat products in binary64).
 #include <cuda_runtime.h>
 
 #include "fixed_device.cuh"
@@ -50,6 +54,10 @@ struct ViscoShape {
     static constexpr int NT = visco::threads(N), NW = NT / 32;
     static constexpr int B = n_modes(N), T = N + 1, PT = NP * T, PUL = (PT + 31) / 32, G = 32 / T;
     static constexpr int XC = visco::columns(N);
+    // normal stresses: a group of lanes per component where a warp holds three groups
+    // for several modes with few left over; modes a warp takes
+    static constexpr bool SPLIT = N <= 2;
+    static constexpr int GN = SPLIT ? G / 3 : G;
     // constants from the time matrices on: Zs[NMECH][T][T], scalars, iso[16]
     static constexpr int EC0 = 3 * visco::STAR_NNZ, EC = visco::elem_const_stride(N) - EC0;
     static constexpr int SC = NMECH * T * T, ISO = visco::ec_iso(N) - EC0;
@@ -104,10 +112,15 @@ __global__ void __launch_bounds__(ViscoShape<N>::NT, ViscoShape<N>::MIN_BLOCKS) 
         const int o = block_offset(g), d = block_size(g);
         // ---- time solves of block g
 #pragma unroll 1
-        for (int t = warp; t < 4 * ((d + G - 1) / G); t += NW) {
-            const int mb = t / 4 * G, kind = t % 4;
-            const bool act = grp < G && mb + grp < d;
-            const int m = o + min(mb + min(grp, G - 1), d - 1);
+        for (int t = warp, nn = (d + S::GN - 1) / S::GN; t < nn + (3 * d + G - 1) / G; t += NW) {
+            // GN modes' normal stresses (SPLIT: three groups of lanes a mode, one for
+            // component i), or G (shear component i, mode) pairs
+            const bool normal = t < nn;
+            const int per = normal && S::SPLIT ? 3 : 1, first = normal ? t * S::GN * per : (t - nn) * G;
+            const int count = normal ? min(d * per, first + S::GN * per) : 3 * d;
+            const bool act = grp < G && first + grp < count;
+            const int item = min(first + min(grp, G - 1), count - 1);
+            const int i = normal ? (S::SPLIT ? item % 3 : 0) : item / d, m = o + (normal ? item / per : item - i * d);
             double* c = C + m * PT + u;
             auto rhs = [&](int q, double a) { return fma(sw, q0[q * B + m], a); };  // S^{-1}w q0 + a
             auto plain = [&](double b) {
@@ -141,26 +154,38 @@ __global__ void __launch_bounds__(ViscoShape<N>::NT, ViscoShape<N>::MIN_BLOCKS) 
                 out(q, x);
                 return x;
             };
-            if (kind == 0) {
+            if (S::SPLIT && normal) {
+                const double g0 = c[0], g1 = c[T], g2 = c[2 * T], gi = i == 0 ? g0 : i == 1 ? g1 : g2;
+                double b = rhs(i, fma(-iso[10], gi, -iso[9] * ((g0 + g1) + g2)));
+                const int lane0 = lane - i * T;  // this u in component 0's group
+#pragma unroll 1
+                for (int l = 0; l < NMECH; ++l) {
+                    const double th = anelastic(l, i, gi);
+                    const double t0 = __shfl_sync(0xffffffffu, th, lane0), t1 = __shfl_sync(0xffffffffu, th, lane0 + T),
+                                 t2 = __shfl_sync(0xffffffffu, th, lane0 + 2 * T);
+                    // (Ylam + 2 Ymu) on the own component, Ylam on the other two
+                    const double off = sc[3 * l + 1], own = sc[3 * l] - off;
+                    b += fma(own, th, off * ((t0 + t1) + t2));
+                }
+                keep(i, plain(b));
+            } else if (normal) {
                 const double gd[3] = {c[0], c[T], c[2 * T]};
                 const double Lm = -iso[9] * ((gd[0] + gd[1]) + gd[2]);
                 double b[3];
 #pragma unroll
-                for (int i = 0; i < 3; ++i) b[i] = rhs(i, fma(-iso[10], gd[i], Lm));
+                for (int k = 0; k < 3; ++k) b[k] = rhs(k, fma(-iso[10], gd[k], Lm));
 #pragma unroll 1
                 for (int l = 0; l < NMECH; ++l) {
-                    // (Ylam + 2 Ymu) on the own component, Ylam on the other two
                     double th[3];
 #pragma unroll
                     for (int k = 0; k < 3; ++k) th[k] = anelastic(l, k, gd[k]);
                     const double off = sc[3 * l + 1], own = sc[3 * l] - off, s = off * ((th[0] + th[1]) + th[2]);
 #pragma unroll
-                    for (int i = 0; i < 3; ++i) b[i] += fma(own, th[i], s);
+                    for (int k = 0; k < 3; ++k) b[k] += fma(own, th[k], s);
                 }
 #pragma unroll
-                for (int i = 0; i < 3; ++i) keep(i, plain(b[i]));
+                for (int k = 0; k < 3; ++k) keep(k, plain(b[k]));
             } else {
-                const int i = kind - 1;
                 const double s = c[(3 + i) * T];
                 double b = rhs(3 + i, -iso[11] * s);
 #pragma unroll 1
