@@ -17,12 +17,14 @@ namespace poro {
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // the next kernel may be set up once every CTA of this one has come here
 __device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// The predictor and the faces let the next kernel in early up to degree 4, where
+// The predictor and the faces let the next kernel in early up to degree 3, where
 // elements are short: a cycle of 384 elements at N = 2 takes 41.3 instead of 43.4
-// microseconds, 12,288 elements in three clusters at N = 3 14.02 instead of
-// 14.10 ms.  At N = 6 (5,184 elements) the early CTAs crowd the SMs that run out
-// first: 6.02 ms a pass instead of 5.97.
-constexpr bool chain_early(int N) { return N <= 4; }
+// microseconds, 12,288 elements in three clusters at N = 3 14.02 instead of 14.10 ms
+// a pass.  Above, the early CTAs crowd the SMs that run out first.  Microseconds a step
+// of 384 and 6,000 elements, early and late: N = 4 binary64 95.1, 912 and 95.5, 911,
+// double-binary32 72.0, 508 and 69.0, 504; N = 5 158.2, 1,615 and 140.2, 1,613, 94.6,
+// 905 and 88.3, 899; N = 6, 5,184 elements, four steps in double-binary32, 6.02 and 5.97 ms.
+constexpr bool chain_early(int N) { return N <= 3; }
 
 template <class... Params, class... Args>
 cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, void* stream,
