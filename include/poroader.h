@@ -60,8 +60,12 @@ typedef struct {
 } poro_material;
 
 typedef enum {
-    PORO_FP64 = 0,          /* IEEE binary64; the Khat products as exact integer sums of
-                               62-bit fixed-point rows, rounded once */
+    PORO_FP64 = 0,          /* IEEE binary64; the Khat products as integer sums of rows in
+                               fixed point, summed exactly and rounded once.  A row (one
+                               quantity and time mode of a degree block) has one scale, 62
+                               bits below a bound on its entries: entries under 2^-9 of the
+                               bound keep fewer than binary64's 53 bits, so the error is
+                               binary64's relative to the block, not to its small entries */
     PORO_FP32_REFINE = 1,   /* double-binary32 (~48 bits) with integer Khat products: within
                                1e-10 of binary64 at the default refinement (about 1e-14);
                                time stepping adds each step's change to a binary64 field */
@@ -494,9 +498,10 @@ poro_status poro_autotune_tiles(poro_ctx* ctx, int64_t sample, int32_t* choice_o
 /* Select a tile choice explicitly.  Errors: PORO_EINVAL (not available). */
 poro_status poro_set_tiles(poro_ctx* ctx, int32_t choice);
 
-/* Floating-point operations one predictor of this context performs, counted
- * from the structural non-zeros the kernels touch (Khat blocks, the 54-entry
- * star pattern, the (N+1)^2 time solves): used for rooflines.  flops_out[0]
+/* Floating-point operations of one predictor of this context as Algorithm 3 is
+ * written, counted from the structural non-zeros (Khat blocks, the 54-entry
+ * star pattern, the (N+1)^2 time solves); the kernels factor the star products and
+ * sum the Khat products in integers, so they issue fewer.  flops_out[0]
  * = FP64 operations (PORO_FP64), flops_out[1] = low-precision operations
  * (refinement modes), flops_out[2] = residual operations (refinement modes,
  * per sweep). */

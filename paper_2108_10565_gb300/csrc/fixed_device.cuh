@@ -2,12 +2,13 @@
 // Khat^j is an integer row c over one denominator d_l (sum |c| < 2^23), so with
 // X in fixed point below a bound on its row, sum_j sum_m c_jlm X^j_m is formed
 // from integer sums.  Binary64 rows: 62 bits in two words, both summed exactly in
-// 64-bit integers, one rounding at the end (with the low word as binary32,
-// summed by FFMA, N = 6 took 110 thousand instead of 114 thousand clocks an element
-// and SM, but its error rose from 2.2e-16 to 2.9e-16).  Double-binary32 rows: a
-// 30-bit word summed in 64-bit integers and the remainder as binary32.  GB300
-// issues binary64 multiply-adds at 2 lanes a clock and SM, 64-bit integer ones at
-// 13 to 19, binary32 ones at 125.
+// 64-bit integers, one rounding at the end.  An entry under 2^-9 of its row's bound
+// thus has less than its own 53 bits: the error is relative to the row's largest
+// entries, not to each.  (With the low word as binary32, summed by FFMA, N = 6 took 110
+// thousand instead of 114 thousand clocks an element and SM, but its error rose from
+// 2.2e-16 to 2.9e-16.)  Double-binary32 rows: a 30-bit word summed in 64-bit integers
+// and the remainder as binary32.  GB300 issues binary64 multiply-adds at 2 lanes a
+// clock and SM, 64-bit integer ones at 13 to 19, binary32 ones at 125.
 #pragma once
 
 #include "dw_device.cuh"

@@ -392,13 +392,15 @@ void triangle_rule(int N, std::vector<double>& a, std::vector<double>& b, std::v
 }
 }  // namespace
 
-// Face trace operators.  With {psi_a} orthonormal on the reference triangle
-// under the quadrature weights (d_f = (N+1)(N+2)/2 functions, from the
-// Cholesky factor of the monomial Gram matrix), the trace of every basis
-// function on a face is a polynomial of degree <= N in the face parameters, so
-//   phi_k(chi_f(t)) = sum_a Pf[f][a][k] psi_a(t)   exactly, and
-//   Floc[f] = Pf[f]^T Pf[f],  Fnb[f,h,s] = Pf[f]^T Pnb[f,h,s]
-// with Pnb the neighbour's trace seen in this face's parameters.
+// Face trace operators.  {psi_a} is the triangle's Dubiner basis, normalised on the
+// reference triangle (d_f = (N+1)(N+2)/2 functions by degree; the polynomials are
+// orthogonal, so each is divided by its norm).  A face is parametrised over it with
+// its vertices in increasing local order, and the trace of every basis function is a
+// polynomial of degree <= N there, so
+//   phi_k(chi_f(t)) = sum_a Pf[f][a][k] psi_a(t)   exactly, and int_f phi_k phi_l = Pf[f]^T Pf[f].
+// A neighbour's trace, taken on its own face h, is seen from this side with the face's
+// vertices permuted: turn[s] maps its coefficients, int phi_k phi_l = Pf[f]^T turn[s] Pf[h],
+// and it mixes only functions of one degree.  Both are sparse in this basis.
 void face_traces(int N, std::vector<double>& Pf, std::vector<double>& turn) {
     const int B = n_modes(N), df = face_modes(N);
     std::vector<double> qa, qb, qw;

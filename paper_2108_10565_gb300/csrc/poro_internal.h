@@ -185,8 +185,10 @@ bool visco_element_constants(const ReferenceData& ref, const double* v12, const 
 // primitive rows, [3][26], then for the variation modes r = 1..3 of the
 // linearly interpolated Jacobians their 9 entries k0..k8 in x-direction
 // (subcell.cu, combine_row) and (e_r, g_r) of E*_r.
-// (N = 3, 500 elements: 1.60 ms on 256 threads, 1.79 on 128; N = 4, where two CTAs
-// fit an SM, 3.73 on 256, 4.69 on 512; N = 6, 100 elements: 5.97 on 512, 6.95 on 256)
+// (N = 1, 100 and 2,000 elements: 165 and 468 microseconds on 128 threads, 197 and 421 on
+// 64; N = 2 525 and 1,616, on 64 676 and 1,822; N = 3, 500 elements: 1.60 ms on 256, 1.79
+// on 128; N = 4, where two CTAs fit an SM, 3.73 on 256, 4.69 on 512; N = 5, 100 and 2,000:
+// 3.22 and 24.9 ms on 512, 3.48 and 27.0 on 256; N = 6, 100: 5.97 on 512, 6.95 on 256)
 constexpr int subcell_threads(int N) { return N >= 5 ? 512 : N >= 3 ? 256 : 128; }
 constexpr int subcell_columns(int N) { return N == 6 ? 30 : 3 * block_size(N); }
 constexpr int PRIM_NNZ = 26, SUBCELL_MODE = 11;
@@ -352,8 +354,9 @@ struct CorrectorData {
     const int32_t* nb = nullptr;      // [ne][4]
     const int32_t* tab = nullptr;     // [ne][4] neighbour table index f*24 + h*6 + s, or -1
     bool dw = false;                  // double-binary32 (mixed-precision contexts), else binary64
-    // [ne][4][2][13][4]: V, then c_f W (c_f = 2 |S_f| / |J|), of each face in
-    // 8-byte words (binary64, or (hi, lo) binary32)
+    // [ne][4][2][13][4]: V, then c_f W (c_f = 2 |S_f| / |J|), of each face in 8-byte
+    // words: binary64, or in double-binary32 two entries in 16 bytes, both high words
+    // and then both low ones (the layout of a packed pair)
     const void* fvw = nullptr;
     const int4* ftab = nullptr;       // face_tables
     const int32_t* krow = nullptr;    // full-row CSR of Khat^j [3][B+1] (absolute)
