@@ -162,7 +162,11 @@ struct DirectShape {
 };
 
 // ------------------------------------------------------------ kernel
-template <int N, int NT_, class P>
+// STEP: a time step's, which writes Q~(1).  With that part in one kernel for both, calls
+// without it took longer, microseconds in binary64 (double-binary32): 40,000 elements at
+// N = 2 758 (468) -> 741 (437), N = 3 1,543 (887) -> 1,513 (876), 20,000 at N = 6 5,821
+// (3,576) -> 5,753 (3,568).
+template <int N, int NT_, class P, bool STEP>
 __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<N>::MIN_BLOCKS : 1)
     stp_direct_kernel(const DirectParams A) {
     using S = DirectShape<N, NT_>;
@@ -249,7 +253,7 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
     const double dt = raw[T * T + 2];
     double* qo = run.qt ? run.qt + e * (int64_t)(B * PT) : nullptr;
     double* io = run.iout ? run.iout + e * (int64_t)(NQ * B) : nullptr;
-    double* qe = run.qend ? run.qend + e * (int64_t)(NQ * B) : nullptr;
+    double* qe = STEP && run.qend ? run.qend + e * (int64_t)(NQ * B) : nullptr;
     int buf = 0;
 #pragma unroll 1
     for (int g = N; g >= 0; --g) {
@@ -467,10 +471,10 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
 template <int N, int NT_, class P>
 int launch_nt(const DirectParams& A, void* stream) {
     using S = DirectShape<N, NT_>;
-    cudaError_t err = cudaFuncSetAttribute(stp_direct_kernel<N, NT_, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           S::SMEM_BYTES);
+    auto* kern = A.qend || A.runs ? stp_direct_kernel<N, NT_, P, true> : stp_direct_kernel<N, NT_, P, false>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BYTES);
     if (err != cudaSuccess) return (int)err;
-    return (int)launch_chained(stp_direct_kernel<N, NT_, P>, (unsigned)A.count, NT_, S::SMEM_BYTES, stream, A);
+    return (int)launch_chained(kern, (unsigned)A.count, NT_, S::SMEM_BYTES, stream, A);
 }
 
 // The default size is for launches that fill the chip several times over.  One
