@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
             const int m = o + min(mb + min(grp, G - 1), d - 1);
             R* c = C + m * PT + u;
             // lane u of a group loads entry u of the task's q0
-            auto load = [&](int q) { return P::of(q0[q * B + m]); };
+            auto load = [&](int q) { return q0[q * B + m]; };
             // b = S^{-1}w q0 + a, with entry i of the task's q0
             auto rhs = [&](R ql, int i, R a) { return P::fma1(sw, P::shfl(ql, base + i), a); };
             auto plain = [&](R b) {
@@ -290,9 +290,9 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
             // of Z^{-1} but the first sum to zero).  In double-binary32 `ends` leaves
             // q0 out of b, and what remains, the step's change, is added to q0 in
             // binary64, so that a field carried from step to step keeps its bits.
-            // q0 may be the array written: its entries read by this task are the
-            // ones it writes.
-            auto finish = [&](auto row, const auto& v, auto ends) {
+            // `old`: the lane's entry of q0.  q0 may be the array written: its entries
+            // read by this task are the ones it writes.
+            auto finish = [&](auto row, const auto& v, const double* old, auto ends) {
                 constexpr int M = sizeof(v) / sizeof(double);
                 if (io) {
 #pragma unroll
@@ -315,18 +315,18 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
 #pragma unroll
                         for (int k = 1; k < T && i + k < M; ++k) w = P::select(u == k, P::shfl(end[i + k], base), w);
                         if (act && i + u < M) {
-                            const int at = row(i + u) * B + m;
                             const double x = P::value(P::normal(w));
-                            qe[at] = P::DW ? q0[at] + x : x;
+                            qe[row(i + u) * B + m] = P::DW ? old[i / T] + x : x;
                         }
                     }
                 }
             };
             if (kind == 0) {
                 // normal stresses and pressure from D, Df, n_x u, n_y v
+                double old[(4 + T - 1) / T];
                 R q[(4 + T - 1) / T];
 #pragma unroll
-                for (int i = 0; i < 4; i += T) q[i / T] = load(i + u < 3 ? i + u : QP);
+                for (int i = 0; i < 4; i += T) q[i / T] = P::of(old[i / T] = load(i + u < 3 ? i + u : QP));
                 const R D = c[0], Df = c[T], gx = c[2 * T], gy = c[9 * T];
                 const R gz = P::sub(P::sub(D, gx), gy);
                 const R Lm = P::neg(P::fma(iso[10], Df, P::mul(iso[9], D)));
@@ -337,15 +337,15 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 b[3] = rhs(q[3 / T], 3 % T, a[3] = P::fma(iso[11], Df, P::mul(iso[10], D)));
                 const double v[4] = {put(SXX, plain(b[0])), put(SXX + 1, plain(b[1])), put(SXX + 2, plain(b[2])),
                                      put(QP, plain(b[3]))};
-                finish([](int r) { return r < 3 ? SXX + r : QP; }, v, [&](R* end) {
+                finish([](int r) { return r < 3 ? SXX + r : QP; }, v, old, [&](R* end) {
 #pragma unroll
                     for (int r = 0; r < 4; ++r) end[r] = P::DW ? a[r] : b[r];
                 });
             } else {
                 // one pair (u, u_f) of velocities and one shear stress
                 const int i = kind - 1;
-                const R q = load(u == 0 ? QU + i : u == 1 ? QUF + i : SXY + i);
-                const R qs = T > 2 ? q : load(SXY + i);
+                const double old[2] = {load(u == 0 ? QU + i : u == 1 ? QUF + i : SXY + i), T > 2 ? 0.0 : load(SXY + i)};
+                const R q = P::of(old[0]), qs = T > 2 ? q : P::of(old[1]);
                 const R as = P::neg(c[(SXY + i) * T]);
                 const R bs = rhs(qs, T > 2 ? 2 : 0, as);
                 const R Sg = c[(QU + i) * T], Gp = c[(QUF + i) * T];
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(NT_, NT_ == DirectSizes<N>::NT0 ? DirectSizes<
                 xf = P::normal(xf);
                 const R by = P::fma(K[T * T + 1], xf, bu);  // + g Q_uf
                 const double v[3] = {put(QU + i, plain(by)), put(QUF + i, xf), put(SXY + i, plain(bs))};
-                finish([i](int r) { return (r == 0 ? QU : r == 1 ? QUF : SXY) + i; }, v, [&](R* end) {
+                finish([i](int r) { return (r == 0 ? QU : r == 1 ? QUF : SXY) + i; }, v, old, [&](R* end) {
                     end[0] = P::DW ? P::fma(K[T * T + 1], xf, au) : by;
                     end[1] = P::fma(K[T * T], xf, P::DW ? af : bf);
                     end[2] = P::DW ? as : bs;
