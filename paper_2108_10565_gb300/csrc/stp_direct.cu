@@ -32,9 +32,9 @@
 // blocks leave few independent operations, so what binds beside the binary64 pipe
 // (72 % busy at N = 6) is latency: the work of each phase is cut fine and the CTA
 // at N = 6 has 16 warps.  Against star products entry by entry, dense Z^{-1} and
-// Khat in binary64, 20,000 elements at N = 6 take 5.86 instead of 22.45 ms; in
+// Khat in binary64, 20,000 elements at N = 6 take 5.73 instead of 22.45 ms; in
 // double-binary32, against a binary32 tensor-core sweep, an exact residual and a
-// correction sweep, 40,009 take 7.05 instead of 16.56 (N = 4, 20,011: 0.91 instead
+// correction sweep, 40,009 take 7.09 instead of 16.56 (N = 4, 20,011: 0.91 instead
 // of 3.67).
 #include <cuda_runtime.h>
 

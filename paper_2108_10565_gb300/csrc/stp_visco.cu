@@ -26,8 +26,8 @@
 // What bounds it: the binary64 pipe, 94 thousand operations an element at N = 5, over
 // half of them the dense solves of the anelastic functions; with star products and
 // Khat on all 27 rows they were 128 thousand, and the integer sums three times as
-// many.  4,001 elements at N = 5: 1.03 ms (1.13 with a task per shear stress, the pipe then
-// 81 % busy; 2.22 on 27 rows, 4.01 with the Khat products in binary64).
+// many.  4,001 elements at N = 5: 1.03 ms, the pipe 83 % busy (1.13 with a task per shear
+// stress, 81 %; 2.22 on 27 rows, 4.01 with the Khat products in binary64).
 #include <cuda_runtime.h>
 
 #include "fixed_device.cuh"

@@ -23,9 +23,9 @@
 // and every mode's term is W combined with 9 of its Jacobians' entries.  That is 2
 // passes of Khat products (integer sums) an iteration, one over W and one in the
 // sweep, instead of 4, and 26 instead of 162 multiply-adds a mode, time mode and
-// direction for the variations.  N = 4, 500 elements: 3.90 -> 2.69 ms a pass, the
-// binary64 pipe 66 % busy.  What bounds it beside that: latency, of the sweep's small blocks and of the barriers between them (2
-// elements an SM at N = 4, 1 from N = 5 on).
+// direction for the variations.  N = 4, 500 elements: 3.90 -> 2.61 ms a pass, the
+// binary64 pipe 65 % busy.  What bounds it beside that: latency, of the sweep's small
+// blocks and of the barriers between them (2 elements an SM at N = 4, 1 from N = 5 on).
 //
 // Shared memory: U (iterate), V (right-hand side, then the next iterate) and W
 // in the b / Q layout of the sweep, its fixed-point X (whose place takes a mode's

@@ -1,6 +1,6 @@
 """Parity at the clustered-LTS configuration's size: the layered graded mesh of
-2,044,416 tetrahedra at N = 5, one global step of the mixed form (bf16 sweeps,
-one refinement sweep, double-word corrector) through the C ABI.
+2,044,416 tetrahedra at N = 5, one global step of the mixed form (one
+refinement sweep: double-binary32 predictor and corrector) through the C ABI.
 
 The oracle cannot step two million elements, so six sampled elements are
 checked one by one: each sampled element and its face neighbours carry random

@@ -214,8 +214,8 @@ def test_graphs_autotune_and_variants_agree(L):
 @pytest.mark.parametrize("N", [5])
 def test_mixed_time_stepping_matches_fp64_at_scale(L, N):
     """48,000 elements (periodic 20^3 Kuhn mesh), random DOFs, two global
-    steps: the mixed-precision form (tensor-core predictor with refinement,
-    double-binary32 corrector) matches the binary64 form to 1e-10 relative per
+    steps: the mixed-precision form (double-binary32 predictor and corrector)
+    matches the binary64 form to 1e-10 relative per
     element.  (Each form is pinned to the oracle on small meshes above; this
     checks the full-size launch configuration.)"""
     mesh = inputs.kuhn_box_mesh(20)

@@ -116,7 +116,7 @@ def test_flux_matrices_match_oracle(L):
 @pytest.mark.parametrize("N", [3, 6])
 def test_library_khat_rows_match_oracle_fractions(L, N):
     """The library's own quadrature gives the same rational rows (numerators
-    over a common denominator) that its mixed residual packs."""
+    over a common denominator) as the oracle's."""
     from tests.test_oracle_pins import khat_row_fractions
 
     _, k = L.poro_reference_matrices(N)

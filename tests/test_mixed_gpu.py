@@ -1,9 +1,9 @@
-"""GPU parity of the mixed-precision predictor (binary32 Algorithm 3 +
-refinement against a double-binary32 residual) against the FP64 oracle.
+"""GPU parity of the mixed-precision predictor (by its refinement sweeps: 1
+double-binary32, 2 binary64, 0 one binary32 sweep) against the FP64 oracle.
 
-Accuracy goal: relative L2 per element <= 1e-10 after refinement (one sweep
-and two sweeps); without refinement the binary32 solve alone is ~1e-6 (shown,
-so the tolerance tests the refinement and not the binary32 solve).
+Accuracy goal: relative L2 per element <= 1e-10 with one sweep and with two;
+the unrefined binary32 solve is ~1e-6 (shown, so the tolerance tells the forms
+apart).
 """
 import numpy as np
 import pytest
@@ -53,8 +53,7 @@ def test_mixed_refined_matches_oracle(L, N, n, n_dense, sweeps):
 
 
 def test_unrefined_is_binary32_level(L):
-    """Refinement is what brings the error down: the binary32 sweep alone is
-    far from 1e-10 (and not garbage)."""
+    """The unrefined binary32 sweep is far from 1e-10 (and not garbage)."""
     d = population(9, 5, seed=11)
     qt, _ = _run(L, d, 0)
     errs = [rel_l2(qt[i], oracle_predictor(d, i)) for i in range(9)]
@@ -133,8 +132,8 @@ def test_cta_size_variants_agree(L, N, sweeps):
 
 @pytest.mark.parametrize("N,n", [(3, 17), (4, 9), (5, 7), (6, 5)])
 def test_bf16x3_refined_matches_oracle(L, N, n):
-    """The bf16 split-product form reaches the 1e-10 goal with one refinement
-    sweep (its default) and with two."""
+    """A bf16 context reaches the 1e-10 goal with one refinement sweep (its
+    default: double-binary32) and with two (binary64)."""
     d = population(n, N, seed=31 + N)
     res = {}
     for sweeps in (1, 2):
@@ -153,8 +152,7 @@ def test_bf16x3_refined_matches_oracle(L, N, n):
 
 
 def test_bf16x3_unrefined_is_low_precision(L):
-    """Without refinement the bf16 form is far from 1e-10 (so the tolerance
-    above tests the refinement)."""
+    """Without refinement the bf16 form is far from 1e-10."""
     N, n = 4, 9
     d = population(n, N, seed=77)
     ctx = L.poro_create(0, N, L.PORO_BF16X3_REFINE)
@@ -173,8 +171,8 @@ def test_bf16x3_unrefined_is_low_precision(L):
 @pytest.mark.parametrize("precision,sweeps", [(0, None), (1, 0), (1, 1), (1, 2), (2, 1)])
 def test_non_finite_input_stays_in_its_element(L, precision, sweeps):
     """A NaN in one element's Q0 gives that element a non-finite predictor
-    (every entry NaN once refinement rounds it onto the fixed-point grid) and
-    leaves every other element bitwise as in a clean run."""
+    (every entry NaN with one or two refinement sweeps) and leaves every other
+    element bitwise as in a clean run."""
     N, n, bad = 3, 40, 7
     d = population(n, N, seed=99)
     out = []
@@ -205,9 +203,9 @@ def test_non_finite_input_stays_in_its_element(L, precision, sweeps):
 @pytest.mark.parametrize("precision", [1, 2])
 def test_mixed_is_scale_invariant(L, scale, precision):
     """The predictor is linear in Q0: Q0 scaled by 1e-20 or 1e20 gives the
-    oracle's predictor scaled alike, within 1e-10, so the fixed-point grid of
-    the refinement (a power of two per quantity from its largest entry)
-    follows the data's magnitude."""
+    oracle's predictor scaled alike, within 1e-10, so the fixed-point
+    scales (a power of two per row of a degree block from a bound on its
+    entries) follow the data's magnitude."""
     N, n = 4, 7
     d = population(n, N, seed=404)
     ctx = L.poro_create(0, N, precision)

@@ -238,10 +238,8 @@ def test_khat_rows_are_small_rationals(N):
     and polynomial integrals of a basis with rational recurrence
     coefficients, so each row is an integer row over a small common
     denominator (a wrong normalisation factor, e.g. a stray sqrt(2), breaks
-    this).  The mixed-precision residual stores Khat in exactly this form:
-    numerators below 2^23 (packable with a 7-bit column), and each row's sum
-    of |numerators| below 2^22, so that its products with 22-bit fixed-point
-    values sum exactly below 2^44 in 64-bit integers."""
+    this).  The predictors' integer sums rely on rows of this kind: numerators
+    below 2^23 and each row's sum of |numerators| below 2^22."""
     worst_den, worst_num, worst_sum = 1, 0, 0
     for K in basis.khat_matrices(N):
         rows = khat_row_fractions(K)
